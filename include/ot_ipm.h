@@ -308,8 +308,9 @@ const char *ot_last_error(void);
  *   u (m), v (n): float64 duals                                      (device)
  *   sup_i, sup_j (psi): support pairs sorted by (i, j), distinct     (device, may be NULL if psi==0)
  *   out_i, out_j, out_d (kmax): selected pairs in (d, jlin) order    (device, caller-owned)
- *   out_count: number selected (device int32)
- * Scratch is allocated from the stream-ordered pool and released before return.
+ *   out_count: number selected (int32 in device memory, or in pinned host memory)
+ * Scratch is allocated from the stream-ordered pool and released before return; the stream is
+ * synchronised once before the call returns, so the outputs are complete then.
  * Errors: OT_ERR_ARG (sizes, m*n > 2^32, null pointers), OT_ERR_OOM, OT_ERR_CUDA.
  * ------------------------------------------------------------------------------------- */
 int ot_price_topk(int32_t m, int32_t n, const int32_t *sx, const int32_t *sy,
@@ -360,8 +361,8 @@ int ot_price_topk_ex(int32_t m, int32_t n, const int32_t *sx, const int32_t *sy,
  * or OT_ERR_BUF_TOO_SMALL with a message (ot_last_error) and changes no output.  Every call on a
  * device uses the same array and leaves its contents behind (each call clears what it needs), so
  * calls that overlap on the GPU -- on two streams, or from two threads -- race and must be
- * serialised by the caller.  The call synchronises its stream twice (to size the candidate set)
- * before it returns.  No cudaMalloc, cudaFree or allocating library routine is called. */
+ * serialised by the caller.  The call synchronises its stream before it returns.  No cudaMalloc,
+ * cudaFree or allocating library routine is called. */
 int ot_price_topk_noalloc(int32_t m, int32_t n, const int32_t *sx, const int32_t *sy,
                           const int32_t *tx, const int32_t *ty, const double *u, const double *v,
                           const int32_t *sup_i, const int32_t *sup_j, int64_t psi, int32_t kmax,
@@ -385,7 +386,7 @@ int64_t ot_kernel_launches(void);
  * per support pair in the row and the column pass, the per-row and per-column vectors, the
  * step's update of x and r, and -- with the FP32 dense factor, whose CG runs as one persistent
  * launch that includes the factor's application -- the triangle of L^-1 read twice):
- *   0 pricing scan (histogram pass)   1 pricing scan (gather pass)   2 FP64 recheck
+ *   0 pricing scan (histogram pass)   1 pricing scan (gather pass)   2 FP64 recheck and tile sort
  *   3 PCG FP64 (persistent kernel)    4 PCG FP32                     5 LDL^T numeric (FP64)
  *   6 LDL^T solve (FP64)              7 FP32 dense LDL^T + L^-1      8 FP32 dense apply
  *   9 FP64 refinement CG operator (S_M p and the step)

@@ -7,6 +7,7 @@ CUDA tensors; the solver handle takes host arrays and owns its device state.
 from __future__ import annotations
 
 import ctypes
+import threading
 from dataclasses import dataclass
 
 import numpy as np
@@ -226,6 +227,19 @@ class Solver:
         self.close()
 
 
+_local = threading.local()
+
+
+def _count_buffer():
+    """One pinned int32 of the calling thread: the library writes the count there and synchronises
+    before it returns, so no device-to-host copy follows (a synchronisation after the call's scratch
+    is released would also hand that memory back to the driver, 0.2 ms to map again)."""
+    import torch
+    if not hasattr(_local, "count"):
+        _local.count = torch.empty(1, dtype=torch.int32, pin_memory=True)
+    return _local.count
+
+
 def price_topk(sx, sy, tx, ty, u, v, sup_i, sup_j, kmax: int, precision: int = 1, stream=None,
                cost: str = "sqeuclid", scan_rows: int = 0, jset_cmax: float = 0.0, C=None):
     """Pricing + selection on device tensors (torch, cuda, contiguous): int32 coordinates,
@@ -243,7 +257,7 @@ def price_topk(sx, sy, tx, ty, u, v, sup_i, sup_j, kmax: int, precision: int = 1
     out_i = torch.empty(max(kmax, 1), dtype=torch.int32, device=dev)
     out_j = torch.empty(max(kmax, 1), dtype=torch.int32, device=dev)
     out_d = torch.empty(max(kmax, 1), dtype=torch.float64, device=dev)
-    cnt = torch.zeros(1, dtype=torch.int32, device=dev)
+    cnt = _count_buffer()
     checks = [(u, torch.float64), (v, torch.float64), (sup_i, torch.int32), (sup_j, torch.int32)]
     if C is None:
         checks += [(sx, torch.int32), (sy, torch.int32), (tx, torch.int32), (ty, torch.int32)]
@@ -270,7 +284,7 @@ def price_topk(sx, sy, tx, ty, u, v, sup_i, sup_j, kmax: int, precision: int = 1
                                    sup_i.data_ptr() if psi else None, sup_j.data_ptr() if psi else None, psi, kmax,
                                    precision, out_i.data_ptr(), out_j.data_ptr(), out_d.data_ptr(), cnt.data_ptr(),
                                    ctypes.byref(po), ctypes.c_void_p(s)))
-    k = int(cnt.item())
+    k = int(cnt[0])
     return out_i[:k], out_j[:k], out_d[:k]
 
 

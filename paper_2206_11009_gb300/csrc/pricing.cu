@@ -5,22 +5,31 @@
 // support (Section 3.2).  Optionally the scan covers only the listed pairs of the heuristic set
 // J = {(i, j) : c_ij < C_max} of Section 3.4.
 //
-// Pipeline (one host synchronisation):
-//   prep     squared cost: rows -> float4 (A_i, X_i, Y_i), cols -> float4 (B_j, x_j, y_j) with
-//            A_i = |x_i|^2 - u_i, X_i = -2 x_i (coordinates shifted to a common origin);
-//            other distances: rows -> (u_i, x_i, y_i), cols -> (v_j, x_j, y_j) in FP32;
-//            plus the magnitudes that bound the FP32 rounding error;
-//   bound    E >= |d_fp32 - d| for every pair (a priori rounding analysis, 1 thread);
-//   pass 1   register-blocked scan (or a pass over the J list), histogram of d < E over 4096
-//            magnitude bins + [0, E], minimum per tile;
-//   support  the support pairs' own contributions are subtracted from the histogram;
-//   thresh   T = edge of the bin holding the kmax-th smallest key; gather threshold
-//            Tg = min(T + 2E, E): every pair of the exact selection has d_fp32 <= Tg;
+// Pipeline (one host synchronisation, at its end):
+//   bounds   bounding box of the points (skipped when the caller knows it);
+//   cells,   the points in Morton order of up to 64 x 64 cells (counting sort), in their FP32 forms:
+//   prep     squared cost: rows (A_i, X_i, Y_i), cols (B_j, x_j, y_j) with A_i = |x_i|^2 - u_i,
+//            X_i = -2 x_i (coordinates shifted to a common origin); other distances: rows
+//            (u_i, x_i, y_i), cols (v_j, x_j, y_j); plus the magnitudes that bound the FP32 rounding
+//            error, and from them (last block) E >= |d_fp32 - d| for every pair (a priori analysis);
+//   tiles    boxes and largest duals of groups of rows and of 256 columns; the pairs of groups
+//            whose least possible reduced cost is at most 2E form the tile list (the others hold
+//            no pair with d_fp32 <= E);
+//   pass 1   one warp per tile: histogram of d < E over 4096 magnitude bins + [0, E], minimum of
+//            the tile; further blocks of the same launch take the histogram of the support's pairs;
+//   thresh   T = edge of the bin holding the kmax-th smallest key outside the support; gather
+//            threshold Tg = min(T + 2E, E): every pair of the exact selection has d_fp32 <= Tg;
 //   pass 2   rescan only tiles whose minimum is <= Tg, append (i, j) with d_fp32 <= Tg;
-//   recheck  FP64 d = (c - u) - v (no fusion), support membership by binary search in the
-//            CSR rows; sort by (d, jlin) with a stable LSD radix sort; keep the first kmax.
-// In the FP64 variant the scan computes d exactly, keys are float(d) (monotone), E = 0.  An
-// explicit cost matrix always takes the FP64 variant.
+//   select   FP64 d = (c - u) - v (no fusion), support membership by binary search in the CSR
+//            rows, sort by (d, jlin), keep the first kmax.
+// The candidate buffer has a fixed capacity (spec_capacity), so nothing waits for the host to learn
+// how many pairs pass 2 gathers: tiles of kSelT candidates are rechecked and sorted in shared memory,
+// one CTA each, and every candidate's final position is its place in its own tile plus the number
+// of smaller candidates in the other tiles (binary searches).  When the host finds at the end that
+// more pairs were gathered, pass 2 and the selection are redone with an exact-size buffer and a
+// stable LSD radix sort.  With a J list the passes go over the list instead of the tiles.
+// In the FP64 variant the scan covers all pairs in tiles of TI rows x kPT * RJ columns, computes d
+// exactly, keys are float(d) (monotone), E = 0.  An explicit cost matrix always takes it.
 #include "pricing.cuh"
 #include "primitives.cuh"
 
@@ -33,25 +42,38 @@ namespace {
 
 constexpr int kBins = 4097;       // bins 0..4095: d < 0 by magnitude (large first); 4096: [0, E]
 constexpr int kPT = 256;          // threads per scan CTA
-constexpr int kRJ = 8;            // columns held in registers per thread
-constexpr int kTJ = kPT * kRJ;    // columns per tile
+// Columns held in registers per thread, kPT * RJ of them per tile: 8, or 2 where n <= kNarrowN (a
+// 2048-column tile would be mostly padding: the FP64 scan of 256 x 256 pairs took 25 us with 8).
+constexpr int kRJ = 8, kRJNarrow = 2;
+constexpr int kNarrowN = 1024;
 // above this many pairs inside the FP32 gather window the selection is redone with the FP64 scan
 constexpr unsigned long long kMaxWindowPairs = 1ull << 27;
 
 struct Geo {
+    unsigned box[4];                             // order-preserving keys of max x, max y, max ~x, max ~y
+    unsigned done, done2;                        // blocks of cells_kernel / prep_kernel that are through
     unsigned long long umax_bits, vmax_bits;     // max |u|, max |v| (nonneg double bit patterns)
     int xs_max, ys_max, xt_max, yt_max;          // max |shifted coordinate|
     unsigned long long x2s_max, x2t_max;         // max |x|^2 (integers)
     float E;                                     // FP32 error window
     float Tg;                                    // gather threshold (inclusive)
     unsigned long long gather_bound;             // upper bound of pairs with key <= Tg
+    unsigned int ntile;                          // tiles of the FP32 passes
     unsigned int ncand;                          // gathered pairs
     unsigned int nvalid;                         // rechecked candidates
 };
 
-__device__ __forceinline__ int bin_of_neg(float d) {  // d <= 0
-    unsigned b = __float_as_uint(-d) >> 19;             // exponent + 4 mantissa bits
-    return 4095 - (int)b;                               // larger magnitude -> smaller bin
+// Magnitude bins of d <= 0: 64 octaves from 2^-30 up, 64 bins each (larger and smaller magnitudes in
+// the first and last bin).  The kmax-th key's bin is gathered whole: with 16 bins an octave it held
+// more pairs than kmax itself at 256x256.
+constexpr int kBinBase = (127 - 30) << 6;
+__device__ __forceinline__ int bin_of_neg(float d) {
+    const int b = (int)(__float_as_uint(-d) >> 17) - kBinBase;   // exponent and 6 mantissa bits
+    return 4095 - min(max(b, 0), 4095);                          // larger magnitude -> smaller bin
+}
+__device__ __forceinline__ float bin_edge(int bin) {             // the least magnitude in the bin
+    const int b = 4095 - bin;
+    return b > 0 ? __uint_as_float((unsigned)(b + kBinBase) << 17) : 0.f;
 }
 
 // ------------------------------------------------------------------------ cost evaluation
@@ -61,12 +83,18 @@ __device__ __forceinline__ int bin_of_neg(float d) {  // d <= 0
 enum : int { K_SQ = OT_COST_SQEUCLID, K_EU = OT_COST_EUCLID, K_L1 = OT_COST_L1, K_LI = OT_COST_LINF,
              K_DN = OT_COST_DENSE };
 
+// v >= 0 as a double: 2^52 + v is exact in the bit pattern, so one FP64 addition converts it (the
+// FP64 pipe is the bound of the FP64 scan and a conversion instruction takes it for longer).
+__device__ __forceinline__ double uint_to_f64(int v) {
+    return __dsub_rn(__hiloint2double(0x43300000, v), 4503599627370496.0);
+}
+
 template <int K>
 __device__ __forceinline__ double cost64(int dx, int dy) {
-    if (K == K_SQ) return (double)(dx * dx + dy * dy);
-    if (K == K_EU) return __dsqrt_rn((double)(dx * dx + dy * dy));
-    if (K == K_L1) return (double)(abs(dx) + abs(dy));
-    return (double)max(abs(dx), abs(dy));
+    if (K == K_SQ) return uint_to_f64(dx * dx + dy * dy);
+    if (K == K_EU) return __dsqrt_rn(uint_to_f64(dx * dx + dy * dy));
+    if (K == K_L1) return uint_to_f64(abs(dx) + abs(dy));
+    return uint_to_f64(max(abs(dx), abs(dy)));
 }
 
 __device__ __forceinline__ double cost64_rt(int kind, int dx, int dy) {
@@ -104,48 +132,69 @@ __device__ __forceinline__ float key32(const float4 &R, float cB, float cx, floa
     return __fsub_rn(__fsub_rn(c, R.x), cB);
 }
 
+// Order-preserving signed key of a double's high word (the low word only refines it).
+__device__ __forceinline__ int hi_key(double d) {
+    const int h = __double2hiint(d);
+    return h ^ ((h >> 31) & 0x7fffffff);
+}
+// A float at or below every double whose hi_key is k.
+__device__ __forceinline__ float hi_key_floor(int k) {
+    const int h = k ^ ((k >> 31) & 0x7fffffff);
+    return __double2float_rd(__hiloint2double(h, h < 0 ? -1 : 0));
+}
+
 // --------------------------------------------------------------------------------- prep
-template <bool SQ>
-__global__ void prep_kernel(int m, int n, const int32_t *__restrict__ sx, const int32_t *__restrict__ sy,
-                            const int32_t *__restrict__ tx, const int32_t *__restrict__ ty,
-                            const double *__restrict__ u, const double *__restrict__ v, int ox, int oy,
-                            float4 *__restrict__ rows, float4 *__restrict__ cols, Geo *geo) {
-    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    double umax = 0, vmax = 0;
-    int xsm = 0, ysm = 0, xtm = 0, ytm = 0;
-    long long x2s = 0, x2t = 0;
-    for (int64_t i = tid; i < m; i += stride) {
-        int x = sx[i] - ox, y = sy[i] - oy;
-        long long x2 = (long long)x * x + (long long)y * y;
-        float uf = __double2float_rn(u[i]);
-        if (rows) {
-            if (SQ) rows[i] = make_float4(__fsub_rn(__ll2float_rn(x2), uf), -2.0f * (float)x, -2.0f * (float)y, 0.f);
-            else rows[i] = make_float4(uf, (float)x, (float)y, 0.f);
-        }
-        umax = fmax(umax, fabs(u[i]));
-        xsm = max(xsm, abs(x)); ysm = max(ysm, abs(y)); x2s = max(x2s, x2);
+// Block-wide maxima: a warp tree, then one value per warp through shared memory; thread 0 gets it.
+template <typename T>
+__device__ __forceinline__ T block_max(T x, T *sh) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x = max(x, __shfl_down_sync(0xffffffffu, x, o));
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = x;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) x = max(x, sh[w]);
+    __syncthreads();
+    return x;
+}
+
+constexpr int kPrepPer = 4;   // points per thread of the passes below (one atomic per block and maximum)
+
+// Bounding box of all points: max over x, y and over ~x, ~y (~x = -x - 1 is decreasing and never
+// overflows) as unsigned keys, so that zero is below every value and idle threads add nothing.
+__global__ void __launch_bounds__(256)
+bounds_kernel(int m, int n, const int32_t *__restrict__ sx, const int32_t *__restrict__ sy,
+              const int32_t *__restrict__ tx, const int32_t *__restrict__ ty, Geo *geo) {
+    __shared__ unsigned sh[8];
+    unsigned k[4] = {0u, 0u, 0u, 0u};
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (int64_t)m + n;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int x = i < m ? sx[i] : tx[i - m], y = i < m ? sy[i] : ty[i - m];
+        k[0] = max(k[0], (unsigned)x ^ 0x80000000u);
+        k[1] = max(k[1], (unsigned)y ^ 0x80000000u);
+        k[2] = max(k[2], (unsigned)~x ^ 0x80000000u);
+        k[3] = max(k[3], (unsigned)~y ^ 0x80000000u);
     }
-    for (int64_t j = tid; j < n; j += stride) {
-        int x = tx[j] - ox, y = ty[j] - oy;
-        long long x2 = (long long)x * x + (long long)y * y;
-        float vf = __double2float_rn(v[j]);
-        if (cols) {
-            if (SQ) cols[j] = make_float4(__fsub_rn(__ll2float_rn(x2), vf), (float)x, (float)y, 0.f);
-            else cols[j] = make_float4(vf, (float)x, (float)y, 0.f);
-        }
-        vmax = fmax(vmax, fabs(v[j]));
-        xtm = max(xtm, abs(x)); ytm = max(ytm, abs(y)); x2t = max(x2t, x2);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const unsigned v = block_max(k[q], sh);
+        if (threadIdx.x == 0) atomicMax(&geo->box[q], v);
     }
-    // NaN duals poison the bound: force it to +inf so the window covers everything
-    if (umax != umax) umax = INFINITY;
-    if (vmax != vmax) vmax = INFINITY;
-    atomicMax(&geo->umax_bits, (unsigned long long)__double_as_longlong(umax));
-    atomicMax(&geo->vmax_bits, (unsigned long long)__double_as_longlong(vmax));
-    atomicMax(&geo->xs_max, xsm); atomicMax(&geo->ys_max, ysm);
-    atomicMax(&geo->xt_max, xtm); atomicMax(&geo->yt_max, ytm);
-    atomicMax(&geo->x2s_max, (unsigned long long)x2s);
-    atomicMax(&geo->x2t_max, (unsigned long long)x2t);
+}
+
+// The same from a box that the caller knows.
+__global__ void box_kernel(int xlo, int ylo, int xhi, int yhi, Geo *geo) {
+    if (threadIdx.x == 0) {
+        geo->box[0] = (unsigned)xhi ^ 0x80000000u;
+        geo->box[1] = (unsigned)yhi ^ 0x80000000u;
+        geo->box[2] = (unsigned)~xlo ^ 0x80000000u;
+        geo->box[3] = (unsigned)~ylo ^ 0x80000000u;
+    }
+}
+
+// Midpoint of the bounding box along axis q (0: x, 1: y).
+__device__ __forceinline__ int box_origin(const Geo *geo, int q) {
+    const int hi = (int)(geo->box[q] ^ 0x80000000u), lo = ~(int)(geo->box[q + 2] ^ 0x80000000u);
+    return (int)(((long long)lo + (long long)hi) / 2);
 }
 
 // A priori bound of |d_fp32 - d|.  Every rounding contributes at most 2^-24 times the magnitude
@@ -157,21 +206,19 @@ __global__ void prep_kernel(int m, int n, const int32_t *__restrict__ sx, const 
 //  other distances, d~ = fl(fl(c~ - fl(u_i)) - fl(v_j)) with c~ exact for L1 and L-infinity and
 //  |c~ - c| <= 2.001 * 2^-24 * c for the Euclidean distance (one rounding of dy*dy, one of the
 //  FMA, one of the square root; the first two enter the root halved).
-__global__ void bound_kernel(Geo *geo, int fp64, int kind) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    if (fp64) { geo->E = 0.f; return; }
+__device__ float error_bound(const Geo &geo, int kind) {
     const double uu = 5.9604644775390625e-08;  // 2^-24
-    double umax = __longlong_as_double((long long)geo->umax_bits);
-    double vmax = __longlong_as_double((long long)geo->vmax_bits);
+    double umax = __longlong_as_double((long long)geo.umax_bits);
+    double vmax = __longlong_as_double((long long)geo.vmax_bits);
     double E;
     if (kind == K_SQ) {
-        double x2s = (double)geo->x2s_max, x2t = (double)geo->x2t_max;
-        double cross = 2.0 * ((double)geo->xs_max * geo->xt_max + (double)geo->ys_max * geo->yt_max);
+        double x2s = (double)geo.x2s_max, x2t = (double)geo.x2t_max;
+        double cross = 2.0 * ((double)geo.xs_max * geo.xt_max + (double)geo.ys_max * geo.yt_max);
         double A = (x2s + umax) * (1 + 2 * uu), B = (x2t + vmax) * (1 + 2 * uu);
         double T1 = (A + B) * (1 + uu), T2 = (T1 + cross) * (1 + uu), D = (T2 + cross) * (1 + uu);
         E = uu * (x2s + umax + A + x2t + vmax + B + T1 + T2 + D) * 1.0001 + 1e-30;
     } else {
-        const double xs = (double)geo->xs_max + geo->xt_max, ys = (double)geo->ys_max + geo->yt_max;
+        const double xs = (double)geo.xs_max + geo.xt_max, ys = (double)geo.ys_max + geo.yt_max;
         double cmax, epsc = 0.0;
         if (kind == K_L1) cmax = xs + ys;
         else if (kind == K_LI) cmax = fmax(xs, ys);
@@ -181,8 +228,213 @@ __global__ void bound_kernel(Geo *geo, int fp64, int kind) {
         const double Dd = T * (1 + uu) + Vp; // |fl(c~ - u~) - v~|
         E = (epsc + uu * (umax + vmax + T + Dd)) * 1.0001 + 1e-30;
     }
-    float Ef = __double2float_ru(E);
-    geo->E = isfinite(Ef) ? Ef : FLT_MAX;
+    const float Ef = __double2float_ru(E);
+    return isfinite(Ef) ? Ef : FLT_MAX;
+}
+
+// ---- spatial order.  Cells of 2^s x 2^s coordinate units, s the least with at most 64 x 64 cells over
+// the bounding box, numbered in Morton order: consecutive points form compact groups.
+constexpr int kCells = 4096;
+constexpr int kCG = 256;     // columns per group (32 lanes x 8)
+
+__device__ __forceinline__ int cell_shift(const Geo *geo) {
+    unsigned ext = 0;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int hi = (int)(geo->box[q] ^ 0x80000000u), lo = ~(int)(geo->box[q + 2] ^ 0x80000000u);
+        ext = max(ext, (unsigned)hi - (unsigned)lo);
+    }
+    return max(0, 26 - __clz(ext));   // ext >> s < 64
+}
+
+__device__ __forceinline__ int cell_of(const Geo *geo, int s, int x, int y) {
+    const int xlo = ~(int)(geo->box[2] ^ 0x80000000u), ylo = ~(int)(geo->box[3] ^ 0x80000000u);
+    auto spread = [](unsigned v) {   // six bits to the even positions
+        v = (v | (v << 4)) & 0x30fu;
+        v = (v | (v << 2)) & 0x333u;
+        return (v | (v << 1)) & 0x555u;
+    };
+    return (int)(spread(((unsigned)x - (unsigned)xlo) >> s) | (spread(((unsigned)y - (unsigned)ylo) >> s) << 1));
+}
+
+// Points per cell (sources, then targets), each point's place in its cell (any order), and by the
+// last block the cells' first positions.
+__global__ void __launch_bounds__(256)
+cells_kernel(int m, int n, const int32_t *__restrict__ sx, const int32_t *__restrict__ sy,
+             const int32_t *__restrict__ tx, const int32_t *__restrict__ ty, Geo *geo, unsigned *cells,
+             unsigned *__restrict__ place) {
+    __shared__ unsigned wsum[8];
+    __shared__ int s_last;
+    const int s = cell_shift(geo);
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < (int64_t)m + n;
+         k += (int64_t)gridDim.x * blockDim.x) {
+        const bool src = k < m;
+        const int64_t e = src ? k : k - m;
+        place[k] = atomicAdd(&cells[(src ? 0 : kCells) + cell_of(geo, s, (src ? sx : tx)[e], (src ? sy : ty)[e])], 1u);
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&geo->done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int side = 0; side < 2; ++side) {   // exclusive scan, 16 cells per thread
+        unsigned *c = cells + side * kCells + threadIdx.x * (kCells / 256);
+        unsigned v[kCells / 256], sum = 0;
+#pragma unroll
+        for (int q = 0; q < kCells / 256; ++q) { v[q] = __ldcg(c + q); }
+#pragma unroll
+        for (int q = 0; q < kCells / 256; ++q) { const unsigned t = v[q]; v[q] = sum; sum += t; }
+        unsigned x = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) wsum[wid] = x;
+        __syncthreads();
+        unsigned first = x - sum;
+        for (int w = 0; w < wid; ++w) first += wsum[w];
+#pragma unroll
+        for (int q = 0; q < kCells / 256; ++q) c[q] = first + v[q];
+        __syncthreads();
+    }
+}
+
+// FP32 forms of the points, in the caller's order (rows, cols) and, with place != NULL, in cell order
+// (srt: sources then targets, the point's index in .w; sdual: its dual rounded up), and the error
+// bound.  The maxima are reduced per block before the atomics: one atomic per thread on eight words
+// took 171 us at m = n = 65536, this takes 11.
+template <bool SQ>
+__global__ void __launch_bounds__(256)
+prep_kernel(int m, int n, int kind, const int32_t *__restrict__ sx, const int32_t *__restrict__ sy,
+            const int32_t *__restrict__ tx, const int32_t *__restrict__ ty, const double *__restrict__ u,
+            const double *__restrict__ v, float4 *__restrict__ rows, float4 *__restrict__ cols,
+            const unsigned *__restrict__ cells, const unsigned *__restrict__ place, float4 *__restrict__ srt,
+            float *__restrict__ sdual, Geo *geo) {
+    __shared__ unsigned long long shl[8];
+    __shared__ int shi[8];
+    const int ox = box_origin(geo, 0), oy = box_origin(geo, 1), s = cell_shift(geo);
+    unsigned long long umax = 0, vmax = 0, x2s = 0, x2t = 0;
+    int xsm = 0, ysm = 0, xtm = 0, ytm = 0;
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < (int64_t)m + n;
+         k += (int64_t)gridDim.x * blockDim.x) {
+        const bool src = k < m;
+        const int64_t e = src ? k : k - m;
+        const int x0 = (src ? sx : tx)[e], y0 = (src ? sy : ty)[e], x = x0 - ox, y = y0 - oy;
+        const long long x2 = (long long)x * x + (long long)y * y;
+        const double dual = (src ? u : v)[e];
+        const float df = __double2float_rn(dual), fac = SQ && src ? -2.0f : 1.0f;
+        // |dual|: its bit pattern orders like its value (a NaN never compares below E: left out)
+        const unsigned long long bits = dual == dual ? (unsigned long long)__double_as_longlong(fabs(dual)) : 0ull;
+        const float4 f = make_float4(SQ ? __fsub_rn(__ll2float_rn(x2), df) : df, fac * (float)x, fac * (float)y,
+                                     __int_as_float((int)e));
+        (src ? rows : cols)[e] = f;
+        if (place) {
+            const int64_t at = (src ? 0 : m) +
+                               (int64_t)cells[(src ? 0 : kCells) + cell_of(geo, s, x0, y0)] + place[k];
+            srt[at] = f;
+            sdual[at] = __double2float_ru(dual);
+        }
+        if (src) {
+            umax = max(umax, bits);
+            xsm = max(xsm, abs(x)); ysm = max(ysm, abs(y)); x2s = max(x2s, (unsigned long long)x2);
+        } else {
+            vmax = max(vmax, bits);
+            xtm = max(xtm, abs(x)); ytm = max(ytm, abs(y)); x2t = max(x2t, (unsigned long long)x2);
+        }
+    }
+    umax = block_max(umax, shl); vmax = block_max(vmax, shl);
+    x2s = block_max(x2s, shl); x2t = block_max(x2t, shl);
+    xsm = block_max(xsm, shi); ysm = block_max(ysm, shi);
+    xtm = block_max(xtm, shi); ytm = block_max(ytm, shi);
+    if (threadIdx.x == 0) {
+        atomicMax(&geo->umax_bits, umax);
+        atomicMax(&geo->vmax_bits, vmax);
+        atomicMax(&geo->x2s_max, x2s);
+        atomicMax(&geo->x2t_max, x2t);
+        atomicMax(&geo->xs_max, xsm); atomicMax(&geo->ys_max, ysm);
+        atomicMax(&geo->xt_max, xtm); atomicMax(&geo->yt_max, ytm);
+        __threadfence();
+        if (atomicAdd(&geo->done2, 1u) == gridDim.x - 1) {   // every block's maxima are in
+            __threadfence();
+            Geo g;
+            volatile Geo *vg = geo;
+            g.umax_bits = vg->umax_bits; g.vmax_bits = vg->vmax_bits;
+            g.xs_max = vg->xs_max; g.ys_max = vg->ys_max; g.xt_max = vg->xt_max; g.yt_max = vg->yt_max;
+            g.x2s_max = vg->x2s_max; g.x2t_max = vg->x2t_max;
+            geo->E = error_bound(g, kind);
+        }
+    }
+}
+
+// Box and largest dual of each group: G consecutive sources, or kCG targets, in cell order.  One warp
+// per group, sources' groups first.
+struct Group { float xlo, xhi, ylo, yhi, dual; };
+
+__global__ void __launch_bounds__(256)
+groups_kernel(int m, int n, int G, int nrg, int ncg, float row_fac, const float4 *__restrict__ srt,
+              const float *__restrict__ sdual, Group *__restrict__ grp) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t w = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); w < (int64_t)nrg + ncg; w += (int64_t)gridDim.x * 8) {
+        const bool src = w < nrg;
+        const int64_t lo = src ? w * G : m + (w - nrg) * kCG;
+        const int64_t hi = src ? min(lo + G, (int64_t)m) : min(lo + kCG, (int64_t)m + n);
+        Group g{INFINITY, -INFINITY, INFINITY, -INFINITY, -INFINITY};
+        for (int64_t k = lo + lane; k < hi; k += 32) {
+            const float4 f = srt[k];
+            const float fac = src ? row_fac : 1.0f;   // -1/2 undoes the squared form's -2 (exact)
+            const float x = fac * f.y, y = fac * f.z;
+            g.xlo = fminf(g.xlo, x); g.xhi = fmaxf(g.xhi, x);
+            g.ylo = fminf(g.ylo, y); g.yhi = fmaxf(g.yhi, y);
+            g.dual = fmaxf(g.dual, sdual[k]);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            g.xlo = fminf(g.xlo, __shfl_xor_sync(0xffffffffu, g.xlo, o));
+            g.xhi = fmaxf(g.xhi, __shfl_xor_sync(0xffffffffu, g.xhi, o));
+            g.ylo = fminf(g.ylo, __shfl_xor_sync(0xffffffffu, g.ylo, o));
+            g.yhi = fmaxf(g.yhi, __shfl_xor_sync(0xffffffffu, g.yhi, o));
+            g.dual = fmaxf(g.dual, __shfl_xor_sync(0xffffffffu, g.dual, o));
+        }
+        if (lane == 0) grp[w] = g;
+    }
+}
+
+// The tile list: pairs of groups (column group h, row group g -> h nrg + g) that can hold a pair with
+// d_fp32 <= E.  Every d there is at least the cost of the boxes' gap minus the largest duals (all
+// rounded down), d_fp32 >= d - E: groups with that bound above 2E are left out.  At 256x256, duals of
+// slope 6 per pixel, 4 % of the pairs remain.
+template <int K>
+__global__ void __launch_bounds__(256)
+tiles_kernel(int nrg, int64_t total, const Group *__restrict__ grp, Geo *geo, unsigned *__restrict__ list) {
+    const float lim = 2.0f * geo->E;
+    const int lane = threadIdx.x & 31;
+    for (int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; t0 < total;
+         t0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t t = t0 + lane;
+        bool keep = false;
+        if (t < total) {
+            const Group a = grp[t % nrg], b = grp[nrg + t / nrg];
+            const float gx = fmaxf(0.f, fmaxf(a.xlo - b.xhi, b.xlo - a.xhi));   // integers: exact
+            const float gy = fmaxf(0.f, fmaxf(a.ylo - b.yhi, b.ylo - a.yhi));
+            float c;
+            if (K == K_L1) c = __fadd_rd(gx, gy);
+            else if (K == K_LI) c = fmaxf(gx, gy);
+            else {
+                c = __fadd_rd(__fmul_rd(gx, gx), __fmul_rd(gy, gy));
+                if (K == K_EU) c = __fsqrt_rd(c);
+            }
+            keep = !(__fsub_rd(__fsub_rd(c, a.dual), b.dual) > lim);   // (kept where it is not a number)
+        }
+        const unsigned bal = __ballot_sync(0xffffffffu, keep);
+        if (!bal) continue;
+        unsigned at = 0;
+        if (lane == 0) at = atomicAdd(&geo->ntile, (unsigned)__popc(bal));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (keep) list[at + __popc(bal & ((1u << lane) - 1u))] = (unsigned)t;
+    }
 }
 
 // One key into the histogram (pass 1) or the candidate list (pass 2).
@@ -203,75 +455,109 @@ __device__ __forceinline__ void take_key(float d, bool neg64, float E, float Tg,
     }
 }
 
-// ---------------------------------------------------------------------------------- scan
-// Tiles of TI source rows x kTJ target columns; kRJ columns per thread in registers, rows from
-// shared memory.  The FP32 variants evaluate keys in groups of 4 rows x kRJ columns with one
-// minimum and one branch per group.
-template <int K, bool FP64, bool GATHER>
+// The support pairs entered the histogram too (the scan does not test membership): their own
+// histogram, with the same arithmetic as the scan so that every key lands in the same bin, by the
+// blocks `part` of `parts` of the histogram launch (shared-memory counts first: global atomics on
+// the few occupied bins took 91 us for 588k pairs).  With a J list only the support pairs inside J
+// were scanned: jlim > 0 (integer cost key < jlim) or, for an explicit matrix, jcmax > 0
+// (c_ij < jcmax) selects them.
+struct SupArgs {
+    const int32_t *si, *sj;
+    int64_t psi;
+    long long jlim;
+    double jcmax;
+    int first;                   // blocks from this one on take the support
+    unsigned long long *hist;
+};
+
+template <int K, bool FP64>
+__device__ __forceinline__ void support_hist(const SupArgs &S, int n, const float4 *__restrict__ rows,
+                                             const float4 *__restrict__ cols, const int32_t *__restrict__ sx,
+                                             const int32_t *__restrict__ sy, const int32_t *__restrict__ tx,
+                                             const int32_t *__restrict__ ty, const double *__restrict__ u,
+                                             const double *__restrict__ v, const double *__restrict__ C, float E,
+                                             unsigned *sh_hist) {
+    const int part = (int)blockIdx.x - S.first, parts = (int)gridDim.x - S.first;
+    for (int64_t e = (int64_t)part * kPT + threadIdx.x; e < S.psi; e += (int64_t)parts * kPT) {
+        const int i = S.si[e], j = S.sj[e];
+        if (K == K_DN) {
+            if (S.jcmax > 0.0 && !(C[(int64_t)i * n + j] < S.jcmax)) continue;
+        } else if (S.jlim > 0 && cost_key(K, sx[i] - tx[j], sy[i] - ty[j]) >= S.jlim) {
+            continue;
+        }
+        if (FP64) {
+            const double cc = K == K_DN ? C[(int64_t)i * n + j] : cost64<K>(sx[i] - tx[j], sy[i] - ty[j]);
+            const double d = __dsub_rn(__dsub_rn(cc, u[i]), v[j]);
+            if (d < 0.0) atomicAdd(&sh_hist[bin_of_neg(__double2float_rn(d))], 1u);
+        } else {
+            const float4 R = rows[i], Q = cols[j];
+            const float d = key32<K>(R, Q.x, Q.y, Q.z);
+            if (d < 0.f) atomicAdd(&sh_hist[bin_of_neg(d)], 1u);
+            else if (d <= E) atomicAdd(&sh_hist[4096], 1u);
+        }
+    }
+}
+
+// ------------------------------------------------------------------------------- FP32 scan
+// One warp per tile of the list: 8 columns per lane in registers, the tile's rows staged through the
+// warp's shared memory 64 at a time, keys in groups of 4 rows x 8 columns with one branch per group.
+// Bound by the issue of the FP32 pipes: one add, two FMAs and one minimum per pair (squared cost).
+// Packed f32x2 arithmetic on two columns was 1.6 times slower, three-input minima no faster
+// (256x256, all pairs: 565 us scalar, 925 packed, 579 with three-input minima).
+constexpr int kStage = 64;
+
+template <int K, bool GATHER>
 __global__ void __launch_bounds__(kPT)
-scan_kernel(int m, int n, int TI, int ncb, int64_t ntiles,
-            const float4 *__restrict__ rows, const float4 *__restrict__ cols,
-            const int32_t *__restrict__ sx, const int32_t *__restrict__ sy,
-            const int32_t *__restrict__ tx, const int32_t *__restrict__ ty,
-            const double *__restrict__ u, const double *__restrict__ v, const double *__restrict__ C,
-            const Geo *__restrict__ geo, float *__restrict__ tile_min,
-            unsigned long long *__restrict__ hist, int32_t *__restrict__ ci,
-            int32_t *__restrict__ cj, unsigned long long cap, unsigned int *__restrict__ ncand) {
-    __shared__ float4 srow[FP64 ? 1 : 256];
-    __shared__ int2 srowi[FP64 ? 256 : 1];
-    __shared__ double srowu[FP64 ? 256 : 1];
+tile_scan_kernel(int m, int n, int G, int nrg, SupArgs S, const float4 *__restrict__ rows,
+                 const float4 *__restrict__ cols, const float4 *__restrict__ srt, const int32_t *__restrict__ sx,
+                 const int32_t *__restrict__ sy, const int32_t *__restrict__ tx, const int32_t *__restrict__ ty,
+                 const double *__restrict__ u, const double *__restrict__ v, const Geo *__restrict__ geo,
+                 const unsigned *__restrict__ list, float *__restrict__ tile_min,
+                 unsigned long long *__restrict__ hist, int32_t *__restrict__ ci, int32_t *__restrict__ cj,
+                 unsigned long long cap, unsigned int *__restrict__ ncand) {
+    __shared__ float4 srow[kPT / 32][kStage];
     __shared__ unsigned sh_hist[GATHER ? 1 : kBins];
-    __shared__ float sred[kPT / 32];
     if (!GATHER) {
         for (int b = threadIdx.x; b < kBins; b += kPT) sh_hist[b] = 0;
+        __syncthreads();
     }
-    const float E = geo->E;
-    const float Tg = geo->Tg;
-    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const int rb = (int)(t / ncb), cb = (int)(t % ncb);
-        if (GATHER && tile_min[t] > Tg) continue;  // uniform over the block
-        const int i0 = rb * TI;
-        const int nrows = min(TI, m - i0);
-        __syncthreads();
-        if (threadIdx.x < nrows) {
-            const int i = i0 + threadIdx.x;
-            if (FP64) {
-                if (K != K_DN) srowi[threadIdx.x] = make_int2(sx[i], sy[i]);
-                srowu[threadIdx.x] = u[i];
-            } else {
-                srow[threadIdx.x] = rows[i];
-            }
-        }
-        // columns into registers
-        float cB[kRJ], cx[kRJ], cy[kRJ];
-        int ix[kRJ], iy[kRJ];
-        double dv[kRJ];
+    const float E = geo->E, Tg = geo->Tg, thr = GATHER ? Tg : E;
+    const bool support = !GATHER && (int)blockIdx.x >= S.first;
+    if constexpr (!GATHER) {
+        if (support) support_hist<K, false>(S, n, rows, cols, sx, sy, tx, ty, u, v, nullptr, E, sh_hist);
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned ntile = support ? 0u : geo->ntile;
+    for (unsigned t = (blockIdx.x * (kPT / 32) + warp); t < ntile; t += S.first * (kPT / 32)) {
+        if (GATHER && tile_min[t] > Tg) continue;   // uniform over the warp
+        const unsigned id = list[t];
+        const int64_t c0 = (int64_t)(id / nrg) * kCG + lane;
+        const int r0 = (int)(id % nrg) * G, nr = min(G, m - r0);
+        // padding columns get key +inf: cB = +inf in the squared form (d = ... + B_j), -inf in the
+        // direct form (d = ... - v_j)
+        float cB[8], cx[8], cy[8];
+        int jj[8];
 #pragma unroll
-        for (int c = 0; c < kRJ; ++c) {
-            const int j = cb * kTJ + c * kPT + threadIdx.x;
-            if (FP64) {
-                if (j < n) { if (K != K_DN) { ix[c] = tx[j]; iy[c] = ty[j]; } dv[c] = v[j]; }
-                else { ix[c] = 0; iy[c] = 0; dv[c] = -INFINITY; }  // d = +inf
-            } else {
-                // padding columns get key +inf: cB = +inf in the squared form (d = ... + B_j),
-                // -inf in the direct form (d = ... - v_j)
-                float4 q = j < n ? cols[j] : make_float4(K == K_SQ ? INFINITY : -INFINITY, 0.f, 0.f, 0.f);
-                cB[c] = q.x; cx[c] = q.y; cy[c] = q.z;
-            }
+        for (int c = 0; c < 8; ++c) {
+            const float4 q = c0 + 32 * c < n ? srt[m + c0 + 32 * c]
+                                             : make_float4(K == K_SQ ? INFINITY : -INFINITY, 0.f, 0.f, __int_as_float(n));
+            cB[c] = q.x; cx[c] = q.y; cy[c] = q.z; jj[c] = __float_as_int(q.w);
         }
-        __syncthreads();
         float tmin = INFINITY;
-        const float thr = GATHER ? Tg : E;
-        int r0 = 0;
-        if (!FP64) {
-            for (; r0 + 4 <= nrows; r0 += 4) {
-                float d[4][kRJ], mq[4];
+        for (int b0 = 0; b0 < nr; b0 += kStage) {
+            const int nb = min(kStage, nr - b0);
+            __syncwarp();
+            for (int k = lane; k < nb; k += 32) srow[warp][k] = srt[r0 + b0 + k];
+            __syncwarp();
+            for (int g0 = 0; g0 < nb; g0 += 4) {
+                float d[4][8], mq[4];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    const float4 R = srow[r0 + q];
+                    // (a ragged last group repeats its last row: the same keys, never taken twice)
+                    const float4 R = srow[warp][min(g0 + q, nb - 1)];
                     mq[q] = INFINITY;
 #pragma unroll
-                    for (int c = 0; c < kRJ; ++c) {
+                    for (int c = 0; c < 8; ++c) {
                         d[q][c] = key32<K>(R, cB[c], cx[c], cy[c]);
                         mq[q] = fminf(mq[q], d[q][c]);
                     }
@@ -281,54 +567,109 @@ scan_kernel(int m, int n, int TI, int ncb, int64_t ntiles,
                 if (dmin <= thr) {
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
-                        if (mq[q] > thr) continue;
+                        if (g0 + q >= nb || mq[q] > thr) continue;
+                        const int i = GATHER ? __float_as_int(srow[warp][g0 + q].w) : 0;
 #pragma unroll
-                        for (int c = 0; c < kRJ; ++c)
-                            take_key<false, GATHER>(d[q][c], false, E, Tg, sh_hist, i0 + r0 + q,
-                                                    cb * kTJ + c * kPT + threadIdx.x, n, ci, cj, cap, ncand);
+                        for (int c = 0; c < 8; ++c)
+                            take_key<false, GATHER>(d[q][c], false, E, Tg, sh_hist, i, jj[c], n, ci, cj, cap, ncand);
                     }
                 }
             }
         }
-        for (int r = r0; r < nrows; ++r) {
-            float d[kRJ];
-            double dd[kRJ];
-            float dmin = INFINITY;
-            if (FP64) {
-                const double ur = srowu[r];
+        if (!GATHER) {   // the tile's minimum (for skipping it in pass 2)
 #pragma unroll
-                for (int c = 0; c < kRJ; ++c) {
-                    double cc;
-                    if (K == K_DN) {
-                        const int j = cb * kTJ + c * kPT + threadIdx.x;
-                        cc = j < n ? C[(int64_t)(i0 + r) * n + j] : 0.0;
-                    } else {
-                        const int2 R = srowi[r];
-                        cc = cost64<K>(R.x - ix[c], R.y - iy[c]);
-                    }
-                    dd[c] = __dsub_rn(__dsub_rn(cc, ur), dv[c]);
-                    d[c] = __double2float_rn(dd[c]);
-                    dmin = fminf(dmin, d[c]);
-                }
-            } else {
-                const float4 R = srow[r];
+            for (int o = 16; o > 0; o >>= 1) tmin = fminf(tmin, __shfl_down_sync(0xffffffffu, tmin, o));
+            if (lane == 0) tile_min[t] = tmin;
+        }
+    }
+    if (!GATHER) {
+        __syncthreads();
+        unsigned long long *out = support ? S.hist : hist;
+        for (int b = threadIdx.x; b < kBins; b += kPT)
+            if (sh_hist[b]) atomicAdd(&out[b], (unsigned long long)sh_hist[b]);
+    }
+}
+
+// ------------------------------------------------------------------------------- FP64 scan
+// Tiles of TI source rows x kPT * RJ target columns; RJ columns per thread in registers, rows from
+// shared memory.  Bound by the FP64 pipe: only the three FP64 operations of the definition per pair,
+// the minima and the sign on the high words.
+template <int K, bool GATHER, int RJ>
+__global__ void __launch_bounds__(kPT)
+scan64_kernel(int m, int n, int TI, int ncb, int64_t ntiles, SupArgs S,
+              const int32_t *__restrict__ sx, const int32_t *__restrict__ sy,
+              const int32_t *__restrict__ tx, const int32_t *__restrict__ ty,
+              const double *__restrict__ u, const double *__restrict__ v, const double *__restrict__ C,
+              const Geo *__restrict__ geo, float *__restrict__ tile_min,
+              unsigned long long *__restrict__ hist, int32_t *__restrict__ ci,
+              int32_t *__restrict__ cj, unsigned long long cap, unsigned int *__restrict__ ncand) {
+    constexpr int TJ = kPT * RJ;
+    __shared__ int2 srowi[256];
+    __shared__ double srowu[256];
+    __shared__ unsigned sh_hist[GATHER ? 1 : kBins];
+    __shared__ float sred[kPT / 32];
+    if (!GATHER) {
+        for (int b = threadIdx.x; b < kBins; b += kPT) sh_hist[b] = 0;
+        __syncthreads();
+    }
+    const float Tg = geo->Tg;
+    const bool support = !GATHER && (int)blockIdx.x >= S.first;
+    if constexpr (!GATHER) {
+        if (support) support_hist<K, true>(S, n, nullptr, nullptr, sx, sy, tx, ty, u, v, C, 0.f, sh_hist);
+    }
+    for (int64_t t = support ? ntiles : blockIdx.x; t < ntiles; t += S.first) {
+        const int rb = (int)(t / ncb), cb = (int)(t % ncb);
+        if (GATHER && tile_min[t] > Tg) continue;  // uniform over the block
+        const int i0 = rb * TI;
+        const int nrows = min(TI, m - i0);
+        __syncthreads();
+        if (threadIdx.x < nrows) {
+            const int i = i0 + threadIdx.x;
+            if (K != K_DN) srowi[threadIdx.x] = make_int2(sx[i], sy[i]);
+            srowu[threadIdx.x] = u[i];
+        }
+        const int j0 = cb * TJ + (int)threadIdx.x;   // this thread's columns: j0 + c * kPT
+        int ix[RJ], iy[RJ];
+        double dv[RJ];
 #pragma unroll
-                for (int c = 0; c < kRJ; ++c) {
-                    d[c] = key32<K>(R, cB[c], cx[c], cy[c]);
-                    dmin = fminf(dmin, d[c]);
+        for (int c = 0; c < RJ; ++c) {
+            const int j = j0 + c * kPT;
+            ix[c] = 0; iy[c] = 0; dv[c] = -INFINITY;   // padding: d = +inf
+            if (j < n) { if (K != K_DN) { ix[c] = tx[j]; iy[c] = ty[j]; } dv[c] = v[j]; }
+        }
+        __syncthreads();
+        // Tg <= 0 here.  A pair is taken when float(d) <= Tg (d < 0 in the histogram pass): its high
+        // word's key is then at most one above Tg's (the rounding to float)
+        const int kthr = GATHER ? hi_key((double)Tg) + 1 : -1;
+        int kmin = INT_MAX;
+        for (int r = 0; r < nrows; ++r) {
+            double dd[RJ];
+            int kq = INT_MAX;
+            const double ur = srowu[r];
+            const int2 R = K != K_DN ? srowi[r] : make_int2(0, 0);
+#pragma unroll
+            for (int c = 0; c < RJ; ++c) {
+                double cc;
+                if (K == K_DN) {
+                    const int j = j0 + c * kPT;
+                    cc = j < n ? C[(int64_t)(i0 + r) * n + j] : 0.0;
+                } else {
+                    cc = cost64<K>(R.x - ix[c], R.y - iy[c]);
                 }
+                dd[c] = __dsub_rn(__dsub_rn(cc, ur), dv[c]);
+                kq = min(kq, hi_key(dd[c]));
             }
-            tmin = fminf(tmin, dmin);
-            if (dmin <= thr) {
+            kmin = min(kmin, kq);
+            if (kq <= kthr) {
 #pragma unroll
-                for (int c = 0; c < kRJ; ++c)
-                    take_key<FP64, GATHER>(d[c], FP64 ? (dd[c] < 0.0) : false, E, Tg, sh_hist, i0 + r,
-                                           cb * kTJ + c * kPT + threadIdx.x, n, ci, cj, cap, ncand);
+                for (int c = 0; c < RJ; ++c)
+                    take_key<true, GATHER>(__double2float_rn(dd[c]), dd[c] < 0.0, 0.f, Tg, sh_hist, i0 + r,
+                                           j0 + c * kPT, n, ci, cj, cap, ncand);
             }
         }
         if (!GATHER) {
             // tile minimum (for skipping tiles in pass 2)
-            float w = tmin;
+            float w = kmin != INT_MAX ? hi_key_floor(kmin) : INFINITY;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) w = fminf(w, __shfl_down_sync(0xffffffffu, w, o));
             if ((threadIdx.x & 31) == 0) sred[threadIdx.x >> 5] = w;
@@ -342,8 +683,9 @@ scan_kernel(int m, int n, int TI, int ncb, int64_t ntiles,
     }
     if (!GATHER) {
         __syncthreads();
+        unsigned long long *out = support ? S.hist : hist;
         for (int b = threadIdx.x; b < kBins; b += kPT)
-            if (sh_hist[b]) atomicAdd(&hist[b], (unsigned long long)sh_hist[b]);
+            if (sh_hist[b]) atomicAdd(&out[b], (unsigned long long)sh_hist[b]);
     }
 }
 
@@ -356,7 +698,8 @@ constexpr int kJT = kPT * kJE;
 
 template <int K, bool FP64, bool GATHER>
 __global__ void __launch_bounds__(kPT)
-jscan_kernel(int n, int64_t jn, int64_t ntiles, const int32_t *__restrict__ ji, const int32_t *__restrict__ jj,
+jscan_kernel(int n, int64_t jn, int64_t ntiles, SupArgs S, const int32_t *__restrict__ ji,
+             const int32_t *__restrict__ jj,
              const float4 *__restrict__ rows, const float4 *__restrict__ cols,
              const int32_t *__restrict__ sx, const int32_t *__restrict__ sy,
              const int32_t *__restrict__ tx, const int32_t *__restrict__ ty,
@@ -372,7 +715,11 @@ jscan_kernel(int n, int64_t jn, int64_t ntiles, const int32_t *__restrict__ ji, 
     }
     const float E = geo->E;
     const float Tg = geo->Tg;
-    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const bool support = !GATHER && (int)blockIdx.x >= S.first;
+    if constexpr (!GATHER) {
+        if (support) support_hist<K, FP64>(S, n, rows, cols, sx, sy, tx, ty, u, v, C, E, sh_hist);
+    }
+    for (int64_t t = support ? ntiles : blockIdx.x; t < ntiles; t += S.first) {
         if (GATHER && tile_min[t] > Tg) continue;  // uniform over the block
         float tmin = INFINITY;
 #pragma unroll 4
@@ -413,113 +760,221 @@ jscan_kernel(int n, int64_t jn, int64_t ntiles, const int32_t *__restrict__ ji, 
     }
     if (!GATHER) {
         __syncthreads();
+        unsigned long long *out = support ? S.hist : hist;
         for (int b = threadIdx.x; b < kBins; b += kPT)
-            if (sh_hist[b]) atomicAdd(&hist[b], (unsigned long long)sh_hist[b]);
+            if (sh_hist[b]) atomicAdd(&out[b], (unsigned long long)sh_hist[b]);
     }
 }
 
-// The support pairs entered the histogram too (the scan does not test membership); take their
-// keys out again.  Same arithmetic as the scan, so every key lands in the same bin.  With a J
-// list only the support pairs inside J were scanned: jlim > 0 (integer cost key < jlim) or, for
-// an explicit matrix, jcmax > 0 (c_ij < jcmax) selects them.
-template <int K, bool FP64>
-__global__ void support_hist_kernel(int n, int64_t psi, const int32_t *__restrict__ si, const int32_t *__restrict__ sj,
-                                    const float4 *__restrict__ rows, const float4 *__restrict__ cols,
-                                    const int32_t *__restrict__ sx, const int32_t *__restrict__ sy,
-                                    const int32_t *__restrict__ tx, const int32_t *__restrict__ ty,
-                                    const double *__restrict__ u, const double *__restrict__ v,
-                                    const double *__restrict__ C, long long jlim, double jcmax,
-                                    const Geo *__restrict__ geo, unsigned long long *__restrict__ hist) {
-    const float E = geo->E;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < psi;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int i = si[e], j = sj[e];
-        if (K == K_DN) {
-            if (jcmax > 0.0 && !(C[(int64_t)i * n + j] < jcmax)) continue;
-        } else if (jlim > 0 && cost_key(K, sx[i] - tx[j], sy[i] - ty[j]) >= jlim) {
-            continue;
-        }
-        int bin = -1;
-        if (FP64) {
-            const double cc = K == K_DN ? C[(int64_t)i * n + j] : cost64<K>(sx[i] - tx[j], sy[i] - ty[j]);
-            const double d = __dsub_rn(__dsub_rn(cc, u[i]), v[j]);
-            if (d < 0.0) bin = bin_of_neg(__double2float_rn(d));
-        } else {
-            const float4 R = rows[i], Q = cols[j];
-            const float d = key32<K>(R, Q.x, Q.y, Q.z);
-            if (d < 0.f) bin = bin_of_neg(d);
-            else if (d <= E) bin = 4096;
-        }
-        if (bin >= 0) atomicAdd(&hist[bin], ~0ull);  // -1
-    }
-}
-
-// One block: find the bin holding the kmax-th smallest key, the gather threshold Tg and an
-// upper bound on the number of pairs (support included) the gather pass will append.
+// One block: find the bin holding the kmax-th smallest key outside the support, the gather
+// threshold Tg and an upper bound on the number of pairs (support included) pass 2 will append.
+// Thread t holds bins 4 t .. 4 t + 3 (the last one also bin 4096).
 __global__ void __launch_bounds__(1024)
-threshold_kernel(const unsigned long long *__restrict__ hist_ns,   // support removed
-                 const unsigned long long *__restrict__ hist_all,  // support included
+threshold_kernel(const unsigned long long *__restrict__ hist_all, const unsigned long long *__restrict__ hist_sup,
                  int kmax, int fp64, Geo *geo) {
-    __shared__ unsigned long long part[1024];
+    __shared__ unsigned long long wsum[32];
     __shared__ int s_bstar;
-    const int t = threadIdx.x;
-    unsigned long long loc = 0;
-    for (int k = 0; k < 4; ++k) {
-        int b = 4 * t + k;
-        if (b < kBins) loc += hist_ns[b];
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    unsigned long long all[5], ns[5], loc = 0;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        const bool have = k < 4 || t == 1023;
+        all[k] = have ? hist_all[4 * t + k] : 0ull;
+        ns[k] = have ? all[k] - hist_sup[4 * t + k] : 0ull;
+        loc += ns[k];
     }
-    if (t == 1023) loc += hist_ns[4096];  // 4*1023+3 = 4095; bin 4096 joins the last group
-    part[t] = loc;
     if (t == 0) s_bstar = -1;
-    __syncthreads();
-    // inclusive scan (Hillis-Steele; 1024 entries)
-    for (int o = 1; o < 1024; o <<= 1) {
-        unsigned long long y = t >= o ? part[t - o] : 0ull;
-        __syncthreads();
-        part[t] += y;
-        __syncthreads();
+    unsigned long long x = loc;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
     }
-    unsigned long long before = t > 0 ? part[t - 1] : 0ull;
-    if (part[t] >= (unsigned long long)kmax && before < (unsigned long long)kmax) {
+    if (lane == 31) wsum[wid] = x;
+    __syncthreads();
+    unsigned long long before = x - loc;
+    for (int w = 0; w < wid; ++w) before += wsum[w];
+    if (before < (unsigned long long)kmax && before + loc >= (unsigned long long)kmax) {
         unsigned long long acc = before;
-        int lim = (t == 1023) ? 5 : 4;
-        for (int k = 0; k < lim; ++k) {
-            acc += hist_ns[4 * t + k];
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+            acc += ns[k];
             if (acc >= (unsigned long long)kmax) { s_bstar = 4 * t + k; break; }
         }
     }
-    __shared__ int s_bg;
+    __syncthreads();
+    const int bstar = s_bstar;
+    const float E = geo->E;
+    float Tg;
+    if (bstar < 0 || bstar == 4096) {
+        Tg = fp64 ? 0.0f : E;                 // take every candidate
+    } else {
+        const float T = -bin_edge(bstar);     // every key in bins <= bstar is <= T
+        if (fp64) Tg = T;
+        else Tg = fminf(__fadd_ru(T, __fmul_ru(2.0f, E)), E);
+    }
+    // bins that can hold keys <= Tg
+    const int bg = Tg < 0.f ? bin_of_neg(Tg) : (fp64 ? 4095 : 4096);
+    unsigned long long take = 0;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) take += 4 * t + k <= bg ? all[k] : 0ull;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) take += __shfl_down_sync(0xffffffffu, take, o);
+    if (lane == 0) wsum[wid] = take;
     __syncthreads();
     if (t == 0) {
-        const int bstar = s_bstar;
-        const float E = geo->E;
-        float Tg;
-        if (bstar < 0 || bstar == 4096) {
-            Tg = fp64 ? 0.0f : E;                 // take every candidate
-        } else {
-            const float lo = __uint_as_float((unsigned)(4095 - bstar) << 19);
-            const float T = -lo;                  // every key in bins <= bstar is <= T
-            if (fp64) Tg = T;
-            else Tg = fminf(__fadd_ru(T, __fmul_ru(2.0f, E)), E);
-        }
+        for (int w = 1; w < 32; ++w) take += wsum[w];
         geo->Tg = Tg;
-        // bins that can hold keys <= Tg
-        s_bg = Tg < 0.f ? bin_of_neg(Tg) : (fp64 ? 4095 : 4096);
+        geo->gather_bound = take;
     }
-    __syncthreads();
-    // the gather bound: the pairs (support included) in bins 0 .. bg, summed by the whole block
-    const int bg = s_bg;
-    unsigned long long loc2 = 0;
-    for (int b = t; b <= bg; b += 1024) loc2 += hist_all[b];
-    part[t] = loc2;
-    __syncthreads();
-    for (int o = 512; o > 0; o >>= 1) {
-        if (t < o) part[t] += part[t + o];
-        __syncthreads();
-    }
-    if (t == 0) geo->gather_bound = part[0];
 }
 
+// FP64 reduced cost of pair (i, j) and whether it is a candidate (d < 0 outside the support)
+__device__ __forceinline__ bool recheck_pair(int i, int j, int n, int kind, const int32_t *__restrict__ sx,
+                                             const int32_t *__restrict__ sy, const int32_t *__restrict__ tx,
+                                             const int32_t *__restrict__ ty, const double *__restrict__ u,
+                                             const double *__restrict__ v, const double *__restrict__ C,
+                                             const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ sup_j,
+                                             double &d) {
+    const int end = row_ptr[i + 1];
+    int lo = row_ptr[i], hi = end;
+    while (lo < hi) {  // lower_bound of j in the sorted columns of row i
+        const int mid = (lo + hi) >> 1;
+        if (sup_j[mid] < j) lo = mid + 1; else hi = mid;
+    }
+    const bool member = lo < end && sup_j[lo] == j;
+    const double cc = kind == K_DN ? C[(int64_t)i * n + j] : cost64_rt(kind, sx[i] - tx[j], sy[i] - ty[j]);
+    d = __dsub_rn(__dsub_rn(cc, u[i]), v[j]);
+    return !member && d < 0.0;
+}
+
+// ------------------------------------------------------------------------ selection
+// Candidates in tiles of kSelT: each CTA rechecks its tile in FP64 and sorts it by (d, jlin) with a
+// bitonic network -- two elements per thread, distances up to 32 in registers by shuffles, the
+// others through shared memory (10 of the 55 steps).  Pairs that are no candidates get the largest
+// key.  Latency-bound; it replaced two radix sorts (11 passes of three launches, 350 us at 12k).
+constexpr int kSelT = 1024;
+
+__device__ __forceinline__ bool key_less(unsigned long long ka, unsigned ja, unsigned long long kb, unsigned jb) {
+    return ka < kb || (ka == kb && ja < jb);
+}
+
+__global__ void __launch_bounds__(kSelT / 2)
+select_sort_kernel(int m, int n, int kind, unsigned cap, const int32_t *__restrict__ ci,
+                   const int32_t *__restrict__ cj, const int32_t *__restrict__ sx, const int32_t *__restrict__ sy,
+                   const int32_t *__restrict__ tx, const int32_t *__restrict__ ty, const double *__restrict__ u,
+                   const double *__restrict__ v, const double *__restrict__ C, const int32_t *__restrict__ row_ptr,
+                   const int32_t *__restrict__ sup_j, Geo *geo, unsigned long long *__restrict__ skey,
+                   unsigned *__restrict__ sjl) {
+    __shared__ unsigned long long sk[kSelT];
+    __shared__ unsigned sj[kSelT];
+    const unsigned count = geo->ncand, base = blockIdx.x * kSelT;
+    if (geo->gather_bound > cap || base >= count) return;   // uniform over the block
+    const int lane = threadIdx.x & 31, p0 = (threadIdx.x >> 5) * 64 + lane;   // positions p0 and p0 + 32
+    unsigned long long k[2];
+    unsigned l[2];
+    int nv = 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const unsigned e = base + p0 + 32 * h;
+        k[h] = ~0ull;
+        l[h] = ~0u;
+        bool ok = false;
+        if (e < count) {
+            const int i = ci[e], j = cj[e];
+            double d;
+            ok = recheck_pair(i, j, n, kind, sx, sy, tx, ty, u, v, C, row_ptr, sup_j, d);
+            if (ok) {
+                k[h] = f64_key(d);
+                l[h] = (unsigned)i + (unsigned)j * (unsigned)m;   // jlin < m n <= 2^32
+            }
+        }
+        nv += __syncthreads_count(ok);
+    }
+    if (threadIdx.x == 0 && nv) atomicAdd(&geo->nvalid, (unsigned)nv);
+    auto keep = [&](int h, unsigned long long ok, unsigned ol, int pos, int dist, int size) {
+        // position pos meets pos ^ dist: the lower position keeps the smaller when ascending
+        const bool lower = (pos & dist) == 0, asc = (pos & size) == 0;
+        const bool less = key_less(ok, ol, k[h], l[h]);
+        if (less == (lower == asc)) { k[h] = ok; l[h] = ol; }
+    };
+    for (int size = 2; size <= kSelT; size <<= 1) {
+        int dist = size >> 1;
+        for (; dist >= 64; dist >>= 1) {
+            __syncthreads();
+            sk[p0] = k[0]; sj[p0] = l[0];
+            sk[p0 + 32] = k[1]; sj[p0 + 32] = l[1];
+            __syncthreads();
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int pos = p0 + 32 * h;
+                keep(h, sk[pos ^ dist], sj[pos ^ dist], pos, dist, size);
+            }
+        }
+        if (dist == 32) {
+            const bool asc = (p0 & size) == 0;
+            if (key_less(k[1], l[1], k[0], l[0]) == asc) {
+                const unsigned long long tk = k[0]; k[0] = k[1]; k[1] = tk;
+                const unsigned tl = l[0]; l[0] = l[1]; l[1] = tl;
+            }
+            dist = 16;
+        }
+        for (; dist > 0; dist >>= 1)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const unsigned long long ok = __shfl_xor_sync(0xffffffffu, k[h], dist);
+                const unsigned ol = __shfl_xor_sync(0xffffffffu, l[h], dist);
+                keep(h, ok, ol, p0 + 32 * h, dist, size);
+            }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        skey[base + p0 + 32 * h] = k[h];
+        sjl[base + p0 + 32 * h] = l[h];
+    }
+}
+
+// Final position of every candidate: its place in its own tile plus, for every other tile, the
+// number of smaller keys there.  Four lanes per candidate share the tiles, each lane two binary
+// searches at a time (the chain of probes is the cost); neighbouring candidates search for
+// neighbouring keys, so their probes share cache lines.  The keys are distinct.
+__global__ void __launch_bounds__(256)
+select_rank_kernel(int m, int kmax, unsigned cap, const unsigned long long *__restrict__ skey,
+                   const unsigned *__restrict__ sjl, const Geo *__restrict__ geo, int32_t *__restrict__ out_i,
+                   int32_t *__restrict__ out_j, double *__restrict__ out_d, int32_t *__restrict__ out_count) {
+    if (geo->gather_bound > cap) return;   // redone by the host with an exact-size buffer
+    const unsigned e = blockIdx.x * 64 + (threadIdx.x >> 2), part = threadIdx.x & 3;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *out_count = (int)min((unsigned)kmax, geo->nvalid);
+    const int ntiles = (int)((geo->ncand + kSelT - 1) / kSelT), own = (int)(e / kSelT);
+    if (own >= ntiles) return;             // uniform over the block (64 candidates of one tile)
+    const unsigned long long k = skey[e];
+    const unsigned l = sjl[e];
+    unsigned rank = part == 0 ? e % kSelT : 0u;
+    auto probe = [&](unsigned at) { return key_less(skey[at], sjl[at], k, l); };
+    for (int t = (int)part; k != ~0ull && t < ntiles && rank < (unsigned)kmax; t += 8) {
+        const int t2 = t + 4;
+        const unsigned ba = (unsigned)t * kSelT, bb = (unsigned)min(t2, ntiles - 1) * kSelT;
+        unsigned a = 0, b = 0;
+#pragma unroll
+        for (int s = kSelT / 2; s > 0; s >>= 1) {
+            if (probe(ba + a + s - 1)) a += s;
+            if (probe(bb + b + s - 1)) b += s;
+        }
+        if (a == kSelT - 1 && probe(ba + a)) ++a;
+        if (b == kSelT - 1 && probe(bb + b)) ++b;
+        if (t != own) rank += a;
+        if (t2 < ntiles && t2 != own) rank += b;
+    }
+    rank += __shfl_xor_sync(0xffffffffu, rank, 1);
+    rank += __shfl_xor_sync(0xffffffffu, rank, 2);
+    if (part == 0 && k != ~0ull && rank < (unsigned)kmax) {
+        out_i[rank] = (int32_t)(l % (unsigned)m);
+        out_j[rank] = (int32_t)(l / (unsigned)m);
+        if (out_d) out_d[rank] = f64_from_key(k);
+    }
+}
+
+// The same for candidate sets beyond the fixed capacity: keys for a stable radix sort by (d, jlin)
 __global__ void recheck_kernel(int m, int n, int kind, unsigned long long count, const int32_t *__restrict__ ci,
                                const int32_t *__restrict__ cj, const int32_t *__restrict__ sx,
                                const int32_t *__restrict__ sy, const int32_t *__restrict__ tx,
@@ -536,16 +991,8 @@ __global__ void recheck_kernel(int m, int n, int kind, unsigned long long count,
         double d = 0.0;
         if (g < ncand) {
             const int i = ci[g], j = cj[g];
-            int lo = row_ptr[i], hi = row_ptr[i + 1];
-            while (lo < hi) {  // lower_bound of j in the sorted columns of row i
-                int mid = (lo + hi) >> 1;
-                if (sup_j[mid] < j) lo = mid + 1; else hi = mid;
-            }
-            const bool member = lo < row_ptr[i + 1] && sup_j[lo] == j;
-            const double cc = kind == K_DN ? C[(int64_t)i * n + j] : cost64_rt(kind, sx[i] - tx[j], sy[i] - ty[j]);
-            d = __dsub_rn(__dsub_rn(cc, u[i]), v[j]);
             kj = (uint64_t)i + (uint64_t)j * (uint64_t)m;
-            if (!member && d < 0.0) {
+            if (recheck_pair(i, j, n, kind, sx, sy, tx, ty, u, v, C, row_ptr, sup_j, d)) {
                 kd = f64_key(d);
                 atomicAdd(&geo->nvalid, 1u);
             }
@@ -579,28 +1026,27 @@ __global__ void finalize_kernel(int kmax, const uint32_t *__restrict__ val, cons
     if (blockIdx.x == 0 && threadIdx.x == 0) *out_count = cnt;
 }
 
+// rp[r] = first entry of row >= r: entry e fills the rows after its predecessor's up to its own (the
+// last one the rest).  A warp's lanes with longer gaps are served by the whole warp in turn.
 __global__ void row_ptr_kernel(const int32_t *__restrict__ sup_i, int64_t psi, int m, int32_t *__restrict__ rp) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i <= m; i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t lo = 0, hi = psi;
-        while (lo < hi) {
-            int64_t mid = (lo + hi) >> 1;
-            if (sup_i[mid] < i) lo = mid + 1; else hi = mid;
+    const int lane = threadIdx.x & 31;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t e0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; e0 <= psi; e0 += stride) {
+        const int64_t e = e0 + lane;
+        int lo = 0, hi = -1;   // rows lo .. hi get e
+        if (e <= psi) {
+            lo = e > 0 ? sup_i[e - 1] + 1 : 0;
+            hi = e < psi ? sup_i[e] : m;
         }
-        rp[i] = (int32_t)lo;
+        if (lo == hi) rp[lo] = (int32_t)e;
+        unsigned wide = __ballot_sync(0xffffffffu, lo < hi);
+        while (wide) {
+            const int q = __ffs(wide) - 1;
+            wide &= wide - 1;
+            const int a = __shfl_sync(0xffffffffu, lo, q), b = __shfl_sync(0xffffffffu, hi, q);
+            for (int r = a + lane; r <= b; r += 32) rp[r] = (int32_t)(e0 + q);
+        }
     }
-}
-
-__global__ void minmax_kernel(int m, int n, const int32_t *sx, const int32_t *sy, const int32_t *tx,
-                              const int32_t *ty, int *mm /* xmin, ymin, -xmax, -ymax */) {
-    int xmin = INT_MAX, ymin = INT_MAX, xmax = INT_MIN, ymax = INT_MIN;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (int64_t)m + n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        int x = i < m ? sx[i] : tx[i - m];
-        int y = i < m ? sy[i] : ty[i - m];
-        xmin = min(xmin, x); ymin = min(ymin, y); xmax = max(xmax, x); ymax = max(ymax, y);
-    }
-    atomicMin(&mm[0], xmin); atomicMin(&mm[1], ymin);
-    atomicMin(&mm[2], -xmax); atomicMin(&mm[3], -ymax);
 }
 
 // J list (Section 3.4): the pairs with c_ij < C_max, sorted by (i, j).  One block per (row,
@@ -667,28 +1113,10 @@ __global__ void jfill_kernel(int m, int n, int kind, const int32_t *__restrict__
 }  // namespace
 
 Error build_row_ptr(const int32_t *sup_i, int64_t psi, int32_t m, int32_t *row_ptr, cudaStream_t st) {
-    row_ptr_kernel<<<(unsigned)ceil_div((int64_t)m + 1, 256), 256, 0, st>>>(sup_i, psi, m, row_ptr);
+    row_ptr_kernel<<<(unsigned)std::min<int64_t>(ceil_div(psi + 1, 256), 4096), 256, 0, st>>>(sup_i, psi, m, row_ptr);
     OT_LAUNCHED();
     return ok();
 }
-
-Error coord_origin(int32_t m, int32_t n, const int32_t *sx, const int32_t *sy, const int32_t *tx,
-                   const int32_t *ty, int32_t *ox, int32_t *oy, cudaStream_t st) {
-    DevTemp<int> mm;
-    OT_TRY(mm.alloc(4, st));
-    int init[4] = {INT_MAX, INT_MAX, INT_MAX, INT_MAX};
-    OT_CUDA(cudaMemcpyAsync(mm.p, init, sizeof(init), cudaMemcpyHostToDevice, st));
-    minmax_kernel<<<(unsigned)std::min<int64_t>(1024, ceil_div((int64_t)m + n, 256)), 256, 0, st>>>(
-        m, n, sx, sy, tx, ty, mm.p);
-    OT_LAUNCHED();
-    int h[4];
-    OT_CUDA(cudaMemcpyAsync(h, mm.p, sizeof(h), cudaMemcpyDeviceToHost, st));
-    OT_CUDA(cudaStreamSynchronize(st));
-    *ox = (int32_t)(((int64_t)h[0] + (int64_t)(-h[2])) / 2);
-    *oy = (int32_t)(((int64_t)h[1] + (int64_t)(-h[3])) / 2);
-    return ok();
-}
-
 
 long long jset_limit(int kind, double cmax) {
     if (!(cmax > 0)) return 0;
@@ -747,64 +1175,88 @@ Error jset_build(int kind, int32_t m, int32_t n, const int32_t *sx, const int32_
 
 namespace {
 
-// One scan pass (full tiles or the J list) for cost kind K.
+// What the passes read: FP32 points in the caller's order and in cell order, the tile list.
+struct ScanData {
+    bool fp64 = false, narrow = false;
+    int TI = 0, ncb = 0;          // FP64 scan
+    int64_t ntiles = 0;           // FP64 tiles or J-list tiles
+    int G = 0, nrg = 0, ncg = 0;  // FP32 tiles: rows per group, row and column groups
+    float4 *rows = nullptr, *cols = nullptr, *srt = nullptr;
+    float *sdual = nullptr;
+    Group *grp = nullptr;
+    unsigned *list = nullptr, *cells = nullptr, *place = nullptr;
+    float *tmin = nullptr;
+    Geo *geo = nullptr;
+    unsigned long long *hist = nullptr;
+};
+
+// One scan pass for cost kind K.  S.first tile blocks; the histogram pass has sup_blocks more for the
+// support.
 template <int K>
-Error scan_pass(const PriceInput &in, bool fp64, bool gather, int TI, int ncb, int64_t ntiles, int grid,
-                const float4 *rows, const float4 *cols, const Geo *geo, float *tmin, unsigned long long *hist,
-                int32_t *ci, int32_t *cj, unsigned long long cap, unsigned *ncand, cudaStream_t st) {
-    const bool jmode = in.jn >= 0;
-#define OT_SCAN_ARGS in.m, in.n, TI, ncb, ntiles, rows, cols, in.sx, in.sy, in.tx, in.ty, in.u, in.v, in.C, geo, tmin, \
-                     hist, ci, cj, cap, ncand
-#define OT_JSCAN_ARGS in.n, in.jn, ntiles, in.ji, in.jj, rows, cols, in.sx, in.sy, in.tx, in.ty, in.u, in.v, in.C, geo, \
-                      tmin, hist, ci, cj, cap, ncand
-    if constexpr (K == K_DN) {
-        if (jmode) {
-            if (gather) jscan_kernel<K, true, true><<<grid, kPT, 0, st>>>(OT_JSCAN_ARGS);
-            else jscan_kernel<K, true, false><<<grid, kPT, 0, st>>>(OT_JSCAN_ARGS);
-        } else {
-            if (gather) scan_kernel<K, true, true><<<grid, kPT, 0, st>>>(OT_SCAN_ARGS);
-            else scan_kernel<K, true, false><<<grid, kPT, 0, st>>>(OT_SCAN_ARGS);
+Error scan_pass(const PriceInput &in, const ScanData &D, bool gather, const SupArgs &S, int sup_blocks, int32_t *ci,
+                int32_t *cj, unsigned long long cap, cudaStream_t st) {
+    const int grid = S.first + (gather ? 0 : sup_blocks);
+    unsigned *ncand = &D.geo->ncand;
+    auto scan = [&](auto ga) {
+        constexpr bool G = decltype(ga)::value;
+        if (in.jn >= 0) {
+            auto j = [&](auto fp) {
+                jscan_kernel<K, decltype(fp)::value, G><<<grid, kPT, 0, st>>>(
+                    in.n, in.jn, D.ntiles, S, in.ji, in.jj, D.rows, D.cols, in.sx, in.sy, in.tx, in.ty, in.u, in.v,
+                    in.C, D.geo, D.tmin, D.hist, ci, cj, cap, ncand);
+            };
+            if constexpr (K == K_DN) j(std::true_type());
+            else D.fp64 ? j(std::true_type()) : j(std::false_type());
+            return;
         }
-    } else {
-        if (jmode) {
-            if (fp64) {
-                if (gather) jscan_kernel<K, true, true><<<grid, kPT, 0, st>>>(OT_JSCAN_ARGS);
-                else jscan_kernel<K, true, false><<<grid, kPT, 0, st>>>(OT_JSCAN_ARGS);
-            } else {
-                if (gather) jscan_kernel<K, false, true><<<grid, kPT, 0, st>>>(OT_JSCAN_ARGS);
-                else jscan_kernel<K, false, false><<<grid, kPT, 0, st>>>(OT_JSCAN_ARGS);
-            }
-        } else {
-            if (fp64) {
-                if (gather) scan_kernel<K, true, true><<<grid, kPT, 0, st>>>(OT_SCAN_ARGS);
-                else scan_kernel<K, true, false><<<grid, kPT, 0, st>>>(OT_SCAN_ARGS);
-            } else {
-                if (gather) scan_kernel<K, false, true><<<grid, kPT, 0, st>>>(OT_SCAN_ARGS);
-                else scan_kernel<K, false, false><<<grid, kPT, 0, st>>>(OT_SCAN_ARGS);
+        if constexpr (K != K_DN) {
+            if (!D.fp64) {
+                tile_scan_kernel<K, G><<<grid, kPT, 0, st>>>(in.m, in.n, D.G, D.nrg, S, D.rows, D.cols, D.srt, in.sx,
+                                                            in.sy, in.tx, in.ty, in.u, in.v, D.geo, D.list, D.tmin,
+                                                            D.hist, ci, cj, cap, ncand);
+                return;
             }
         }
-    }
-#undef OT_SCAN_ARGS
-#undef OT_JSCAN_ARGS
+        auto f = [&](auto rj) {
+            scan64_kernel<K, G, decltype(rj)::value><<<grid, kPT, 0, st>>>(
+                in.m, in.n, D.TI, D.ncb, D.ntiles, S, in.sx, in.sy, in.tx, in.ty, in.u, in.v, in.C, D.geo, D.tmin,
+                D.hist, ci, cj, cap, ncand);
+        };
+        D.narrow ? f(std::integral_constant<int, kRJNarrow>()) : f(std::integral_constant<int, kRJ>());
+    };
+    gather ? scan(std::true_type()) : scan(std::false_type());
     OT_LAUNCHED();
     return ok();
 }
 
+// FP32 forms, error bound and tile list.
 template <int K>
-Error support_pass(const PriceInput &in, bool fp64, int blocks, const float4 *rows, const float4 *cols,
-                   const Geo *geo, unsigned long long *hist, cudaStream_t st) {
-    const bool jmode = in.jn >= 0;
-    const long long jlim = jmode ? in.jlim : 0;
-    const double jcmax = jmode ? in.jcmax : 0.0;
-    if (fp64 || K == K_DN)
-        support_hist_kernel<K, true><<<blocks, 256, 0, st>>>(in.n, in.psi, in.sup_i, in.sup_j, rows, cols, in.sx,
-                                                             in.sy, in.tx, in.ty, in.u, in.v, in.C, jlim, jcmax,
-                                                             geo, hist);
-    else
-        support_hist_kernel<K, false><<<blocks, 256, 0, st>>>(in.n, in.psi, in.sup_i, in.sup_j, rows, cols, in.sx,
-                                                              in.sy, in.tx, in.ty, in.u, in.v, in.C, jlim, jcmax,
-                                                              geo, hist);
+Error prepare_tiles(const PriceInput &in, const ScanData &D, int sms, cudaStream_t st) {
+    const int m = in.m, n = in.n;
+    const int pb = (int)std::min<int64_t>(4 * sms, ceil_div((int64_t)m + n, 256 * kPrepPer));
+    const bool sort = in.jn < 0;
+    if (in.have_box) {
+        box_kernel<<<1, 32, 0, st>>>(in.box_lo[0], in.box_lo[1], in.box_hi[0], in.box_hi[1], D.geo);
+    } else {
+        bounds_kernel<<<pb, 256, 0, st>>>(m, n, in.sx, in.sy, in.tx, in.ty, D.geo);
+    }
     OT_LAUNCHED();
+    if (sort) {
+        cells_kernel<<<pb, 256, 0, st>>>(m, n, in.sx, in.sy, in.tx, in.ty, D.geo, D.cells, D.place);
+        OT_LAUNCHED();
+    }
+    prep_kernel<K == K_SQ><<<pb, 256, 0, st>>>(m, n, K, in.sx, in.sy, in.tx, in.ty, in.u, in.v, D.rows, D.cols,
+                                               D.cells, sort ? D.place : nullptr, D.srt, D.sdual, D.geo);
+    OT_LAUNCHED();
+    if (sort) {
+        const int64_t total = (int64_t)D.nrg * D.ncg;
+        groups_kernel<<<(unsigned)std::min<int64_t>(ceil_div((int64_t)D.nrg + D.ncg, 8), 8LL * sms), 256, 0, st>>>(
+            m, n, D.G, D.nrg, D.ncg, K == K_SQ ? -0.5f : 1.0f, D.srt, D.sdual, D.grp);
+        OT_LAUNCHED();
+        tiles_kernel<K><<<(unsigned)std::min<int64_t>(ceil_div(total, 256), 8LL * sms), 256, 0, st>>>(
+            D.nrg, total, D.grp, D.geo, D.list);
+        OT_LAUNCHED();
+    }
     return ok();
 }
 
@@ -818,6 +1270,22 @@ Error by_kind(int kind, F &&f) {
     case K_DN: return f(std::integral_constant<int, K_DN>());
     default: return fail(OT_ERR_ARG, "price_topk: unknown cost kind");
     }
+}
+
+// Capacity of the candidate buffer that needs no host round trip (a multiple of kSelT): four times
+// kmax, at least 8 and at most 128 tiles (the rank searches grow with tiles per candidate).
+unsigned spec_capacity(int32_t kmax) {
+    const int64_t want = ceil_div(4LL * kmax, kSelT) * kSelT;
+    return (unsigned)std::max<int64_t>(8 * kSelT, std::min<int64_t>(want, 128 * kSelT));
+}
+
+PriceStats stats_of(const Geo &g, int32_t kmax) {
+    PriceStats s;
+    s.gathered = g.ncand;
+    s.valid = g.nvalid;
+    s.selected = std::min<uint32_t>((uint32_t)kmax, g.nvalid);
+    s.err_bound = g.E;
+    return s;
 }
 
 }  // namespace
@@ -840,64 +1308,111 @@ Error price_topk(const PriceInput &in, int32_t *out_i, int32_t *out_j, double *o
         OT_CUDA(cudaGetDevice(&dev));
         OT_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     }
-    // tiles: TI rows x 2048 columns (aim for >= 4 tiles per SM), or kJT entries of the J list
-    const int ncb = (int)ceil_div(n, kTJ);
-    int TI = kPT;
-    while (TI > 8 && ceil_div(m, TI) * (int64_t)ncb < 4LL * sms) TI >>= 1;
-    if (in.rows > 0) TI = std::max(8, std::min(kPT, in.rows));
-    const int64_t ntiles = jmode ? ceil_div(in.jn, kJT) : (int64_t)ceil_div(m, TI) * ncb;
+    // FP64 tiles: TI rows x kPT * RJ columns (aim for >= 4 tiles per SM); J list: kJT entries; FP32
+    // tiles: G rows x 256 columns, one per warp (aim for >= 16 per SM before pruning)
+    ScanData D;
+    D.fp64 = fp64;
+    const bool tiled32 = !fp64 && !jmode;
+    D.narrow = n <= kNarrowN;
+    D.ncb = (int)ceil_div(n, kPT * (D.narrow ? kRJNarrow : kRJ));
+    D.TI = kPT;
+    while (D.TI > (D.narrow ? 4 : 8) && ceil_div(m, D.TI) * (int64_t)D.ncb < 4LL * sms) D.TI >>= 1;
+    D.ncg = (int)ceil_div(n, kCG);
+    D.G = 64;
+    while (D.G > 16 && ceil_div(m, D.G) * (int64_t)D.ncg < 16LL * sms) D.G >>= 1;
+    if (in.rows > 0) D.TI = D.G = std::max(8, std::min(kPT, in.rows));
+    D.nrg = (int)ceil_div(m, D.G);
+    D.ntiles = jmode ? ceil_div(in.jn, kJT) : (int64_t)ceil_div(m, D.TI) * D.ncb;
+    const int64_t ntiles = tiled32 ? (int64_t)D.nrg * D.ncg : D.ntiles;
 
-    DevTemp<Geo> geo;
-    DevTemp<float4> rows, cols;
-    DevTemp<float> tmin;
-    DevTemp<unsigned long long> hist;  // [2][kBins]: support removed / support included
-    OT_TRY(geo.alloc(1, st));
+    // one workspace: Geo, the two histograms (all pairs, the support's), FP32 points, tiles
+    DevTemp<char> ws;
+    size_t need = 0;
+    auto take = [&](size_t bytes) { const size_t at = need; need += (bytes + 255) & ~(size_t)255; return at; };
+    const size_t pts = (size_t)m + n;
+    const size_t o_geo = take(sizeof(Geo)), o_hist = take(sizeof(unsigned long long) * 2 * kBins);
+    const size_t o_cells = take(tiled32 ? sizeof(unsigned) * 2 * kCells : 0), zeroed = need;
+    const size_t o_rows = take(fp64 ? 0 : sizeof(float4) * m), o_cols = take(fp64 ? 0 : sizeof(float4) * n);
+    const size_t o_srt = take(tiled32 ? sizeof(float4) * pts : 0), o_dual = take(tiled32 ? sizeof(float) * pts : 0);
+    const size_t o_place = take(tiled32 ? sizeof(unsigned) * pts : 0);
+    const size_t o_grp = take(tiled32 ? sizeof(Group) * ((size_t)D.nrg + D.ncg) : 0);
+    const size_t o_list = take(tiled32 ? sizeof(unsigned) * ntiles : 0);
+    const size_t o_tmin = take(sizeof(float) * std::max<int64_t>(ntiles, 1));
+    const size_t o_rp = take(in.row_ptr ? 0 : sizeof(int32_t) * ((size_t)m + 1));
+    OT_TRY(ws.alloc((int64_t)need, st));
+    Geo *geo = D.geo = (Geo *)(ws.p + o_geo);
+    unsigned long long *hist = D.hist = (unsigned long long *)(ws.p + o_hist), *hist_sup = hist + kBins;
+    D.tmin = (float *)(ws.p + o_tmin);
     if (!fp64) {
-        OT_TRY(rows.alloc(m, st));
-        OT_TRY(cols.alloc(n, st));
+        D.rows = (float4 *)(ws.p + o_rows);
+        D.cols = (float4 *)(ws.p + o_cols);
     }
-    OT_TRY(tmin.alloc(ntiles, st));
-    OT_TRY(hist.alloc(2 * kBins, st));
-    OT_CUDA(cudaMemsetAsync(geo.p, 0, sizeof(Geo), st));
-    OT_CUDA(cudaMemsetAsync(hist.p, 0, sizeof(unsigned long long) * 2 * kBins, st));
+    if (tiled32) {
+        D.cells = (unsigned *)(ws.p + o_cells);
+        D.srt = (float4 *)(ws.p + o_srt);
+        D.sdual = (float *)(ws.p + o_dual);
+        D.place = (unsigned *)(ws.p + o_place);
+        D.grp = (Group *)(ws.p + o_grp);
+        D.list = (unsigned *)(ws.p + o_list);
+    }
+    OT_CUDA(cudaMemsetAsync(ws.p, 0, zeroed, st));
 
-    if (kind != K_DN) {
-        const int prep_blocks = (int)std::min<int64_t>(4 * sms, ceil_div(std::max(m, n), 256));
-        if (kind == K_SQ)
-            prep_kernel<true><<<prep_blocks, 256, 0, st>>>(m, n, in.sx, in.sy, in.tx, in.ty, in.u, in.v, in.origin_x,
-                                                           in.origin_y, rows.p, cols.p, geo.p);
-        else
-            prep_kernel<false><<<prep_blocks, 256, 0, st>>>(m, n, in.sx, in.sy, in.tx, in.ty, in.u, in.v, in.origin_x,
-                                                            in.origin_y, rows.p, cols.p, geo.p);
-        OT_LAUNCHED();
+    const int32_t *rp = in.row_ptr;   // support membership needs CSR rows
+    if (!rp) {
+        int32_t *own = (int32_t *)(ws.p + o_rp);
+        OT_TRY(build_row_ptr(in.sup_i, in.psi, m, own, st));
+        rp = own;
     }
-    bound_kernel<<<1, 32, 0, st>>>(geo.p, fp64 ? 1 : 0, kind);
-    OT_LAUNCHED();
+    if (!fp64)   // (E stays 0 in the FP64 variant)
+        OT_TRY(by_kind(kind, [&](auto kc) -> Error {
+            if constexpr (decltype(kc)::value == K_DN) return ok();
+            else return prepare_tiles<decltype(kc)::value>(in, D, sms, st);
+        }));
 
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(ntiles, 8LL * sms));
-    if (ntiles > 0) {
-        ktimer_begin(KT_SCAN_HIST, st);
+    SupArgs S{in.sup_i, in.sup_j, in.psi, jmode ? in.jlim : 0, jmode ? in.jcmax : 0.0, 0, hist_sup};
+    S.first = (int)std::max<int64_t>(1, tiled32 ? std::min<int64_t>(ceil_div(ntiles, kPT / 32), 3LL * sms)
+                                                : std::min<int64_t>(ntiles, 8LL * sms));
+    const int sup_blocks = (int)std::min<int64_t>(2 * sms, ceil_div(in.psi, 4 * kPT));
+    auto pass = [&](bool gather, int32_t *ci, int32_t *cj, unsigned long long cap) -> Error {
+        ktimer_begin(gather ? KT_SCAN_GATHER : KT_SCAN_HIST, st);
         OT_TRY(by_kind(kind, [&](auto kc) {
-            return scan_pass<decltype(kc)::value>(in, fp64, false, TI, ncb, ntiles, grid, rows.p, cols.p, geo.p,
-                                                  tmin.p, hist.p, nullptr, nullptr, 0, nullptr, st);
+            return scan_pass<decltype(kc)::value>(in, D, gather, S, sup_blocks, ci, cj, cap, st);
         }));
-        ktimer_end(KT_SCAN_HIST, st);
-        const double per_pair = kind == K_SQ ? 4.0 : (kind == K_EU ? 8.0 : 6.0);
-        ktimer_add_work(KT_SCAN_HIST, per_pair * (jmode ? (double)in.jn : (double)m * (double)n));
-    }
-    OT_CUDA(cudaMemcpyAsync(hist.p + kBins, hist.p, sizeof(unsigned long long) * kBins,
-                            cudaMemcpyDeviceToDevice, st));
-    if (in.psi > 0) {
-        const int sb = (int)std::min<int64_t>(4 * sms, ceil_div(in.psi, 256));
-        OT_TRY(by_kind(kind, [&](auto kc) {
-            return support_pass<decltype(kc)::value>(in, fp64, sb, rows.p, cols.p, geo.p, hist.p, st);
-        }));
-    }
-    threshold_kernel<<<1, 1024, 0, st>>>(hist.p, hist.p + kBins, std::max(in.kmax, 1), fp64 ? 1 : 0, geo.p);
+        ktimer_end(gather ? KT_SCAN_GATHER : KT_SCAN_HIST, st);
+        return ok();
+    };
+    if (ntiles > 0) OT_TRY(pass(false, nullptr, nullptr, 0));   // (an empty J list holds no support pair either)
+    threshold_kernel<<<1, 1024, 0, st>>>(hist, hist_sup, std::max(in.kmax, 1), fp64 ? 1 : 0, geo);
     OT_LAUNCHED();
     Geo hg;
-    OT_CUDA(cudaMemcpyAsync(&hg, geo.p, sizeof(Geo), cudaMemcpyDeviceToHost, st));
-    OT_CUDA(cudaStreamSynchronize(st));
+    {
+        // the gathered set rarely passes a few times kmax (its last bin is a sixteenth of an octave of
+        // |d|, plus the support's pairs and the FP32 window)
+        const unsigned cap = spec_capacity(in.kmax);
+        DevTemp<char> cand;
+        OT_TRY(cand.alloc((int64_t)cap * (2 * sizeof(int32_t) + sizeof(unsigned long long) + sizeof(unsigned)), st));
+        unsigned long long *skey = (unsigned long long *)cand.p;
+        unsigned *sjl = (unsigned *)(skey + cap);
+        int32_t *ci = (int32_t *)(sjl + cap), *cj = ci + cap;
+        if (ntiles > 0) OT_TRY(pass(true, ci, cj, cap));
+        ktimer_begin(KT_RECHECK, st);
+        select_sort_kernel<<<cap / kSelT, kSelT / 2, 0, st>>>(m, n, kind, cap, ci, cj, in.sx, in.sy, in.tx, in.ty, in.u,
+                                                              in.v, in.C, rp, in.sup_j, geo, skey, sjl);
+        OT_LAUNCHED();
+        ktimer_end(KT_RECHECK, st);
+        select_rank_kernel<<<cap / 64, 256, 0, st>>>(m, in.kmax, cap, skey, sjl, geo, out_i, out_j, out_d, out_count);
+        OT_LAUNCHED();
+        OT_CUDA(cudaMemcpyAsync(&hg, geo, sizeof(Geo), cudaMemcpyDeviceToHost, st));
+        OT_CUDA(cudaStreamSynchronize(st));
+        // the pairs that pass 1 evaluated, in FP32 operations
+        const double per_pair = kind == K_SQ ? 4.0 : (kind == K_EU ? 8.0 : 6.0);
+        ktimer_add_work(KT_SCAN_HIST, per_pair * (jmode ? (double)in.jn
+                                                  : tiled32 ? (double)hg.ntile * D.G * kCG : (double)m * (double)n));
+        if (hg.gather_bound <= cap) {
+            if (stats) *stats = stats_of(hg, in.kmax);
+            return ok();
+        }
+    }
     const unsigned long long cap = hg.gather_bound;
     if (!fp64 && cap > kMaxWindowPairs) {
         // fewer negative keys than kmax and a flood of pairs inside the FP32 window [0, E] (duals
@@ -908,58 +1423,39 @@ Error price_topk(const PriceInput &in, int32_t *out_i, int32_t *out_j, double *o
     }
     if (cap > 0x7fffffffull) return fail(OT_ERR_OOM, "price_topk: candidate set exceeds 2^31 pairs");
 
+    // beyond the fixed capacity: pass 2 again into buffers of the exact size, then stable radix sorts
+    const int64_t cnt = (int64_t)cap;
     DevTemp<int32_t> ci, cj;
-    OT_TRY(ci.alloc((int64_t)cap, st));
-    OT_TRY(cj.alloc((int64_t)cap, st));
-    if (cap > 0 && ntiles > 0) {
-        ktimer_begin(KT_SCAN_GATHER, st);
-        OT_TRY(by_kind(kind, [&](auto kc) {
-            return scan_pass<decltype(kc)::value>(in, fp64, true, TI, ncb, ntiles, grid, rows.p, cols.p, geo.p,
-                                                  tmin.p, nullptr, ci.p, cj.p, cap, &geo.p->ncand, st);
-        }));
-        ktimer_end(KT_SCAN_GATHER, st);
-    }
-    // support membership needs CSR rows
-    DevTemp<int32_t> rp_tmp;
-    const int32_t *rp = in.row_ptr;
-    if (!rp) {
-        OT_TRY(rp_tmp.alloc((int64_t)m + 1, st));
-        OT_TRY(build_row_ptr(in.sup_i, in.psi, m, rp_tmp.p, st));
-        rp = rp_tmp.p;
-    }
+    OT_TRY(ci.alloc(cnt, st));
+    OT_TRY(cj.alloc(cnt, st));
+    OT_CUDA(cudaMemsetAsync(&geo->ncand, 0, sizeof(unsigned), st));
+    OT_CUDA(cudaMemsetAsync(&geo->nvalid, 0, sizeof(unsigned), st));
+    OT_TRY(pass(true, ci.p, cj.p, cap));
     DevTemp<uint64_t> key, dkey;
     DevTemp<uint32_t> val;
     DevTemp<double> dval;
-    const int64_t cnt = (int64_t)cap;
     OT_TRY(key.alloc(cnt, st));
     OT_TRY(dkey.alloc(cnt, st));
     OT_TRY(val.alloc(cnt, st));
     OT_TRY(dval.alloc(cnt, st));
-    if (cnt > 0) {
-        const int rb = (int)std::min<int64_t>(8 * sms, ceil_div(cnt, 256));
-        ktimer_begin(KT_RECHECK, st);
-        recheck_kernel<<<rb, 256, 0, st>>>(m, n, kind, (unsigned long long)cnt, ci.p, cj.p, in.sx, in.sy, in.tx,
-                                           in.ty, in.u, in.v, in.C, rp, in.sup_j, geo.p, key.p, val.p, dkey.p, dval.p);
-        OT_LAUNCHED();
-        ktimer_end(KT_RECHECK, st);
-        int jbits = 1;
-        while (jbits < 64 && ((uint64_t)m * (uint64_t)n - 1) >> jbits) ++jbits;
-        OT_TRY(radix_sort_pairs(key.p, val.p, cnt, jbits, st));
-        rekey_kernel<<<rb, 256, 0, st>>>((unsigned long long)cnt, val.p, dkey.p, key.p);
-        OT_LAUNCHED();
-        OT_TRY(radix_sort_pairs(key.p, val.p, cnt, 64, st));
-    }
-    finalize_kernel<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(in.kmax, 256), 4 * sms)), 256, 0, st>>>(
-        in.kmax, val.p, ci.p, cj.p, dval.p, geo.p, out_i, out_j, out_d, out_count);
+    const int rb = (int)std::min<int64_t>(8 * sms, ceil_div(cnt, 256));
+    ktimer_begin(KT_RECHECK, st);
+    recheck_kernel<<<rb, 256, 0, st>>>(m, n, kind, cap, ci.p, cj.p, in.sx, in.sy, in.tx, in.ty, in.u, in.v, in.C, rp,
+                                       in.sup_j, geo, key.p, val.p, dkey.p, dval.p);
     OT_LAUNCHED();
-    if (stats) {
-        OT_CUDA(cudaMemcpyAsync(&hg, geo.p, sizeof(Geo), cudaMemcpyDeviceToHost, st));
-        OT_CUDA(cudaStreamSynchronize(st));
-        stats->gathered = hg.ncand;
-        stats->valid = hg.nvalid;
-        stats->selected = std::min<uint32_t>((uint32_t)in.kmax, hg.nvalid);
-        stats->err_bound = hg.E;
-    }
+    ktimer_end(KT_RECHECK, st);
+    int jbits = 1;
+    while (jbits < 64 && ((uint64_t)m * (uint64_t)n - 1) >> jbits) ++jbits;
+    OT_TRY(radix_sort_pairs(key.p, val.p, cnt, jbits, st));
+    rekey_kernel<<<rb, 256, 0, st>>>(cap, val.p, dkey.p, key.p);
+    OT_LAUNCHED();
+    OT_TRY(radix_sort_pairs(key.p, val.p, cnt, 64, st));
+    finalize_kernel<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(in.kmax, 256), 4 * sms)), 256, 0, st>>>(
+        in.kmax, val.p, ci.p, cj.p, dval.p, geo, out_i, out_j, out_d, out_count);
+    OT_LAUNCHED();
+    OT_CUDA(cudaMemcpyAsync(&hg, geo, sizeof(Geo), cudaMemcpyDeviceToHost, st));
+    OT_CUDA(cudaStreamSynchronize(st));
+    if (stats) *stats = stats_of(hg, in.kmax);
     return ok();
 }
 

@@ -16,7 +16,9 @@ struct PriceInput {
     int64_t psi = 0;
     int32_t kmax = 0;
     int32_t precision = 1;  // 1: FP32 scan + FP64 recheck; 0: FP64 scan
-    int32_t origin_x = 0, origin_y = 0;  // coordinate shift applied before the FP32 form
+    // bounding box of all points (x, y); found on the device unless have_box
+    bool have_box = false;
+    int32_t box_lo[2] = {0, 0}, box_hi[2] = {0, 0};
     int32_t num_sms = 0;
     int32_t rows = 0;       // rows per scan tile (8..256); 0: chosen from the problem size
     int32_t kind = OT_COST_SQEUCLID;   // ot_cost_kind
@@ -53,13 +55,9 @@ struct PriceStats {
 };
 
 // Selection written to out_i/out_j/out_d (capacity kmax, device) and *out_count (device).
-// One host synchronisation (to size the candidate buffer).  Stats filled when non-null.
+// Synchronises the stream once, at the end.  Stats filled when non-null.
 Error price_topk(const PriceInput &in, int32_t *out_i, int32_t *out_j, double *out_d,
                  int32_t *out_count, PriceStats *stats, cudaStream_t st);
-
-// Integer origin (midpoint of the bounding box of all points), device inputs, host result.
-Error coord_origin(int32_t m, int32_t n, const int32_t *sx, const int32_t *sy, const int32_t *tx,
-                   const int32_t *ty, int32_t *ox, int32_t *oy, cudaStream_t st);
 
 // row_ptr[i] = first support index with sup_i >= i (i in [0, m]); sup_i sorted.
 Error build_row_ptr(const int32_t *sup_i, int64_t psi, int32_t m, int32_t *row_ptr, cudaStream_t st);

@@ -68,8 +68,7 @@ extern "C" int ot_price_topk_noalloc(int32_t m, int32_t n, const int32_t *sx, co
         in.sup_i = sup_i; in.sup_j = sup_j; in.psi = psi;
         in.kmax = kmax;
         in.precision = precision;
-        e = coord_origin(m, n, sx, sy, tx, ty, &in.origin_x, &in.origin_y, st);
-        if (e.code == OT_OK) e = price_topk(in, out_i, out_j, out_d, out_count, nullptr, st);
+        e = price_topk(in, out_i, out_j, out_d, out_count, nullptr, st);
     }
     if (e.code == OT_ERR_BUF_TOO_SMALL)
         e.msg = "ot_price_topk_noalloc: the candidate set of this call does not fit the fixed 24 MiB scratch; "

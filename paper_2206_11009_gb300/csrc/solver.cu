@@ -228,7 +228,7 @@ struct ot_ipm {
     // device problem
     double *a_s = nullptr, *b_s = nullptr, *C = nullptr;
     int32_t *sx = nullptr, *sy = nullptr, *tx = nullptr, *ty = nullptr;
-    int32_t ox = 0, oy = 0;
+    int32_t box_lo[2] = {0, 0}, box_hi[2] = {0, 0};   // bounding box of all points
     CostDev cd;
     double *u = nullptr, *v = nullptr;
     Support S[2];
@@ -369,6 +369,11 @@ Error forest_setup(ot_ipm *h, const Support &S, bool *is_forest, cudaStream_t st
     return ok();
 }
 
+void set_box(PriceInput &in, const ot_ipm *h) {
+    in.have_box = true;
+    for (int q = 0; q < 2; ++q) { in.box_lo[q] = h->box_lo[q]; in.box_hi[q] = h->box_hi[q]; }
+}
+
 Error price_support(ot_ipm *h, const Support &S, int32_t kmax, int32_t *count, PriceStats *ps, bool use_j) {
     PriceInput in;
     in.kind = h->cd.kind;
@@ -389,12 +394,11 @@ Error price_support(ot_ipm *h, const Support &S, int32_t kmax, int32_t *count, P
     in.sup_i = S.i; in.sup_j = S.j; in.row_ptr = S.row_ptr; in.psi = S.psi;
     in.kmax = kmax;
     in.precision = h->opt.precision;
-    in.origin_x = h->ox; in.origin_y = h->oy;
+    set_box(in, h);
     in.num_sms = h->num_sms;
     in.rows = h->opt.scan_rows;
     OT_TRY(price_topk(in, h->pi, h->pj, h->pd, h->pcount, ps, h->st));
-    OT_CUDA(cudaMemcpyAsync(count, h->pcount, sizeof(int32_t), cudaMemcpyDeviceToHost, h->st));
-    OT_CUDA(cudaStreamSynchronize(h->st));
+    *count = (int32_t)ps->selected;
     return ok();
 }
 
@@ -900,13 +904,11 @@ Error warm_support(ot_ipm *h, const ot_options &o, cudaStream_t st) {
     in.precision = o.precision;
     in.kind = h->cd.kind;
     in.C = h->C;
-    in.origin_x = h->ox;
-    in.origin_y = h->oy;
+    set_box(in, h);
     in.num_sms = h->num_sms;
-    OT_TRY(price_topk(in, wi.p, wj.p, dd.p, wc.p, nullptr, st));
-    int32_t k = 0;
-    OT_CUDA(cudaMemcpyAsync(&k, wc.p, sizeof(k), cudaMemcpyDeviceToHost, st));
-    OT_CUDA(cudaStreamSynchronize(st));
+    PriceStats ps;
+    OT_TRY(price_topk(in, wi.p, wj.p, dd.p, wc.p, &ps, st));
+    const int32_t k = (int32_t)ps.selected;
     if (k <= 0) return ok();
     OT_TRY(merge_support(A, keep.p, wi.p, wj.p, k, 1.0, m, n, B, st));
     h->cur = 1 - h->cur;
@@ -1156,8 +1158,8 @@ Error create_impl(const ot_problem *P, const ot_options *O, ot_ipm *h) {
     for (int j = 0; j < n0; ++j) { xmin = std::min(xmin, G0[j]); xmax = std::max(xmax, G0[j]); ymin = std::min(ymin, H0[j]); ymax = std::max(ymax, H0[j]); }
     if (xmin <= -(1 << 14) || ymin <= -(1 << 14) || xmax >= (1 << 14) || ymax >= (1 << 14))
         return fail(OT_ERR_ARG, "problem: coordinates must satisfy |x|, |y| < 2^14");
-    h->ox = (int32_t)(((int64_t)xmin + xmax) / 2);
-    h->oy = (int32_t)(((int64_t)ymin + ymax) / 2);
+    h->box_lo[0] = xmin; h->box_lo[1] = ymin;
+    h->box_hi[0] = xmax; h->box_hi[1] = ymax;
 
     int dev;
     OT_CUDA(cudaGetDevice(&dev));
@@ -1734,8 +1736,7 @@ int ot_price_topk(int32_t m, int32_t n, const int32_t *sx, const int32_t *sy, co
     in.sup_i = sup_i; in.sup_j = sup_j; in.psi = psi;
     in.kmax = kmax;
     in.precision = precision;
-    Error e = coord_origin(m, n, sx, sy, tx, ty, &in.origin_x, &in.origin_y, st);
-    if (e.code == OT_OK) e = price_topk(in, out_i, out_j, out_d, out_count, nullptr, st);
+    Error e = price_topk(in, out_i, out_j, out_d, out_count, nullptr, st);
     if (e.code != OT_OK) set_thread_error(e.msg.c_str());
     return e.code;
 }
@@ -1767,7 +1768,6 @@ int ot_price_topk_ex(int32_t m, int32_t n, const int32_t *sx, const int32_t *sy,
     in.rows = po.scan_rows;
     JSet J;
     Error e = ok();
-    if (!dense) e = coord_origin(m, n, sx, sy, tx, ty, &in.origin_x, &in.origin_y, st);
     if (e.code == OT_OK && po.jset_cmax > 0) {
         e = jset_build(po.cost, m, n, sx, sy, tx, ty, po.C, po.jset_cmax, &J, st);
         in.ji = J.i; in.jj = J.j; in.jn = J.n; in.jlim = J.lim; in.jcmax = J.cmax;
