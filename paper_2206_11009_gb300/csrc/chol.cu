@@ -61,26 +61,38 @@ __global__ void sp_rows_kernel(int m, const int32_t *__restrict__ rp, const doub
     }
 }
 
+// one warp per row i: lane by lane the pairs (a, b) of its kept entries in the order of the serial
+// double loop (entry a's pairs start at rank(a) (d - 1), d the row's kept entries)
 __global__ void asm_emit_kernel(int m, int n, const int32_t *__restrict__ rp, const int32_t *__restrict__ sj,
                                 const double *__restrict__ th, const uint8_t *__restrict__ keep,
                                 const double *__restrict__ Mt, const uint32_t *__restrict__ off,
                                 uint64_t *__restrict__ key, uint32_t *__restrict__ val, double *__restrict__ raw) {
-    GS(i, m) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < m;
+         i += ((int64_t)gridDim.x * blockDim.x) >> 5) {
         const int lo = rp[i], hi = rp[i + 1];
-        uint32_t o = off[i];
         const double mi = Mt[i] > 0 ? 1.0 / Mt[i] : 0.0;
+        uint32_t o = off[i];
         for (int a = lo; a < hi; ++a) {
             if (!keep[a]) continue;
-            for (int b = lo; b < hi; ++b) {
-                if (a == b || !keep[b]) continue;
-                key[o] = (uint64_t)sj[a] * (uint64_t)n + (uint64_t)sj[b];
-                val[o] = o;
-                raw[o] = -(th[a] * th[b]) * mi;
-                ++o;
+            const double ta = th[a];
+            const uint64_t ka = (uint64_t)sj[a] * (uint64_t)n;
+            for (int b0 = lo; b0 < hi; b0 += 32) {
+                const int b = b0 + lane;
+                const bool take = b < hi && b != a && keep[b];
+                const unsigned bal = __ballot_sync(0xffffffffu, take);
+                if (take) {
+                    const uint32_t at = o + __popc(bal & ((1u << lane) - 1u));
+                    key[at] = ka + (uint64_t)sj[b];
+                    val[at] = at;
+                    raw[at] = -(ta * th[b]) * mi;
+                }
+                o += __popc(bal);
             }
         }
     }
 }
+
 
 // diagonal of the kept graph's Schur complement: sum over kept pairs theta * (kept others) / Mt
 __global__ void sp_diag_kernel(int n, const int32_t *__restrict__ cp, const int32_t *__restrict__ perm,
@@ -353,7 +365,7 @@ Error chol_assemble(Chol &C, Newton &W, const Support &S, double drop, bool *pat
     OT_TRY(flag.alloc(total, st)); OT_TRY(pos.alloc(total, st)); OT_TRY(start.alloc(total, st));
     uint32_t nu = 0;
     if (total > 0) {
-        asm_emit_kernel<<<gridn(m), kT, 0, st>>>(m, n, S.row_ptr, S.j, W.theta, C.keep, C.Mt, off.p, key.p, val.p,
+        asm_emit_kernel<<<gridn(32LL * m), kT, 0, st>>>(m, n, S.row_ptr, S.j, W.theta, C.keep, C.Mt, off.p, key.p, val.p,
                                                  raw.p);
         OT_LAUNCHED();
         int bits = 1;
@@ -386,6 +398,7 @@ Error chol_assemble(Chol &C, Newton &W, const Support &S, double drop, bool *pat
                                             C.Adiag);
     OT_LAUNCHED();
     C.nnzA = nu;
+    if (!pattern_changed) return ok();
     // pattern on the host (for the symbolic analysis and change detection)
     std::vector<int32_t> hp(n + 1), hj(nu);
     OT_CUDA(cudaMemcpyAsync(hp.data(), C.Ap, sizeof(int32_t) * (n + 1), cudaMemcpyDeviceToHost, st));

@@ -52,10 +52,9 @@ struct Chol {
 struct DenseLDL {
     int32_t n = 0;
     double *A = nullptr;      // n x n column-major; strictly lower part holds L after dense_factor
-    double *LD = nullptr;     // n x 64 panel scratch (L21 D1)
-    double *Linv = nullptr;   // n x 64: inverses of the unit lower diagonal blocks
-    double *D = nullptr, *d0 = nullptr, *z = nullptr, *part = nullptr;
-    unsigned *bar = nullptr;
+    double *LD = nullptr;     // n x 32 panel scratch (L21 D1; the block's L in the block's rows)
+    double *Linv = nullptr;   // n x 32: inverses of the unit lower diagonal blocks
+    double *D = nullptr, *d0 = nullptr, *z = nullptr;
     int *err = nullptr;
 };
 
@@ -72,7 +71,8 @@ void chol_free(Chol &C);
 // Assemble the Schur complement of the support graph with its negligible pairs dropped: a pair
 // whose theta is below drop x (largest theta of its source row) is left out (drop = 0: the exact
 // S_M = N - V^T M^-1 V).  Off-diagonal part by rows of V; diagonal by the cancellation-free form
-// over the kept pairs, so every connected component still has S e = 0.  Sets *pattern_changed.
+// over the kept pairs, so every connected component still has S e = 0.  Sets *pattern_changed; NULL
+// (the dense factor, which needs no symbolic analysis) leaves the host's copy of the pattern alone.
 Error chol_assemble(Chol &C, Newton &W, const Support &S, double drop, bool *pattern_changed, cudaStream_t st);
 
 // Minimum-degree ordering and the pattern of L (host), uploaded to the device.  Returns

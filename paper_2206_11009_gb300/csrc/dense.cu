@@ -4,12 +4,17 @@
 // (a quarter of n^2 on 64x64 images), and a sparse factorisation then only adds dependency-chain
 // latency.  This path factors the dense matrix (column-major, FP64) with a blocked right-looking
 // LDL^T: per panel of kB columns
-//   (1) the kB x kB diagonal block in shared memory, one CTA (pivots keeping less than eps of
-//       their original diagonal become +infinity: the column is zeroed, Section 4.2);
-//   (2) the panel below, L21 = A21 L11^-T D1^-1, one thread per row, and LD = L21 D1;
-//   (3) the trailing update A22 -= LD L21^T on 64 x 64 tiles of the lower triangle.
-// Solves run in one cooperative launch: forward and backward substitution panel by panel with a
-// bounded grid barrier between the diagonal-block step and the update of the rest.
+//   (1) panel: every CTA eliminates the kB x kB diagonal block and its own 32 rows below together
+//       (pivots keeping less than eps of their original diagonal become +infinity: the column is
+//       zeroed, Section 4.2), which yields L21 and LD = L21 D1 without a separate block inverse;
+//   (2) the trailing update A22 -= LD L21^T on tiles of the lower triangle; one CTA more inverts
+//       the panel's unit block for the solves.
+// What bounds it here: a warp's FP64 multiply-add occupies its scheduler for 64 cycles (measured;
+// 1.7 per cycle and SM in all), a division for 650, so the work goes to as many SMs as there are
+// and nothing is computed twice on the chain except the small diagonal block.
+// Solves run in one cooperative launch, one CTA per block row: each waits for the blocks of the
+// solution it needs as they appear, so a panel costs one block product and one hand-over instead
+// of two grid barriers.
 #include "chol.cuh"
 #include "primitives.cuh"
 
@@ -18,7 +23,7 @@
 namespace ot {
 namespace {
 
-constexpr int kB = 64;      // panel width
+constexpr int kB = 32;      // panel width
 constexpr int kT = 256;
 
 #define GSD(var, count) \
@@ -28,256 +33,269 @@ inline unsigned gridd(int64_t work) {
     return (unsigned)std::max<int64_t>(1, std::min<int64_t>(4096, ceil_div(work, kT)));
 }
 
+// one warp per row
 __global__ void dense_scatter_kernel(int n, const int32_t *__restrict__ Ap, const int32_t *__restrict__ Aj,
                                      const double *__restrict__ Ax, const double *__restrict__ Adiag,
                                      double *__restrict__ A, double *__restrict__ d0) {
-    GSD(r, n) {
-        for (int e = Ap[r]; e < Ap[r + 1]; ++e) A[(int64_t)Aj[e] * n + r] = Ax[e];
-        A[(int64_t)r * n + r] = Adiag[r];
-        d0[r] = Adiag[r];
+    const int lane = threadIdx.x & 31;
+    for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n;
+         r += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        // the values of row r, at (r, column): the matrix is symmetric, so they fill column r
+        for (int e = Ap[r] + lane; e < Ap[r + 1]; e += 32) A[r * n + Aj[e]] = Ax[e];
+        if (lane == 0) {
+            A[r * n + r] = Adiag[r];
+            d0[r] = Adiag[r];
+        }
     }
 }
 
-// (1) diagonal block [k, k+bs) in shared memory
+// (1) Panel [k, k + bs): warps 0-3 hold the diagonal block's rows, warps 4-7 the CTA's 32 rows below
+// (one row per lane, columns w, w + 4, ... of warp w in registers).  Step j: the owners of column j
+// publish it, then every row takes l = a_rj / d_j and a_rc -= l a_cj for its later columns.  1 / d
+// from the hardware's approximation by one step of Halley's iteration (cubic: the relative error e
+// becomes e^3), applied to the quotient: three dependent multiply-adds instead of a division.
+// CTA 0 writes D and the block's L.  32 steps of about 500 cycles; the substitution with one thread
+// per row that it replaced took 350 us per 64 columns at n = 961 (and the diagonal block 210 us).
 __global__ void __launch_bounds__(kT)
-dense_diag_kernel(int n, int k, int bs, double *__restrict__ A, double *__restrict__ D,
-                  const double *__restrict__ d0, double eps, double *__restrict__ Linv) {
-    __shared__ double S[kB][kB + 1];
-    __shared__ double s_d;
-    __shared__ int s_inf;
-    for (int t = threadIdx.x; t < bs * bs; t += blockDim.x) {
-        const int i = t % bs, j = t / bs;
-        S[i][j] = (i >= j) ? A[(int64_t)(k + j) * n + (k + i)] : 0.0;
+dense_panel_kernel(int n, int k, int bs, double *__restrict__ A, double *__restrict__ D,
+                   const double *__restrict__ d0, double eps, double *__restrict__ LD) {
+    __shared__ double col[2][2][kB];
+    __shared__ double thr[kB];
+    const int lane = threadIdx.x & 31, half = threadIdx.x >> 7, w = (threadIdx.x >> 5) & 3;
+    const int r = half ? k + bs + (int)blockIdx.x * 32 + lane : k + lane;
+    const bool live = r < n && (half || lane < bs);
+    if (threadIdx.x < kB) thr[threadIdx.x] = (int)threadIdx.x < bs ? eps * d0[k + threadIdx.x] : 0.0;
+    double a[kB / 4];
+#pragma unroll
+    for (int q = 0; q < kB / 4; ++q) {
+        const int c = w + 4 * q;
+        a[q] = live && c < bs ? A[(int64_t)(k + c) * n + r] : 0.0;
     }
-    __syncthreads();
-    for (int j = 0; j < bs; ++j) {
-        if (threadIdx.x == 0) {
-            const double d = S[j][j];
-            s_inf = !(d > eps * d0[k + j]);
-            s_d = d;
-            D[k + j] = s_inf ? INFINITY : d;
-        }
-        __syncthreads();
-        const double d = s_d;
-        const int inf = s_inf;
-        for (int i = j + 1 + threadIdx.x; i < bs; i += blockDim.x) S[i][j] = inf ? 0.0 : S[i][j] / d;
-        __syncthreads();
-        if (!inf) {
-            // S[i][l] -= l_ij d l_lj  for j < l <= i < bs
-            const int m2 = bs - j - 1;
-            for (int t = threadIdx.x; t < m2 * m2; t += blockDim.x) {
-                const int i = j + 1 + t / m2, l = j + 1 + t % m2;
-                if (l <= i) S[i][l] -= S[i][j] * d * S[l][j];
-            }
-        }
-        __syncthreads();
-    }
-    for (int t = threadIdx.x; t < bs * bs; t += blockDim.x) {
-        const int i = t % bs, j = t / bs;
-        if (i > j) A[(int64_t)(k + j) * n + (k + i)] = S[i][j];
-    }
-    // inverse of the unit lower block, column by column: X[:,c] solves L X[:,c] = e_c, written
-    // to Linv (row k+i, column c) so that the solves need no serial substitution
-    __syncthreads();
-    for (int c = threadIdx.x; c < bs; c += blockDim.x) {
-        double x[kB];
-        for (int i = 0; i < bs; ++i) {
-            double t = (i == c) ? 1.0 : 0.0;
-            for (int l = c; l < i; ++l) t -= S[i][l] * x[l];
-            x[i] = (i < c) ? 0.0 : t;
-        }
-        for (int i = 0; i < bs; ++i) Linv[(int64_t)c * n + (k + i)] = x[i];
-    }
-}
-
-// (2) panel rows r in [k+bs, n): x D1 L11^T = A(r, k:k+bs)  ->  L21(r,:) = x, LD(r,:) = x D1
-__global__ void __launch_bounds__(kT)
-dense_panel_kernel(int n, int k, int bs, double *__restrict__ A, const double *__restrict__ D,
-                   double *__restrict__ LD /* n x kB, column-major with ld n */) {
-    __shared__ double L11[kB][kB + 1];
-    __shared__ double Ds[kB];
-    for (int t = threadIdx.x; t < bs * bs; t += blockDim.x) {
-        const int i = t % bs, j = t / bs;
-        L11[i][j] = (i > j) ? A[(int64_t)(k + j) * n + (k + i)] : 0.0;
-    }
-    for (int t = threadIdx.x; t < bs; t += blockDim.x) Ds[t] = D[k + t];
-    __syncthreads();
-    const int r = k + bs + blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n) return;
-    double x[kB];
-#pragma unroll 8
+#pragma unroll
     for (int j = 0; j < kB; ++j) {
         if (j >= bs) break;
-        double t = A[(int64_t)(k + j) * n + r];
-        for (int l = 0; l < j; ++l) t -= x[l] * Ds[l] * L11[j][l];
-        const double dj = Ds[j];
-        x[j] = isinf(dj) ? 0.0 : t / dj;
+        double (*cj)[kB] = col[j & 1];
+        if (w == (j & 3)) cj[half][lane] = a[j >> 2];
+        __syncthreads();
+        const double d = cj[0][j], v = cj[half][lane];
+        const bool inf = !(d > thr[j]);
+        double r0;
+        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(d));
+        const double e = fma(-d, r0, 1.0), v0 = v * r0;
+        const double t = fma(e, e, e);
+        const double l = inf ? 0.0 : fma(v0, t, v0);
+#pragma unroll
+        for (int q = 0; q < kB / 4; ++q)
+            if (w + 4 * q > j) a[q] = fma(-l, cj[0][w + 4 * q], a[q]);
+        if (w == (j & 3) && live) {
+            if (half) {
+                A[(int64_t)(k + j) * n + r] = l;
+                LD[(int64_t)j * n + r] = inf ? 0.0 : v;
+            } else if (blockIdx.x == 0) {
+                a[j >> 2] = l;   // stored after the other CTAs' reads: see below
+                if (lane == 0) D[k + j] = inf ? INFINITY : d;
+            }
+        }
     }
-    for (int j = 0; j < bs; ++j) {
-        A[(int64_t)(k + j) * n + r] = x[j];
-        const double dj = Ds[j];
-        LD[(int64_t)j * n + r] = isinf(dj) ? 0.0 : x[j] * dj;
+    // the block's L goes to LD's rows of the block (the other CTAs read A's block unscaled);
+    // dense_update_kernel's last CTA moves it to A
+    if (!half && blockIdx.x == 0) {
+#pragma unroll
+        for (int q = 0; q < kB / 4; ++q) {
+            const int c = w + 4 * q;
+            if (c < bs && lane < bs) LD[(int64_t)c * n + k + lane] = lane > c ? a[q] : 0.0;
+        }
     }
 }
 
-// (3) A22(r, c) -= sum_l LD(r, l) L21(c, l) on the lower triangle, 64x64 tiles, 4x4 per thread
+// X = L11^-1 of panel k (unit lower, from LD's rows of the block), written to Linv, and L11 to A.
+// One CTA of kT threads: lane = column of X, warp w the rows w, w + 8, ...; step j publishes row j.
+__device__ void dense_invert_block(int n, int k, int bs, double *__restrict__ A, const double *__restrict__ LD,
+                                   double *__restrict__ Linv, double (*L)[kB + 1], double (*row)[kB]) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int t = threadIdx.x; t < kB * kB; t += kT) {
+        const int i = t % kB, j = t / kB;
+        const double l = i < bs && j < bs && i > j ? LD[(int64_t)j * n + k + i] : 0.0;
+        L[i][j] = l;
+        if (i < bs && j < bs && i > j) A[(int64_t)(k + j) * n + k + i] = l;
+    }
+    double x[kB / 8];
+#pragma unroll
+    for (int q = 0; q < kB / 8; ++q) x[q] = w + 8 * q == lane ? 1.0 : 0.0;
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kB; ++j) {
+        if (w == (j & 7)) row[j & 1][lane] = x[j >> 3];
+        __syncthreads();
+        const double xj = row[j & 1][lane];
+#pragma unroll
+        for (int q = 0; q < kB / 8; ++q)
+            if (w + 8 * q > j) x[q] = fma(-L[w + 8 * q][j], xj, x[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < kB / 8; ++q)
+        if (w + 8 * q < bs && lane < bs) Linv[(int64_t)lane * n + k + w + 8 * q] = x[q];
+}
+
+// (2) A22(r, c) -= sum_l LD(r, l) L21(c, l) on the lower triangle in T x T tiles (64: 4 x 4 per
+// thread; 32 while fewer than four tiles of 64 per SM are left: 2 x 2 per thread).  The last CTA
+// inverts the panel's block.
+template <int T>
 __global__ void __launch_bounds__(kT)
-dense_update_kernel(int n, int k, int bs, double *__restrict__ A, const double *__restrict__ LD) {
+dense_update_kernel(int n, int k, int bs, double *__restrict__ A, const double *__restrict__ LD,
+                    double *__restrict__ Linv) {
+    __shared__ double sm[2 * kB * T > kB * (kB + 1) + 2 * kB ? 2 * kB * T : kB * (kB + 1) + 2 * kB];
+    if (blockIdx.x == gridDim.x - 1) {
+        dense_invert_block(n, k, bs, A, LD, Linv, (double (*)[kB + 1])sm, (double (*)[kB])(sm + kB * (kB + 1)));
+        return;
+    }
+    constexpr int Q = T / 16;
+    double (*Ls)[T] = (double (*)[T])sm, (*Rs)[T] = (double (*)[T])(sm + kB * T);   // [depth][row], [depth][column]
     const int base = k + bs;
-    const int t = (n - base + 63) / 64;
     // tile index -> (ti, tj) with ti >= tj
     const int idx = blockIdx.x;
-    int ti = (int)((sqrt(8.0 * idx + 1.0) - 1.0) * 0.5);
+    int ti = (int)((sqrtf(8.0f * idx + 1.0f) - 1.0f) * 0.5f);
     while ((ti + 1) * (ti + 2) / 2 <= idx) ++ti;
     while (ti * (ti + 1) / 2 > idx) --ti;
     const int tj = idx - ti * (ti + 1) / 2;
-    if (ti >= t) return;
-    __shared__ double Ls[32][64 + 1];   // LD rows of tile ti   [l][r]
-    __shared__ double Rs[32][64 + 1];   // L21 rows of tile tj  [l][c]
-    const int r0 = base + ti * 64, c0 = base + tj * 64;
-    const int tr = (threadIdx.x % 16) * 4, tc = (threadIdx.x / 16) * 4;
-    double acc[4][4] = {};
-    for (int l0 = 0; l0 < bs; l0 += 32) {
-        const int lb = min(32, bs - l0);
-        __syncthreads();
-        for (int q = threadIdx.x; q < lb * 64; q += blockDim.x) {
-            const int l = q / 64, rr = q % 64;
-            const int r = r0 + rr, c = c0 + rr;
-            Ls[l][rr] = r < n ? LD[(int64_t)(l0 + l) * n + r] : 0.0;
-            Rs[l][rr] = c < n ? A[(int64_t)(k + l0 + l) * n + c] : 0.0;
+    const int r0 = base + ti * T, c0 = base + tj * T;
+    for (int q = threadIdx.x; q < kB * T; q += kT) {
+        const int l = q / T, rr = q % T;
+        Ls[l][rr] = r0 + rr < n ? LD[(int64_t)l * n + r0 + rr] : 0.0;
+        Rs[l][rr] = c0 + rr < n ? A[(int64_t)(k + l) * n + c0 + rr] : 0.0;
+    }
+    const int tr = (threadIdx.x % 16) * Q, tc = (threadIdx.x / 16) * Q;
+    double acc[Q][Q];
+#pragma unroll
+    for (int w = 0; w < Q; ++w)
+#pragma unroll
+        for (int u = 0; u < Q; ++u) {
+            const int r = r0 + tr + u, c = c0 + tc + w;
+            acc[u][w] = r < n && c < n && r >= c ? A[(int64_t)c * n + r] : 0.0;
         }
-        __syncthreads();
-        for (int l = 0; l < lb; ++l) {
-            double a[4], b[4];
+    __syncthreads();
+    for (int l = 0; l < kB; ++l) {   // (a panel with rows below it is full)
+        double a[Q], b[Q];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) { a[u] = Ls[l][tr + u]; b[u] = Rs[l][tc + u]; }
+        for (int u = 0; u < Q; ++u) { a[u] = Ls[l][tr + u]; b[u] = Rs[l][tc + u]; }
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
+        for (int u = 0; u < Q; ++u)
 #pragma unroll
-                for (int w = 0; w < 4; ++w) acc[u][w] += a[u] * b[w];
-        }
+            for (int w = 0; w < Q; ++w) acc[u][w] = fma(-a[u], b[w], acc[u][w]);
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+    for (int w = 0; w < Q; ++w)
 #pragma unroll
-        for (int w = 0; w < 4; ++w) {
+        for (int u = 0; u < Q; ++u) {
             const int r = r0 + tr + u, c = c0 + tc + w;
-            if (r < n && c < n && r >= c) A[(int64_t)c * n + r] -= acc[u][w];
+            if (r < n && c < n && r >= c) A[(int64_t)c * n + r] = acc[u][w];
         }
 }
 
-// forward L z = b, y = D^-1 z, backward L^T x = y; one cooperative launch.  The diagonal blocks
-// are applied through their stored inverses (small GEMVs by block 0), the off-diagonal panels by
-// all blocks; one grid barrier after each step.
-__global__ void __launch_bounds__(kT)
+// ------------------------------------------------------------------------ solves
+// Forward L z = b, y = D^-1 z, backward L^T x = y.  CTA i owns block row i (kB rows, four warps: warp
+// g takes depths 8 g .. 8 g + 7 of every block product); the blocks of L that it will need are loaded
+// ahead of the wait.  z and x are preset to an all-ones pattern that no result has; a value that
+// differs is complete, so data and flag arrive in one load.  Every wait is bounded.
+constexpr int kST = 128;
+constexpr unsigned long long kUnset = ~0ull;
+
+__device__ __forceinline__ void publish(double *p, double v) {
+    unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    if (b == kUnset) b = 0x7ff8000000000000ull;   // a NaN from the caller's data stays a NaN
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" :: "l"(p), "l"(b) : "memory");
+}
+
+// this lane's value of p[0 .. 7] (lane & 7; entries at or beyond `valid` are zero) once all are set;
+// false when the wait gave up
+__device__ __forceinline__ bool await8(const double *p, int valid, double &v, int *err) {
+    const int q = threadIdx.x & 7;
+    unsigned long long b = q < valid ? kUnset : 0ull;
+    for (unsigned spin = 0;; ++spin) {
+        if (b == kUnset) asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(b) : "l"(p + q) : "memory");
+        if (__all_sync(0xffffffffu, b != kUnset)) break;
+        if (spin > kSpinLimit || ((spin & 63u) == 63u && *(volatile int *)err)) {
+            atomicCAS(err, 0, (int)OT_ERR_TIMEOUT);
+            return false;
+        }
+    }
+    v = __longlong_as_double((long long)b);
+    return true;
+}
+
+__global__ void __launch_bounds__(kST)
 dense_solve_kernel(int n, const double *__restrict__ A, const double *__restrict__ Linv,
-                   const double *__restrict__ D, const double *__restrict__ b, double *z, double *x,
-                   double *part /* gridDim x kB */, unsigned *bar, int *err) {
-    __shared__ double vb[kB];
-    __shared__ double red[kT / 32][32];
-    __shared__ double Ls[kB][kB + 1];      // inverse diagonal block (block 0 only)
-    const int lane = threadIdx.x & 31;
-    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t r = tid; r < n; r += stride) z[r] = b[r];
-    if (!grid_barrier(bar, gridDim.x, err)) return;
-    // ---- forward
-    for (int k = 0; k < n; k += kB) {
-        const int bs = min(kB, n - k);
-        if (blockIdx.x == 0) {
-            // z_blk = L11^-1 z_blk, the inverse block staged in shared memory
-            for (int q = threadIdx.x; q < kB * kB; q += blockDim.x) {
-                const int i = q % kB, c = q / kB;
-                Ls[c][i] = (i < bs && c < bs) ? Linv[(int64_t)c * n + (k + i)] : 0.0;
-            }
-            if (threadIdx.x < kB) vb[threadIdx.x] = threadIdx.x < bs ? z[k + threadIdx.x] : 0.0;
-            __syncthreads();
-            if (threadIdx.x < bs) {
-                const int i = threadIdx.x;
-                double t = 0;
-#pragma unroll 16
-                for (int c = 0; c < kB; ++c) t += Ls[c][i] * vb[c];
-                z[k + i] = t;
-            }
-            __syncthreads();
-        }
-        if (!grid_barrier(bar, gridDim.x, err)) return;
-        if (k + bs < n) {
-            if (threadIdx.x < kB) vb[threadIdx.x] = threadIdx.x < bs ? z[k + threadIdx.x] : 0.0;
-            __syncthreads();
-            for (int64_t r = k + bs + tid; r < n; r += stride) {
-                double acc = 0;
-                if (bs == kB) {
-#pragma unroll 16
-                    for (int l = 0; l < kB; ++l) acc += A[(int64_t)(k + l) * n + r] * vb[l];
-                } else {
-                    for (int l = 0; l < bs; ++l) acc += A[(int64_t)(k + l) * n + r] * vb[l];
-                }
-                z[r] -= acc;
-            }
-            __syncthreads();
-            if (!grid_barrier(bar, gridDim.x, err)) return;
-        }
+                   const double *__restrict__ D, const double *__restrict__ b, double *z, double *x, int *err) {
+    __shared__ double red[4][kB];
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, nb = (n + kB - 1) / kB;
+    const int i = (int)blockIdx.x, k = i * kB, bs = min(kB, n - k);
+    const bool live = lane < bs;
+    // the inverse block: row `lane`, columns 8 g .. (forward), column `lane`, rows 8 g .. (backward)
+    double Fi[8], Bi[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const int c = 8 * g + q;
+        Fi[q] = live && c < bs ? Linv[(int64_t)c * n + k + lane] : 0.0;
+        Bi[q] = live && c < bs ? Linv[(int64_t)lane * n + k + c] : 0.0;
     }
-    // ---- diagonal
-    for (int64_t r = tid; r < n; r += stride) x[r] = isinf(D[r]) ? 0.0 : z[r] / D[r];
-    if (!grid_barrier(bar, gridDim.x, err)) return;
-    // ---- backward: t = y_blk - L21^T x_rest, then x_blk = L11^-T t
-    for (int k = ((n - 1) / kB) * kB; k >= 0; k -= kB) {
-        const int bs = min(kB, n - k);
-        if (k + bs < n) {
-            for (int h = 0; h < bs; h += 32) {
-                const int hb = min(32, bs - h);
-                double acc[32];
+    const double bv = live ? b[k + lane] : 0.0, dv = live ? D[k + lane] : 1.0;
+    auto reduce = [&](double v) {   // the four warps' parts, in every warp
+        red[g][lane] = v;
+        __syncthreads();
+        const double s = (red[0][lane] + red[1][lane]) + (red[2][lane] + red[3][lane]);
+        __syncthreads();
+        return s;
+    };
+    bool ok = true;
+    // ---- forward: z_i = L_ii^-1 (b_i - sum_{j < i} L_ij z_j)
+    double acc = 0.0, cur[8], nxt[8];
 #pragma unroll
-                for (int j = 0; j < 32; ++j) acc[j] = 0.0;
-                for (int64_t r = k + bs + tid; r < n; r += stride) {
-                    const double xr = x[r];
+    for (int q = 0; q < 8; ++q) nxt[q] = live && i > 0 ? A[(int64_t)(8 * g + q) * n + k + lane] : 0.0;
+    for (int j = 0; j < i; ++j) {
 #pragma unroll
-                    for (int j = 0; j < 32; ++j)
-                        if (j < hb) acc[j] += A[(int64_t)(k + h + j) * n + r] * xr;
-                }
+        for (int q = 0; q < 8; ++q) cur[q] = nxt[q];
+        if (j + 1 < i)
 #pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const double v = warp_sum(acc[j]);
-                    if (lane == 0) red[threadIdx.x >> 5][j] = v;
-                }
-                __syncthreads();
-                if (threadIdx.x < hb) {
-                    double sum = 0;
-                    for (int w = 0; w < kT / 32; ++w) sum += red[w][threadIdx.x];
-                    part[(int64_t)blockIdx.x * kB + h + threadIdx.x] = sum;
-                }
-                __syncthreads();
-            }
-            if (!grid_barrier(bar, gridDim.x, err)) return;
-        }
-        if (blockIdx.x == 0) {
-            for (int q = threadIdx.x; q < kB * kB; q += blockDim.x) {
-                const int i = q % kB, c = q / kB;
-                Ls[c][i] = (i < bs && c < bs) ? Linv[(int64_t)c * n + (k + i)] : 0.0;
-            }
-            if (threadIdx.x < kB) {
-                double t = 0.0;
-                if (threadIdx.x < bs) {
-                    t = x[k + threadIdx.x];
-                    if (k + bs < n)
-                        for (unsigned g = 0; g < gridDim.x; ++g) t -= part[(int64_t)g * kB + threadIdx.x];
-                }
-                vb[threadIdx.x] = t;
-            }
-            __syncthreads();
-            if (threadIdx.x < bs) {
-                const int c = threadIdx.x;  // x_c = sum_i Linv(i, c) t_i   (L11^-T t)
-                double v = 0;
-#pragma unroll 16
-                for (int i = 0; i < kB; ++i) v += Ls[c][i] * vb[i];
-                x[k + c] = v;
-            }
-            __syncthreads();
-        }
-        if (!grid_barrier(bar, gridDim.x, err)) return;
+            for (int q = 0; q < 8; ++q) nxt[q] = live ? A[(int64_t)((j + 1) * kB + 8 * g + q) * n + k + lane] : 0.0;
+        double zv = 0.0;
+        ok = ok && await8(z + j * kB + 8 * g, 8, zv, err);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) acc = fma(cur[q], __shfl_sync(0xffffffffu, zv, q), acc);
     }
+    double t = bv - reduce(acc);
+    acc = 0.0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) acc = fma(Fi[q], __shfl_sync(0xffffffffu, t, 8 * g + q), acc);
+    t = reduce(acc);
+    if (__syncthreads_or(!ok)) return;
+    if (g == 0 && live) publish(z + k + lane, t);
+    // ---- backward: x_i = L_ii^-T (D_i^-1 z_i - sum_{j > i} L_ji^T x_j)
+    const double y = isinf(dv) ? 0.0 : t / dv;
+    acc = 0.0;
+    const double *Ai = A + (int64_t)(k + lane) * n;   // column k + lane
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const int r = (nb - 1) * kB + 8 * g + q;
+        nxt[q] = live && i < nb - 1 && r < n ? Ai[r] : 0.0;
+    }
+    for (int j = nb - 1; j > i; --j) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) cur[q] = nxt[q];
+        if (j - 1 > i)
+#pragma unroll
+            for (int q = 0; q < 8; ++q) nxt[q] = live ? Ai[(j - 1) * kB + 8 * g + q] : 0.0;
+        double xv = 0.0;
+        ok = ok && await8(x + j * kB + 8 * g, n - (j * kB + 8 * g), xv, err);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) acc = fma(cur[q], __shfl_sync(0xffffffffu, xv, q), acc);
+    }
+    t = y - reduce(acc);
+    acc = 0.0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) acc = fma(Bi[q], __shfl_sync(0xffffffffu, t, 8 * g + q), acc);
+    t = reduce(acc);
+    if (__syncthreads_or(!ok)) return;
+    if (g == 0 && live) publish(x + k + lane, t);
 }
 
 }  // namespace
@@ -290,36 +308,36 @@ Error dense_alloc(DenseLDL &M, int32_t n) {
     OT_CUDA(cudaMalloc((void **)&M.D, sizeof(double) * n));
     OT_CUDA(cudaMalloc((void **)&M.d0, sizeof(double) * n));
     OT_CUDA(cudaMalloc((void **)&M.z, sizeof(double) * n));
-    OT_CUDA(cudaMalloc((void **)&M.part, sizeof(double) * 4096 * kB));
-    OT_CUDA(cudaMalloc((void **)&M.bar, sizeof(unsigned) * 2));
     OT_CUDA(cudaMalloc((void **)&M.err, sizeof(int)));
     return ok();
 }
 
 void dense_free(DenseLDL &M) {
-    for (void *p : {(void *)M.A, (void *)M.LD, (void *)M.Linv, (void *)M.D, (void *)M.d0, (void *)M.z, (void *)M.part,
-                    (void *)M.bar, (void *)M.err})
+    for (void *p : {(void *)M.A, (void *)M.LD, (void *)M.Linv, (void *)M.D, (void *)M.d0, (void *)M.z, (void *)M.err})
         if (p) cudaFree(p);
     M = DenseLDL();
 }
 
 Error dense_factor(DenseLDL &M, const Chol &C, double eps, cudaStream_t st) {
     const int n = M.n;
+    int dev = 0, sms = 0;
+    OT_CUDA(cudaGetDevice(&dev));
+    OT_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     OT_CUDA(cudaMemsetAsync(M.A, 0, sizeof(double) * (size_t)n * n, st));
-    dense_scatter_kernel<<<gridd(n), kT, 0, st>>>(n, C.Ap, C.Aj, C.Ax, C.Adiag, M.A, M.d0);
+    dense_scatter_kernel<<<gridd(32LL * n), kT, 0, st>>>(n, C.Ap, C.Aj, C.Ax, C.Adiag, M.A, M.d0);
     OT_LAUNCHED();
     ktimer_begin(KT_LDL_NUMERIC, st);
     for (int k = 0; k < n; k += kB) {
-        const int bs = std::min(kB, n - k);
-        dense_diag_kernel<<<1, kT, 0, st>>>(n, k, bs, M.A, M.D, M.d0, eps, M.Linv);
+        const int bs = std::min(kB, n - k), rest = n - k - bs;
+        dense_panel_kernel<<<(unsigned)std::max<int64_t>(1, ceil_div(rest, 32)), kT, 0, st>>>(n, k, bs, M.A, M.D, M.d0,
+                                                                                             eps, M.LD);
         OT_LAUNCHED();
-        if (k + bs < n) {
-            dense_panel_kernel<<<(unsigned)ceil_div(n - k - bs, kT), kT, 0, st>>>(n, k, bs, M.A, M.D, M.LD);
-            OT_LAUNCHED();
-            const int t = (int)ceil_div(n - k - bs, 64);
-            dense_update_kernel<<<(unsigned)(t * (t + 1) / 2), kT, 0, st>>>(n, k, bs, M.A, M.LD);
-            OT_LAUNCHED();
-        }
+        const int64_t t = ceil_div(rest, 64), t2 = ceil_div(rest, 32);
+        if (t * (t + 1) / 2 >= 4LL * sms)
+            dense_update_kernel<64><<<(unsigned)(t * (t + 1) / 2 + 1), kT, 0, st>>>(n, k, bs, M.A, M.LD, M.Linv);
+        else
+            dense_update_kernel<32><<<(unsigned)(t2 * (t2 + 1) / 2 + 1), kT, 0, st>>>(n, k, bs, M.A, M.LD, M.Linv);
+        OT_LAUNCHED();
     }
     ktimer_end(KT_LDL_NUMERIC, st);
     ktimer_add_work(KT_LDL_NUMERIC, (double)n * n * n / 3.0);  // L D L^T: n^3/3 flops
@@ -327,21 +345,16 @@ Error dense_factor(DenseLDL &M, const Chol &C, double eps, cudaStream_t st) {
 }
 
 Error dense_solve(DenseLDL &M, const double *b, double *x, cudaStream_t st) {
-    int dev = 0, sms = 0, per_sm = 0;
-    OT_CUDA(cudaGetDevice(&dev));
-    OT_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    OT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, dense_solve_kernel, kT, 0));
-    int grid = std::max(1, std::min<int>(std::min(per_sm, 2) * sms, (int)ceil_div(M.n, kT)));
-    grid = std::min(grid, 4096);
-    OT_CUDA(cudaMemsetAsync(M.bar, 0, 2 * sizeof(unsigned), st));
     int n = M.n;
+    OT_CUDA(cudaMemsetAsync(M.z, 0xff, sizeof(double) * n, st));
+    OT_CUDA(cudaMemsetAsync(x, 0xff, sizeof(double) * n, st));
     const double *A = M.A, *Li = M.Linv, *D = M.D;
-    double *z = M.z, *part = M.part;
-    unsigned *bar = M.bar;
+    double *z = M.z;
     int *err = M.err;
-    void *args[] = {&n, &A, &Li, &D, &b, &z, &x, &part, &bar, &err};
+    void *args[] = {&n, &A, &Li, &D, &b, &z, &x, &err};
     ktimer_begin(KT_LDL_SOLVE, st);
-    OT_CUDA(cudaLaunchCooperativeKernel((void *)dense_solve_kernel, dim3(grid), dim3(kT), args, 0, st));
+    OT_CUDA(cudaLaunchCooperativeKernel((void *)dense_solve_kernel, dim3((unsigned)ceil_div(n, kB)), dim3(kST), args, 0,
+                                        st));
     OT_LAUNCHED();
     ktimer_end(KT_LDL_SOLVE, st);
     ktimer_add_work(KT_LDL_SOLVE, 8.0 * (double)n * n);  // reads L twice

@@ -1635,8 +1635,18 @@ static Error solve_direct(Newton &W, const Support &S, double tol, int max_cg, d
         // index (4) and a gathered vector entry (8) in each pass; per row the offset, M^-1 and w;
         // per column the offset, q, p twice and the step's reads of x, r and writes of x, r
         const double dcg_bytes = 40.0 * (double)S.psi + 20.0 * (double)W.m + 68.0 * (double)W.n;
-        auto issue = [&](int k) -> Error {
+        const bool ahead = C == nullptr;  // iterations queued ahead only where the preconditioner is cheap
+        auto direction = [&](int k) -> Error {   // z = M^-1 r and the direction after iteration k
             const int cur = (k & 1) ? SC_RZ1 : SC_RZ0, nxt = (k & 1) ? SC_RZ0 : SC_RZ1;
+            OT_TRY(precond(r, z));
+            dot_kernel<<<gn, kT, 0, st>>>(W.n, r, z, W.part, nxt);
+            OT_LAUNCHED();
+            dcg_dir2_kernel<<<gn, kT, 0, st>>>(W.n, (int)gn, (int)gn, W.scal, cur, nxt, z, p, W.part);
+            OT_LAUNCHED();
+            return ok();
+        };
+        auto issue = [&](int k) -> Error {
+            const int cur = (k & 1) ? SC_RZ1 : SC_RZ0;
             ktimer_begin(KT_DCG, st);
             if (G == 16) {
                 mvg_rows_kernel<16><<<gmr, kT, 0, st>>>(W.m, S.row_ptr, S.j, W.theta, W.Minv, p, W.w64);
@@ -1656,11 +1666,12 @@ static Error solve_direct(Newton &W, const Support &S, double tol, int max_cg, d
             OT_LAUNCHED();
             ktimer_end(KT_DCG, st);
             ktimer_add_work(KT_DCG, dcg_bytes);
-            OT_TRY(precond(r, z));
-            dot_kernel<<<gn, kT, 0, st>>>(W.n, r, z, W.part, nxt);
-            OT_LAUNCHED();
-            dcg_dir2_kernel<<<gn, kT, 0, st>>>(W.n, (int)gn, (int)gn, W.scal, cur, nxt, z, p, W.part);
-            OT_LAUNCHED();
+            if (!ahead) {   // r.r for the test, before the next preconditioner is paid for
+                Finish f{1, {SC_NORM_A}, {(int)gn}, {0}};
+                OT_TRY(finish(f, W, st));
+            } else {
+                OT_TRY(direction(k));
+            }
             OT_CUDA(cudaMemcpyAsync(W.hscal + (k & 1) * SC_COUNT, W.scal, sizeof(double) * SC_COUNT,
                                     cudaMemcpyDeviceToHost, st));
             OT_CUDA(cudaEventRecord(W.ev_scal2[k & 1], st));
@@ -1673,9 +1684,8 @@ static Error solve_direct(Newton &W, const Support &S, double tol, int max_cg, d
             OT_TRY(issue(0));
             issued = 1;
         }
-        const bool ahead = C == nullptr;  // only where the preconditioner is cheap
         while (it < issued) {
-            if (issued < cap && (ahead || issued == it)) {
+            if (issued < cap && ahead) {
                 OT_TRY(issue(issued));
                 ++issued;
             }
@@ -1691,6 +1701,11 @@ static Error solve_direct(Newton &W, const Support &S, double tol, int max_cg, d
             rr = h[SC_NORM_A];
             ++it;
             if (rr <= target * target * bb) break;
+            if (!ahead && it < cap) {
+                OT_TRY(direction(it - 1));
+                OT_TRY(issue(issued));
+                ++issued;
+            }
         }
         // an iteration still queued ahead completes before the copy below (stream order)
     }

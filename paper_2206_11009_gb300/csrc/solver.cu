@@ -585,8 +585,7 @@ Error do_step(ot_ipm *h, ot_iter_info *info) {
         if (n <= dense_max) {
             // moderate n: exact assembly and a dense blocked LDL^T (the exact factor is dense-ish)
             if (!h->dense.A) OT_TRY(dense_alloc(h->dense, n));
-            bool changed = false;
-            OT_TRY(chol_assemble(h->chol, W, S, 0.0, &changed, st));
+            OT_TRY(chol_assemble(h->chol, W, S, 0.0, nullptr, st));
             OT_CUDA(cudaMemsetAsync(h->dense.err, 0, sizeof(int), st));
             OT_TRY(dense_factor(h->dense, h->chol, kPivotEps, st));
             W.direct = &h->chol;
@@ -1561,8 +1560,7 @@ int ot_ipm_newton_direction(ot_ipm_t *h, int32_t solver, double cg_tol, int32_t 
         } else if (solver == OT_LS_DENSE64) {
             if (n > kDenseMaxN) return fail(OT_ERR_UNSUPPORTED, "FP64 dense factor: n above its limit");
             if (!h->dense.A) OT_TRY(dense_alloc(h->dense, n));
-            bool changed = false;
-            OT_TRY(chol_assemble(h->chol, W, S, 0.0, &changed, st));
+            OT_TRY(chol_assemble(h->chol, W, S, 0.0, nullptr, st));
             OT_CUDA(cudaMemsetAsync(h->dense.err, 0, sizeof(int), st));
             OT_TRY(dense_factor(h->dense, h->chol, kPivotEps, st));
             W.direct = &h->chol;
