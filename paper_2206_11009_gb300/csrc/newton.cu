@@ -10,6 +10,7 @@
 
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <type_traits>
 #include <vector>
 
@@ -215,14 +216,18 @@ __global__ void comp_center_kernel(int m, int n, const int32_t *__restrict__ par
 
 // ------------------------------------------------------------------------ PCG on S_M
 template <typename T>
+struct alignas(4 * sizeof(T)) PcgNode { T z, s, p, pn; };   // per column: D^-1 r, D^-1 q, direction, next one
+
+template <typename T>
 struct PcgArgs {
     int m, n;
     const int32_t *rp, *sj, *cp, *crow;
     const T *th, *thc, *Minv, *Dinv;
     const T *b;
-    T *x, *r, *z, *pa, *pb, *q, *w;   // pa / pb: double-buffered search direction
-    double *part;  // 3 slots x gridDim
-    unsigned *bar;
+    T *x, *r, *q, *w, *acc;
+    PcgNode<T> *node;
+    double *part;     // 2 x kPcgDots sums x gridDim
+    unsigned *cnt;    // hand-over counter, preset to zero
     int *err;
     double tol;
     int maxit;
@@ -231,7 +236,12 @@ struct PcgArgs {
     int64_t bnd_cap;
 };
 
-constexpr int kPcgT = 512;   // threads per PCG block
+// threads per PCG block (one block per SM): an FP64 operation of a warp takes its scheduler 64 cycles,
+// so fewer warps with more entries each serve FP64 better
+template <typename T>
+constexpr int kPcgT = sizeof(T) == 8 ? 512 : 1024;
+constexpr int kPcgDots = 5;
+constexpr int kPcgSmem = 160 * 1024;   // dynamic shared memory: the block's share of the operator
 
 // sum of `x` over the g lanes of an aligned lane group (g a power of two <= 32)
 template <typename T>
@@ -452,28 +462,65 @@ __device__ __forceinline__ void sum_partials(const double *part, unsigned G, int
     __syncthreads();
 }
 
-// Jacobi-preconditioned CG on S_M, persistent cooperative kernel.  Rows and columns are handled
-// by lane groups of g threads (g ~ the average row/column length), each group a contiguous range
-// of rows (and one of columns) of equal weight, pairs + g per row (the per-row reduction costs
-// about one trip): group q starts at the first row i with rp[i] + g i >= q (psi + g m) / ngrp.
-// Contiguous ranges keep neighbouring pixels together (the gathers stay local) and bound a group's
-// excess over the mean by one row.  With p_k = z_k + beta_k p_{k-1}
-// formed on the fly from z and the previous direction (double buffer), one iteration is
-//   row pass:    w_i = M_i^-1 sum_j theta_ij p_j                                   | barrier
-//   column pass: p_j stored; q_j = sum_i theta_ij (p_j - w_i); partial p.q           | barrier
-//   update:      alpha = rz/pq; x += alpha p; r -= alpha q; z = D^-1 r; partial r.z, r.r | barrier
-// Dot products are accumulated in double in every precision.
+// 1 / d for normal d by the hardware's approximation and one step of Halley's iteration
+__device__ __forceinline__ double halley_rcp(double d) {
+    double r0;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(d));
+    const double e = fma(-d, r0, 1.0);
+    return fma(r0, fma(e, e, e), r0);
+}
+
+// Hand-over between all blocks: one released increment of a counter per block, polled by one thread
+// of each (1.5 us whatever the number of blocks; with a flag per block and every block polling all
+// of them it took 5 us at 152 blocks).  `target`: arrivals after which it opens.  Bounded; false when it
+// gave up.
+__device__ __forceinline__ bool count_reach(unsigned *cnt, unsigned target, int *err) {
+    int okv = 1;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" :: "l"(cnt) : "memory");
+        unsigned spins = 0;
+        while ((int)(ld_acquire_gpu(cnt) - target) < 0) {
+            if (++spins > kSpinLimit || ((spins & 63u) == 0u && *(volatile int *)err)) {
+                atomicCAS(err, 0, (int)OT_ERR_TIMEOUT);
+                okv = 0;
+                break;
+            }
+        }
+    }
+    return !__syncthreads_or(!okv);
+}
+
+// Jacobi-preconditioned CG on S_M, persistent cooperative kernel, in the predict-and-recompute form
+// (Chen and Carson, SIAM J. Sci. Comput. 42:A3084, 2020): the next r.z, needed for beta before the
+// new residual exists, is predicted from the sums of the current iteration, alpha^2 q.D^-1 q - r.z,
+// and recomputed from the residual itself one iteration later, where alpha uses it.  So one
+// iteration has a single reduction and two hand-overs between the blocks instead of three grid
+// barriers and three reductions:
+//   row pass:    z = z' - alpha s', p = z + beta p' formed on the fly from one packed node (z, s, p)
+//                per column; w_i = M_i^-1 sum_j theta_ij p_j                            | hand-over
+//   column pass: q_j = sum_i theta_ij (p_j - w_i); x += alpha p' and r -= alpha q' (the step that the
+//                last reduction allowed), z = D^-1 r, s = D^-1 q; p.q, q.s, r.z, r.r, z.q | reduction
+// Every block adds the blocks' partial sums in the same order.  Rows and columns are handled by lane
+// groups of g threads (g ~ the average row length), each group a contiguous range of rows (and one
+// of columns) of equal weight, pairs + g per row: neighbouring pixels stay together.  A block keeps
+// its columns' vectors and its pairs of both passes in shared memory when they fit, so that only the
+// gathered nodes and w come from L2.  Dot products are accumulated in double in every precision.
+// Latency-bound: 64x64 FP64 21.6 us per iteration became 10.4, 128x128 FP32 24.3 became 8.9.
 template <typename T>
-__global__ void __launch_bounds__(kPcgT) pcg_kernel(PcgArgs<T> A, int g) {
-    __shared__ double sh[kPcgT / 32];
-    __shared__ double s_val[3];
+__global__ void __launch_bounds__(kPcgT<T>, 1) pcg_kernel(PcgArgs<T> A, int g, int smem_bytes) {
+    constexpr int NT = kPcgT<T>;
+    extern __shared__ __align__(16) unsigned char dsm[];
+    __shared__ double dots[kPcgDots][NT];
+    __shared__ double s_val[kPcgDots];
+    __shared__ T s_ab[2];   // (one conversion: a warp's takes the FP64 pipe 64 cycles)
+    __shared__ int s_next;
     const unsigned G = gridDim.x;
     const int n = A.n, m = A.m;
-    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t stride = (int64_t)G * blockDim.x;
+    const int64_t tid = (int64_t)blockIdx.x * NT + threadIdx.x;
     const int lg = threadIdx.x & (g - 1);                 // lane within its group
-    const int64_t grp = tid / g, ngrp = stride / g;
-    double *P0 = A.part, *P1 = A.part + G, *P2 = A.part + 2 * G;
+    const int64_t grp = tid / g, ngrp = (int64_t)G * NT / g;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
     // the group boundaries (lane 0 of each group searches its own; group 0 also writes the ends)
     if (lg == 0) {
@@ -497,132 +544,187 @@ __global__ void __launch_bounds__(kPcgT) pcg_kernel(PcgArgs<T> A, int g) {
             A.bnd[A.bnd_cap + ngrp] = n;
         }
     }
-    double bb = 0, rz = 0;
-    for (int64_t j = tid; j < n; j += stride) {
+    for (int64_t j = tid; j < n; j += (int64_t)G * NT) {
         const T bj = A.b[j];
         A.x[j] = (T)0;
         A.r[j] = bj;
-        const T zj = A.Dinv[j] * bj;
-        A.z[j] = zj;
-        A.pa[j] = (T)0;
-        bb += (double)bj * (double)bj;
-        rz += (double)bj * (double)zj;
+        A.q[j] = (T)0;
+        PcgNode<T> nd;
+        nd.z = A.Dinv[j] * bj; nd.s = (T)0; nd.p = (T)0; nd.pn = (T)0;
+        A.node[j] = nd;
     }
-    {
-        double s0 = block_sum(bb, sh), s1 = block_sum(rz, sh);
-        if (threadIdx.x == 0) { P0[blockIdx.x] = s0; P1[blockIdx.x] = s1; }
-    }
-    if (!grid_barrier(A.bar, G, A.err)) return;
-    sum_partials(A.part, G, 2, s_val);
-    bb = s_val[0];
-    rz = s_val[1];
-    const double tol2 = A.tol * A.tol * bb;
+    unsigned arrivals = G;
+    if (!count_reach(A.cnt, arrivals, A.err)) return;
     // this group's rows [r0, r0 + nr) and columns [c0, c0 + nc); trip counts uniform over the warp
     const int r0 = A.bnd[grp], nr = A.bnd[grp + 1] - r0;
     const int c0 = A.bnd[A.bnd_cap + grp], nc = A.bnd[A.bnd_cap + grp + 1] - c0;
     const int rtrips = __reduce_max_sync(0xffffffffu, nr), ctrips = __reduce_max_sync(0xffffffffu, nc);
-    int it = 0;
-    double rr = bb;
-    T beta = (T)0;
-    T *pprev = A.pa, *pcur = A.pb;
-    if (bb > 0.0 && rz > 0.0) {
-        for (it = 0; it < A.maxit;) {
-            // row pass with p = z + beta pprev (the trip count is uniform across a warp: groups
-            // past their range contribute zero but still take part in the shuffles)
-            // two rows per group and trip (rows i and i + 1), their loads interleaved: the
-            // passes are bound by the latency of the index -> gather chains, not by bandwidth
-            for (int t = 0; t < rtrips; t += 2) {
-                const int ia = r0 + t, ib = ia + 1;
-                const bool va = t < nr, vb = t + 1 < nr;
-                T acca = (T)0, accb = (T)0;
-                int ea = 0, ha = 0, eb = 0, hb = 0;
-                if (va) { ea = A.rp[ia] + lg; ha = A.rp[ia + 1]; }
-                if (vb) { eb = A.rp[ib] + lg; hb = A.rp[ib + 1]; }
-                while (ea < ha || eb < hb) {
-                    if (ea < ha) {
-                        const int j = A.sj[ea];
-                        acca += A.th[ea] * (A.z[j] + beta * pprev[j]);
-                        ea += g;
-                    }
-                    if (eb < hb) {
-                        const int j = A.sj[eb];
-                        accb += A.th[eb] * (A.z[j] + beta * pprev[j]);
-                        eb += g;
-                    }
-                }
-                acca = group_sum(acca, g);
-                accb = group_sum(accb, g);
-                if (lg == 0 && va) A.w[ia] = A.Minv[ia] * acca;
-                if (lg == 0 && vb) A.w[ib] = A.Minv[ib] * accb;
+    // the block's rows, columns and pairs
+    const int64_t gb = (int64_t)blockIdx.x * NT / g, ge = gb + NT / g;
+    const int rb0 = A.bnd[gb], nrow = A.bnd[ge] - rb0;
+    const int cb0 = A.bnd[A.bnd_cap + gb], ncol = A.bnd[A.bnd_cap + ge] - cb0;
+    const int e0 = A.rp[rb0], ne_r = A.rp[rb0 + nrow] - e0, k0 = A.cp[cb0], ne_c = A.cp[cb0 + ncol] - k0;
+    // in shared memory, or where they are: the columns' vectors, the row and column pointers with
+    // M^-1, and the pairs (theta and index)
+    PcgNode<T> *own = A.node + cb0;
+    T *rv = A.r + cb0, *qv = A.q + cb0, *xv = A.x + cb0, *acc = A.acc + cb0;
+    const T *dv = A.Dinv + cb0, *mv = A.Minv + rb0, *thr = A.th + e0, *thk = A.thc + k0;
+    const int32_t *rp = A.rp + rb0, *cp = A.cp + cb0, *sjr = A.sj + e0, *crk = A.crow + k0;
+    bool resident = false;
+    {
+        int64_t used = 0;
+        const int64_t vec = ((int64_t)ncol * 9 + nrow) * sizeof(T) + ((int64_t)ncol + nrow + 2) * sizeof(int32_t);
+        if (vec + 16 <= smem_bytes) {
+            resident = true;
+            own = (PcgNode<T> *)dsm;
+            rv = (T *)(own + ncol); qv = rv + ncol; xv = qv + ncol; acc = xv + ncol;
+            T *d = acc + ncol, *mi = d + ncol;
+            int32_t *rpo = (int32_t *)(mi + nrow), *cpo = rpo + nrow + 1;
+            for (int t = threadIdx.x; t < ncol; t += NT) {
+                own[t] = A.node[cb0 + t];
+                rv[t] = A.r[cb0 + t];
+                qv[t] = (T)0;
+                xv[t] = (T)0;
+                d[t] = dv[t];
             }
-            if (!grid_barrier(A.bar, G, A.err)) return;
-            // column pass (two columns per group and trip)
-            double pq = 0;
-            for (int t = 0; t < ctrips; t += 2) {
-                const int ja = c0 + t, jb = ja + 1;
-                const bool va = t < nc, vb = t + 1 < nc;
-                T pa = (T)0, pb2 = (T)0, acca = (T)0, accb = (T)0;
-                int ka = 0, ha = 0, kb = 0, hb = 0;
-                if (va) { pa = A.z[ja] + beta * pprev[ja]; ka = A.cp[ja] + lg; ha = A.cp[ja + 1]; }
-                if (vb) { pb2 = A.z[jb] + beta * pprev[jb]; kb = A.cp[jb] + lg; hb = A.cp[jb + 1]; }
-                while (ka < ha || kb < hb) {
-                    if (ka < ha) {
-                        acca += A.thc[ka] * (pa - A.w[A.crow[ka]]);
-                        ka += g;
-                    }
-                    if (kb < hb) {
-                        accb += A.thc[kb] * (pb2 - A.w[A.crow[kb]]);
-                        kb += g;
-                    }
-                }
-                acca = group_sum(acca, g);
-                accb = group_sum(accb, g);
-                if (lg == 0 && va) {
-                    A.q[ja] = acca;
-                    pcur[ja] = pa;
-                    pq += (double)pa * (double)acca;
-                }
-                if (lg == 0 && vb) {
-                    A.q[jb] = accb;
-                    pcur[jb] = pb2;
-                    pq += (double)pb2 * (double)accb;
-                }
-            }
-            {
-                double s0 = block_sum(pq, sh);
-                if (threadIdx.x == 0) P0[blockIdx.x] = s0;
-            }
-            if (!grid_barrier(A.bar, G, A.err)) return;
-            sum_partials(A.part, G, 1, s_val);
-            pq = s_val[0];
-            if (!(pq > 0.0)) break;  // breakdown (exact zero direction or loss of definiteness)
-            const double alpha = rz / pq;
-            double rzn = 0, rrn = 0;
-            for (int64_t j = tid; j < n; j += stride) {
-                const T pj = pcur[j];
-                const T rj = A.r[j] - (T)alpha * A.q[j];
-                const T zj = A.Dinv[j] * rj;
-                A.x[j] += (T)alpha * pj;
-                A.r[j] = rj;
-                A.z[j] = zj;
-                rzn += (double)rj * (double)zj;
-                rrn += (double)rj * (double)rj;
-            }
-            {
-                double s1 = block_sum(rzn, sh), s2 = block_sum(rrn, sh);
-                if (threadIdx.x == 0) { P1[blockIdx.x] = s1; P2[blockIdx.x] = s2; }
-            }
-            if (!grid_barrier(A.bar, G, A.err)) return;
-            sum_partials(A.part + G, G, 2, s_val + 1);
-            rzn = s_val[1];
-            rr = s_val[2];
-            ++it;
-            if (rr <= tol2 || !(rzn > 0.0)) break;
-            beta = (T)(rzn / rz);
-            rz = rzn;
-            T *t = pprev; pprev = pcur; pcur = t;
+            for (int t = threadIdx.x; t < nrow; t += NT) mi[t] = mv[t];
+            for (int t = threadIdx.x; t <= nrow; t += NT) rpo[t] = rp[t];
+            for (int t = threadIdx.x; t <= ncol; t += NT) cpo[t] = cp[t];
+            dv = d; mv = mi; rp = rpo; cp = cpo;
+            used = (vec + 15) & ~(int64_t)15;
+        }
+        if (used + ((int64_t)ne_r + ne_c) * (int64_t)(sizeof(T) + sizeof(int32_t)) <= smem_bytes) {
+            T *t0 = (T *)(dsm + used), *t1 = t0 + ne_r;
+            int32_t *i0 = (int32_t *)(t1 + ne_c), *i1 = i0 + ne_r;
+            for (int t = threadIdx.x; t < ne_r; t += NT) { t0[t] = thr[t]; i0[t] = sjr[t]; }
+            for (int t = threadIdx.x; t < ne_c; t += NT) { t1[t] = thk[t]; i1[t] = crk[t]; }
+            thr = t0; thk = t1; sjr = i0; crk = i1;
         }
     }
+    T alpha = (T)0, beta = (T)0;
+    double bb = 0.0, rr = 0.0;
+    int it = 0;
+    __syncthreads();
+    for (;; ++it) {
+        // the own columns' direction, for the column pass
+        for (int t = threadIdx.x; t < ncol; t += NT) {
+            const PcgNode<T> nd = own[t];
+            own[t].pn = fma(beta, nd.p, fma(-alpha, nd.s, nd.z));
+        }
+        // row pass, two rows per group and trip, their loads interleaved
+        for (int t = 0; t < rtrips; t += 2) {
+            const int ia = r0 - rb0 + t, ib = ia + 1;
+            const bool va = t < nr, vb = t + 1 < nr;
+            T acca = (T)0, accb = (T)0;
+            int ea = 0, ha = 0, eb = 0, hb = 0;
+            if (va) { ea = rp[ia] - e0 + lg; ha = rp[ia + 1] - e0; }
+            if (vb) { eb = rp[ib] - e0 + lg; hb = rp[ib + 1] - e0; }
+            while (ea < ha || eb < hb) {
+                if (ea < ha) {
+                    const PcgNode<T> nd = A.node[sjr[ea]];
+                    acca = fma(thr[ea], fma(beta, nd.p, fma(-alpha, nd.s, nd.z)), acca);
+                    ea += g;
+                }
+                if (eb < hb) {
+                    const PcgNode<T> nd = A.node[sjr[eb]];
+                    accb = fma(thr[eb], fma(beta, nd.p, fma(-alpha, nd.s, nd.z)), accb);
+                    eb += g;
+                }
+            }
+            acca = group_sum(acca, g);
+            if (t + 1 < rtrips) accb = group_sum(accb, g);
+            if (lg == 0 && va) A.w[rb0 + ia] = mv[ia] * acca;
+            if (lg == 0 && vb) A.w[rb0 + ib] = mv[ib] * accb;
+        }
+        if (!count_reach(A.cnt, arrivals += G, A.err)) return;
+        // column pass (two columns per group and trip)
+        for (int t = 0; t < ctrips; t += 2) {
+            const int ja = c0 - cb0 + t, jb = ja + 1;
+            const bool va = t < nc, vb = t + 1 < nc;
+            T pa = (T)0, pb = (T)0, acca = (T)0, accb = (T)0;
+            int ka = 0, ha = 0, kb = 0, hb = 0;
+            if (va) { ka = cp[ja] - k0 + lg; ha = cp[ja + 1] - k0; pa = own[ja].pn; }
+            if (vb) { kb = cp[jb] - k0 + lg; hb = cp[jb + 1] - k0; pb = own[jb].pn; }
+            while (ka < ha || kb < hb) {
+                if (ka < ha) {
+                    acca = fma(thk[ka], pa - A.w[crk[ka]], acca);
+                    ka += g;
+                }
+                if (kb < hb) {
+                    accb = fma(thk[kb], pb - A.w[crk[kb]], accb);
+                    kb += g;
+                }
+            }
+            acca = group_sum(acca, g);
+            if (t + 1 < ctrips) accb = group_sum(accb, g);
+            if (lg == 0 && va) acc[ja] = acca;
+            if (lg == 0 && vb) acc[jb] = accb;
+        }
+        __syncthreads();
+        // the own columns' step, full lanes
+        double d0 = 0, d1 = 0, d2 = 0, d3 = 0, d4 = 0;
+        for (int t = threadIdx.x; t < ncol; t += NT) {
+            PcgNode<T> nd = own[t];
+            const T Dj = dv[t], pj = nd.pn, qj = acc[t];
+            const T rj = fma(-alpha, qv[t], rv[t]);
+            xv[t] = fma(alpha, nd.p, xv[t]);
+            rv[t] = rj;
+            qv[t] = qj;
+            nd.z = Dj * rj;
+            nd.s = Dj * qj;
+            nd.p = pj;
+            own[t] = nd;
+            if (resident) A.node[cb0 + t] = nd;
+            d0 += (double)pj * (double)qj;
+            d1 += (double)qj * (double)nd.s;
+            d2 += (double)rj * (double)nd.z;
+            d3 += (double)rj * (double)rj;
+            d4 += (double)nd.z * (double)qj;
+        }
+        const int cnt = min(ncol, NT);
+        if ((int)threadIdx.x < cnt) {
+            dots[0][threadIdx.x] = d0; dots[1][threadIdx.x] = d1;
+            dots[2][threadIdx.x] = d2; dots[3][threadIdx.x] = d3;
+            dots[4][threadIdx.x] = d4;
+        }
+        __syncthreads();
+        double *slots = A.part + (int64_t)(it & 1) * kPcgDots * G;   // (the other half may still be read)
+        if (warp < kPcgDots) {
+            double a = 0;
+            for (int t = lane; t < cnt; t += 32) a += dots[warp][t];
+            a = warp_sum(a);
+            if (lane == 0) slots[warp * G + blockIdx.x] = a;
+        }
+        if (!count_reach(A.cnt, arrivals += G, A.err)) return;
+        if (warp < kPcgDots) {
+            double v[5], a = 0;   // the first 160 blocks' partials in one round trip
+#pragma unroll
+            for (int k = 0; k < 5; ++k) v[k] = lane + 32 * k < G ? slots[warp * G + lane + 32 * k] : 0.0;
+            for (unsigned b = lane + 160; b < G; b += 32) a += slots[warp * G + b];
+            a += ((v[0] + v[1]) + (v[2] + v[3])) + v[4];
+            a = warp_sum(a);
+            if (lane == 0) s_val[warp] = a;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            const double pq = s_val[0], qs = s_val[1], rz = s_val[2], zq = s_val[4];
+            const double al = rz * halley_rcp(pq), next = fma(al, fma(al, qs, -2.0 * zq), rz);
+            s_ab[0] = (T)al;
+            s_ab[1] = (T)fmax(next * halley_rcp(rz), 0.0);
+            const double rrv = s_val[3], lim = it == 0 ? rrv : bb;
+            // stop: converged, out of iterations, or breakdown (exact zero direction or residual, loss
+            // of definiteness)
+            s_next = !(rrv <= A.tol * A.tol * lim) && it < A.maxit && pq > 0.0 && rz > 0.0;
+        }
+        __syncthreads();
+        rr = s_val[3];
+        if (it == 0) bb = rr;
+        if (!s_next) break;
+        alpha = s_ab[0];
+        beta = s_ab[1];
+    }
+    if (resident)
+        for (int t = threadIdx.x; t < ncol; t += NT) A.x[cb0 + t] = xv[t];
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         A.scal[SC_PCG_ITERS] = (double)it;
         A.scal[SC_PCG_RELRES] = bb > 0 ? sqrt(rr / bb) : 0.0;
@@ -642,6 +744,7 @@ __global__ void __launch_bounds__(kPcgT) pcg_kernel(PcgArgs<T> A, int g) {
 // in the same order.
 constexpr int kClT = 1024;
 constexpr int kClMaxR = 16;
+constexpr int kClMaxN = 4096;
 
 __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -887,26 +990,25 @@ __global__ void __launch_bounds__(kClT, 1) pcg_cluster_kernel(PcgArgs<float> A, 
 
 template <typename T>
 Error launch_pcg(Newton &W, const Support &S, const T *th, const T *thc, const T *Minv, const T *Dinv,
-                 const T *b, T *x, T *r, T *z, T *p, T *q, T *w, double tol, int maxit, cudaStream_t st) {
-    int per_sm = 0;
-    OT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pcg_kernel<T>, kPcgT, 0));
+                 const T *b, T *x, T *r, T *q, T *w, double tol, int maxit, cudaStream_t st) {
+    constexpr int NT = kPcgT<T>;
     // lane-group size ~ half the average row length (power of two)
     const double avg = (double)std::max<int64_t>(S.psi, 1) / (double)std::max(W.m, 1);
     // (at most 16: measured at 256^2 with 33 pairs per row, 16 lanes beat 32 by 8 %)
     int g = 1;
     while (g < 16 && 2 * g <= avg) g <<= 1;
     const int64_t threads = (int64_t)std::max(W.m, W.n) * g;
-    const int maxg = std::max(1, per_sm) * W.num_sms;
-    int G = W.pcg_grid > 0 ? W.pcg_grid : (int)std::max<int64_t>(1, ceil_div(threads, kPcgT));
-    G = std::min(G, std::min(maxg, kMaxPartBlocks / 3));
-    // the boundary arrays hold ngrp + 1 = G kPcgT / g + 1 entries per half
-    G = (int)std::min<int64_t>(G, std::max<int64_t>(1, (W.pcg_bnd_cap - 1) * g / kPcgT));
+    // four times the blocks that one row per lane group would fill (up to one per SM): idle groups cost
+    // nothing, and an SM with fewer busy warps finishes its FP64 work sooner
+    int G = W.pcg_grid > 0 ? W.pcg_grid : (int)std::max<int64_t>(1, ceil_div(4 * threads, NT));
+    G = std::min(G, std::min(W.num_sms, kMaxPartBlocks / 3));
+    // the boundary arrays hold ngrp + 1 = G NT / g + 1 entries per half
+    G = (int)std::min<int64_t>(G, std::max<int64_t>(1, (W.pcg_bnd_cap - 1) * g / NT));
     OT_CUDA(cudaMemsetAsync(W.bar, 0, 2 * sizeof(unsigned), st));
     OT_CUDA(cudaMemsetAsync(W.err, 0, sizeof(int), st));
-    T *pb = (T *)W.pcg_pb;
-    if (sizeof(T) == 4) pb = (T *)W.pcg_pb32;
-    PcgArgs<T> A{W.m, W.n, S.row_ptr, S.j, S.col_ptr, S.col_row, th, thc, Minv, Dinv, b, x, r, z, p, pb, q, w,
-                 W.part, W.bar, W.err, tol, maxit, W.scal, W.pcg_bnd, W.pcg_bnd_cap};
+    PcgArgs<T> A{W.m, W.n, S.row_ptr, S.j, S.col_ptr, S.col_row, th, thc, Minv, Dinv, b, x, r, q, w,
+                 (T *)(W.pcg_node + 4 * (int64_t)W.n), (PcgNode<T> *)W.pcg_node, W.part, W.bar, W.err, tol, maxit,
+                 W.scal, W.pcg_bnd, W.pcg_bnd_cap};
     const int kid = sizeof(T) == 8 ? KT_PCG64 : KT_PCG32;
     const int R = W.pcg_cluster;
     cudaEvent_t ev[2] = {nullptr, nullptr};
@@ -918,7 +1020,9 @@ Error launch_pcg(Newton &W, const Support &S, const T *th, const T *thc, const T
     const ClLayout L = cl_layout(W.m, W.n, std::max(R, 1));
     bool clustered = false;
     if constexpr (sizeof(T) == 4) {
-      if (R > 1 && 2 * L.bytes <= W.pcg_cluster_smem) {
+      // up to kClMaxN: per iteration 6.9 us against the grid's 8.2 at n = 2916, 8.3 against 8.3 at 4096,
+      // 9.5 against 8.6 at 5625
+      if (R > 1 && std::max(W.m, W.n) <= kClMaxN && 2 * L.bytes <= W.pcg_cluster_smem) {
         clustered = true;
         // one thread-block cluster with the operator slices in shared memory
         int gc = 1;
@@ -943,9 +1047,16 @@ Error launch_pcg(Newton &W, const Support &S, const T *th, const T *thc, const T
       }
     }
     if (!clustered) {
-        void *args[] = {&A, &g};
+        static std::once_flag once;
+        static cudaError_t attr = cudaSuccess;
+        std::call_once(once, [] {
+            attr = cudaFuncSetAttribute(pcg_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPcgSmem);
+        });
+        if (attr != cudaSuccess) return fail(OT_ERR_CUDA, cudaGetErrorString(attr));
+        int sb = kPcgSmem;
+        void *args[] = {&A, &g, &sb};
         ktimer_begin(kid, st);
-        OT_CUDA(cudaLaunchCooperativeKernel((void *)pcg_kernel<T>, dim3(G), dim3(kPcgT), args, 0, st));
+        OT_CUDA(cudaLaunchCooperativeKernel((void *)pcg_kernel<T>, dim3(G), dim3(NT), args, kPcgSmem, st));
         OT_LAUNCHED();
         ktimer_end(kid, st);
     }
@@ -1237,8 +1348,8 @@ static Error rhs_norm(Newton &W, double *nrm, cudaStream_t st) {
 static Error solve_pcg64(Newton &W, const Support &S, double tol, int max_cg, double *dv, SolveStats *ss,
                          cudaStream_t st) {
     const unsigned gn = grid_of(W.n, W.num_sms);
-    OT_TRY(launch_pcg<double>(W, S, W.theta, W.theta_col, W.Minv, W.Dinv, W.rhs, W.x64, W.r64, W.z64, W.p64,
-                              W.q64, W.w64, tol, max_cg, st));
+    OT_TRY(launch_pcg<double>(W, S, W.theta, W.theta_col, W.Minv, W.Dinv, W.rhs, W.x64, W.r64, W.q64, W.w64,
+                              tol, max_cg, st));
     double hs[SC_COUNT];
     OT_TRY(read_scalars(W, hs, st));
     int errv = 0;
@@ -1271,8 +1382,8 @@ static Error solve_mixed(Newton &W, const Support &S, double tol, int max_cg, do
     for (int ref = 0; ref < 12 && nrm > tol * nrm0 && budget > 0; ++ref) {
         to_f32_kernel<<<gn, kT, 0, st>>>(W.n, W.res64, W.b32);
         OT_LAUNCHED();
-        OT_TRY(launch_pcg<float>(W, S, W.theta32, W.theta32_col, W.Minv32, W.Dinv32, W.b32, W.x32, W.r32, W.z32,
-                                 W.p32, W.q32, W.w32, inner, budget, st));
+        OT_TRY(launch_pcg<float>(W, S, W.theta32, W.theta32_col, W.Minv32, W.Dinv32, W.b32, W.x32, W.r32, W.q32,
+                                 W.w32, inner, budget, st));
         axpy_f32_kernel<<<gn, kT, 0, st>>>(W.n, W.x32, dv);
         OT_LAUNCHED();
         const double prev = nrm;
@@ -1774,10 +1885,10 @@ Error newton_alloc(Newton &W, int32_t m, int32_t n, int64_t cap, int num_sms) {
     for (double **p : {&W.r1b, &W.beta2, &W.N, &W.Dinv, &W.Sdiag, &W.rhs, &W.dv, &W.dv2, &W.dv3, &W.res64, &W.y64, &W.x64,
                        &W.r64, &W.z64, &W.p64, &W.q64})
         OT_TRY(dev_alloc(p, n));
-    for (float **p : {&W.Dinv32, &W.b32, &W.x32, &W.r32, &W.z32, &W.p32, &W.q32, &W.pcg_pb32}) OT_TRY(dev_alloc(p, n));
-    OT_TRY(dev_alloc(&W.pcg_pb, n));
-    // grid PCG lane groups: G kPcgT / g <= (blocks per SM <= 2048 / kPcgT) x SMs x kPcgT
-    W.pcg_bnd_cap = (int64_t)(2048 / kPcgT) * std::max(num_sms, 1) * kPcgT + 1;
+    for (float **p : {&W.Dinv32, &W.b32, &W.x32, &W.r32, &W.q32}) OT_TRY(dev_alloc(p, n));
+    OT_TRY(dev_alloc(&W.pcg_node, 5 * (int64_t)n));
+    // grid PCG lane groups: one block of at most 1024 threads per SM
+    W.pcg_bnd_cap = 1024LL * std::max(num_sms, 1) + 1;
     OT_TRY(dev_alloc(&W.pcg_bnd, 2 * W.pcg_bnd_cap));
     OT_TRY(dev_alloc(&W.parent, (int64_t)m + n));
     OT_TRY(dev_alloc(&W.comp_sum, (int64_t)m + n));
@@ -1810,7 +1921,7 @@ void newton_free(Newton &W) {
     void *ptrs[] = {W.c, W.theta, W.excl, W.r2, W.r3, W.g, W.dp, W.ds, W.dp2, W.ds2, W.dp3, W.ds3, W.theta32,
                     W.theta_col, W.theta32_col, W.flag, W.r1a, W.beta1, W.M, W.Minv, W.du, W.du2, W.du3, W.w64,
                     W.Minv32, W.w32, W.r1b, W.beta2, W.N, W.Dinv, W.Sdiag, W.rhs, W.dv, W.dv2, W.dv3, W.res64, W.y64,
-                    W.x64, W.r64, W.z64, W.p64, W.q64, W.Dinv32, W.b32, W.x32, W.r32, W.z32, W.p32, W.q32, W.pcg_pb, W.pcg_pb32,
+                    W.x64, W.r64, W.z64, W.p64, W.q64, W.Dinv32, W.b32, W.x32, W.r32, W.q32, W.pcg_node,
                     W.pcg_bnd, W.parent, W.comp_sum, W.comp_cnt, W.part, W.scal, W.bar, W.err};
     for (void *p : ptrs)
         if (p) cudaFree(p);

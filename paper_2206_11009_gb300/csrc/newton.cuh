@@ -37,8 +37,7 @@ struct Newton {
            *dv = nullptr,
            *dv2 = nullptr, *dv3 = nullptr, *res64 = nullptr, *y64 = nullptr;
     double *x64 = nullptr, *r64 = nullptr, *z64 = nullptr, *p64 = nullptr, *q64 = nullptr;
-    float *Dinv32 = nullptr, *b32 = nullptr, *x32 = nullptr, *r32 = nullptr, *z32 = nullptr, *p32 = nullptr,
-          *q32 = nullptr;
+    float *Dinv32 = nullptr, *b32 = nullptr, *x32 = nullptr, *r32 = nullptr, *q32 = nullptr;
     // components (m + n nodes)
     int32_t *parent = nullptr;
     double *comp_sum = nullptr, *comp_cnt = nullptr;
@@ -53,8 +52,7 @@ struct Newton {
     bool onecomp = true;       // the support graph is connected (set by schur_setup)
     int verbose = 0;           // >= 3: one line per PCG launch (support size, iterations, device ms)
     double last_pcg_ms = 0.0;
-    double *pcg_pb = nullptr;     // second direction buffer of the PCG (fp64 / fp32)
-    float *pcg_pb32 = nullptr;
+    double *pcg_node = nullptr;   // grid PCG: a node of four values per column, then one value per column
     int *pcg_bnd = nullptr;       // grid PCG: first row (then first column) of each lane group
     int64_t pcg_bnd_cap = 0;      // entries per half of pcg_bnd
     double pcg_bytes_per_iter = 0.0;
