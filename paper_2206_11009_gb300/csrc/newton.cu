@@ -1567,6 +1567,7 @@ __global__ void __launch_bounds__(kCgT) d32_cg_kernel(D32CgArgs A) {
     int it = 0;
     bool extra = false;
     double rr_test = rr;
+    const double rz0 = rz;
     if (bb > 0.0 && rz > 0.0 && A.maxit > 0) {
         for (;;) {
             // the new direction p must be complete before the row pass gathers it
@@ -1634,6 +1635,9 @@ __global__ void __launch_bounds__(kCgT) d32_cg_kernel(D32CgArgs A) {
             if (!grid_barrier(A.bar, G, A.err)) return;
             sum_partials(A.red + G, G, 1, s_val + 1);
             rzn = s_val[1];
+            // what is left of r when its preconditioned norm has fallen that far lies in the null space
+            // of S_M (rounding of the mean, about 1e-12 of b from n = 9216 on): no iteration reduces it
+            if (rzn <= A.target2 * rz0) extra = true;
             const double beta = (rz > 0.0 && rzn > 0.0) ? rzn / rz : 0.0;
             for (int64_t j = tid; j < n; j += stride) A.p[j] = A.z[j] + beta * A.p[j];
             rz = rzn;
