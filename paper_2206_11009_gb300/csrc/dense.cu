@@ -165,13 +165,16 @@ dense_update_kernel(int n, int k, int bs, double *__restrict__ A, const double *
         Rs[l][rr] = c0 + rr < n ? A[(int64_t)(k + l) * n + c0 + rr] : 0.0;
     }
     const int tr = (threadIdx.x % 16) * Q, tc = (threadIdx.x / 16) * Q;
-    double acc[Q][Q];
+    // the products are summed by themselves and subtracted once (an accumulator started from A would
+    // round every term at A's magnitude)
+    double acc[Q][Q], old[Q][Q];
 #pragma unroll
     for (int w = 0; w < Q; ++w)
 #pragma unroll
         for (int u = 0; u < Q; ++u) {
             const int r = r0 + tr + u, c = c0 + tc + w;
-            acc[u][w] = r < n && c < n && r >= c ? A[(int64_t)c * n + r] : 0.0;
+            acc[u][w] = 0.0;
+            old[u][w] = r < n && c < n && r >= c ? A[(int64_t)c * n + r] : 0.0;
         }
     __syncthreads();
     for (int l = 0; l < kB; ++l) {   // (a panel with rows below it is full)
@@ -181,14 +184,14 @@ dense_update_kernel(int n, int k, int bs, double *__restrict__ A, const double *
 #pragma unroll
         for (int u = 0; u < Q; ++u)
 #pragma unroll
-            for (int w = 0; w < Q; ++w) acc[u][w] = fma(-a[u], b[w], acc[u][w]);
+            for (int w = 0; w < Q; ++w) acc[u][w] = fma(a[u], b[w], acc[u][w]);
     }
 #pragma unroll
     for (int w = 0; w < Q; ++w)
 #pragma unroll
         for (int u = 0; u < Q; ++u) {
             const int r = r0 + tr + u, c = c0 + tc + w;
-            if (r < n && c < n && r >= c) A[(int64_t)c * n + r] = acc[u][w];
+            if (r < n && c < n && r >= c) A[(int64_t)c * n + r] = old[u][w] - acc[u][w];
         }
 }
 
