@@ -1,7 +1,7 @@
 // Helpers for the fifth-generation tensor-core kernels (tcgen05 MMAs reading operands from shared
 // memory, accumulators in tensor memory, completion on mbarriers).
 //
-// Operand layout used by every caller: K-major, no swizzle, built from core matrices of 8 rows x
+// Operand layout used by every caller: no swizzle, K-major unless said, core matrices of 8 rows x
 // 16 bytes (4 TF32 or 8 BF16 values along K).  The shared-memory matrix descriptor carries the
 // start address, the leading byte offset (between core matrices adjacent along K) and the stride
 // byte offset (between core matrices adjacent along M or N, here always 128: the 8-row groups are
@@ -21,6 +21,17 @@ __device__ __forceinline__ uint64_t tc_desc(uint32_t addr, uint32_t lbo) {
     uint64_t d = (uint64_t)((addr >> 4) & 0x3FFFu);
     d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
     d |= (uint64_t)((128u >> 4) & 0x3FFFu) << 32;
+    d |= (uint64_t)1 << 46;
+    return d;
+}
+
+// the same with both offsets given.  Operands read MN-major (bits 15 / 16 of the instruction descriptor)
+// have core matrices of 8 depths x 16 bytes along M or N: lbo is the offset between core matrices
+// adjacent along K, sbo between those adjacent along M or N.
+__device__ __forceinline__ uint64_t tc_desc2(uint32_t addr, uint32_t lbo, uint32_t sbo) {
+    uint64_t d = (uint64_t)((addr >> 4) & 0x3FFFu);
+    d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
+    d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
     d |= (uint64_t)1 << 46;
     return d;
 }
@@ -101,6 +112,17 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, float (&out)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int j = 0; j < 32; ++j) out[j] = __uint_as_float(v[j]);
+}
+
+// the same for 8 columns
+__device__ __forceinline__ void tc_ld8(uint32_t taddr, float (&out)[8]) {
+    uint32_t v[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                 : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int j = 0; j < 8; ++j) out[j] = __uint_as_float(v[j]);
 }
 
 }  // namespace ot
