@@ -154,12 +154,12 @@ typedef struct {
      * (Section 4.3) is unchanged. */
     int32_t precond;
     double ic_tau;
-    /* Bulk update of the FP32 dense factorisation: 1 = on the tensor cores (tcgen05 MMAs in split
-     * TF32, a = a_hi + a_lo, three products per term, FP32 accumulation in tensor memory: FP32
-     * accuracy; operands pre-split per panel, fetched by bulk copies; persistent warp-specialised
-     * CTAs with two accumulators), -1 = the FP32 SIMT update with the fused panel step, 0 = the
-     * tensor cores from n = 8192 on, SIMT below (the default; measured per factorisation:
-     * n = 16384 75 ms against 93 ms, n = 4096 2.9 ms either way). */
+    /* Rest-update of the FP32 dense factorisation: 1 = on the tensor cores (tcgen05 MMAs, each FP32
+     * operand as three BF16 pieces, six products per term, FP32 accumulation in tensor memory;
+     * operands pre-split, two panels per pass, fetched by bulk copies; persistent warp-specialised
+     * CTAs with two pairs of accumulators), -1 = the FP32 SIMT update, 0 = the tensor cores from
+     * n = 8192 on, SIMT below, where it is the more accurate by a factor of 2.5 (the default; per
+     * factorisation: n = 16384 34 ms against 95 ms, n = 8281 7.4 against 15.6, n = 4096 2.4 against 2.9). */
     int32_t tc_update;
     /* Relative residual at which the CG preconditioned by a factorisation (the FP32 dense factor,
      * the direct branch) stops: 0 = min(CG tolerance, 1e-10) (near-exact Newton directions);

@@ -15,6 +15,8 @@
 #include "primitives.cuh"
 #include "tc05.cuh"
 
+#include <cuda_bf16.h>
+
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -110,12 +112,12 @@ d32_colsum_kernel(int n, int ld, int bs, const float *__restrict__ A, float *__r
 // micro-panel with its 64 rows in registers (lane q: rows q and q+32; shuffles only): each pivot
 // is minus the sum of the column's remaining entries plus its below-block sum (np fixed-order
 // partials in csum[p * kP + l]), kept as sums of same-sign terms by a recurrence over the
-// micro-panel's own 8 x 8 block (the warp-wide sums are taken once per micro-panel).  Then all warps apply the micro-panel's rank-8 update to the rest of
-// the block (two barriers per micro-panel instead of one per column).  Columns stay unscaled until
-// the end (l_ij = S_ij / d_j).  The inverse of the unit block is formed afterwards by 8x8 block
-// rows: X_II = L_II^-1 by warp 0, X_IJ = -X_II sum_K L_IK X_KJ by all threads.
+// micro-panel's own 8 x 8 block (the warp-wide sums are taken once per micro-panel).  Meanwhile the
+// other warps apply the micro-panel before's rank-8 update to the rest of the block (one barrier per
+// micro-panel) and carry the inverse of the unit block on.  Columns stay unscaled in shared memory
+// (l_ij = S_ij / d_j on the way out).
 constexpr int kMp = 8;   // micro-panel width
-static_assert(kTT / 32 == kP / kMp && kTT == 4 * kP, "one warp per 8x8 diagonal block, 8b threads per b-pair");
+static_assert(kTT == 4 * kP, "warp 0, three threads per column, one warp");
 
 // Warp 0's elimination of one micro-panel (columns c0 .. c0 + nc - 1) with the block's 64 rows in
 // registers (lane q: rows q and q + 32).  prev >= 0: the micro-panel's columns first receive the
@@ -253,17 +255,17 @@ __device__ __forceinline__ void d32_micro_panel(int lane, int k, int c0, int nc,
 struct DiagSmem {
     float (*S)[kP + 1];
     float (*Xs)[kP + 1];
-    float (*Ts)[kP / 2 + 1];
+    float (*red)[kP];
     float *g, *thr, *ids;
 };
-constexpr int kDiagSmem = (2 * kP * (kP + 1) + (kP / 2) * (kP / 2 + 1) + 3 * kP) * 4;
+constexpr int kDiagSmem = (2 * kP * (kP + 1) + 4 * kP + 3 * kP) * 4;
 
 __device__ __forceinline__ DiagSmem diag_smem(float *buf) {
     DiagSmem m;
     m.S = (float (*)[kP + 1])buf;
     m.Xs = (float (*)[kP + 1])(buf + kP * (kP + 1));
-    m.Ts = (float (*)[kP / 2 + 1])(buf + 2 * kP * (kP + 1));
-    m.g = buf + 2 * kP * (kP + 1) + (kP / 2) * (kP / 2 + 1);
+    m.red = (float (*)[kP])(buf + 2 * kP * (kP + 1));
+    m.g = buf + 2 * kP * (kP + 1) + 4 * kP;
     m.thr = m.g + kP;
     m.ids = m.thr + kP;
     return m;
@@ -278,7 +280,6 @@ __device__ __forceinline__ void d32_diag_block(const DiagSmem &m, int ld, int k,
                                                float *__restrict__ Linv) {
     float (*S)[kP + 1] = m.S;
     float (*Xs)[kP + 1] = m.Xs;
-    float (*Ts)[kP / 2 + 1] = m.Ts;
     float *g = m.g, *thr = m.thr, *ids = m.ids;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // every global load of the block, of the first kP rows of partial sums and of the diagonal
@@ -310,38 +311,41 @@ __device__ __forceinline__ void d32_diag_block(const DiagSmem &m, int ld, int k,
         Xs[t / kP][t % kP] = cv[q];
     }
     __syncthreads();
-    // each column's partials: four threads take every fourth row, then one adds the four in order
-    // (further chunks of kP rows, for n above 4096, the same way)
+    // each column's partials: four threads take every fourth row (those beyond kP, for n above 4096,
+    // straight from memory), then one adds the four in order
     float gs = 0.f;
     {
         const int c = threadIdx.x % kP, h = threadIdx.x / kP;
         float part = 0.f;
         for (int q = h; q < nq0; q += kTT / kP) part += Xs[q][c];
-        float *red = &Ts[0][0];   // free until the block inverse: [4][kP] here
-        red[h * kP + c] = part;
-        __syncthreads();
-        if (threadIdx.x < kP && (int)threadIdx.x < bs) gs = red[c] + red[kP + c] + red[2 * kP + c] + red[3 * kP + c];
-    }
-    for (int q0 = kP; q0 < np; q0 += kP) {
-        const int nq = min(kP, np - q0);
-        for (int t = threadIdx.x; t < nq * kP; t += blockDim.x) {
-            const int row = q0 + t / kP, col = t % kP;
-            float v = __ldcg(csum + (size_t)(row * per) * kP + col);
-            if (per == 2) v += __ldcg(csum + (size_t)(row * per + 1) * kP + col);
-            Xs[t / kP][col] = v;
+#pragma unroll 16
+        for (int q = kP + h; q < np; q += kTT / kP) {
+            float v = __ldcg(csum + (size_t)(q * per) * kP + c);
+            if (per == 2) v += __ldcg(csum + (size_t)(q * per + 1) * kP + c);
+            part += v;
         }
+        m.red[h][c] = part;
         __syncthreads();
-        if (threadIdx.x < kP && threadIdx.x < bs)
-            for (int q = 0; q < nq; ++q) gs += Xs[q][threadIdx.x];
-        __syncthreads();
+        if ((int)threadIdx.x < bs) gs = m.red[0][c] + m.red[1][c] + m.red[2][c] + m.red[3][c];
     }
     if (threadIdx.x < kP) {
         g[threadIdx.x] = gs;
         thr[threadIdx.x] = eps * d0v;
+        ids[threadIdx.x] = 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+        const int t = (int)threadIdx.x + q * kTT;
+        Xs[t / kP][t % kP] = t / kP == t % kP ? 1.f : 0.f;
     }
     __syncthreads();
     // micro-panel 0, then per step: warp 0 updates and eliminates the next micro-panel while the
-    // other warps apply the current one's rank-8 update to the columns after it
+    // other warps apply the current one's rank-8 update to the columns after it, carry the inverse X =
+    // L^-1 on by its 8 rows, and write those and the micro-panel's columns of L out.  X starts as the
+    // identity: X_I = L_II^-1 X_I (a thread per column, the 8 values in registers), then X_r -= L_rI X_I
+    // for the rows r below.  L <= 0 below the diagonal and X >= 0, so every sum has terms of one sign.
+    // Done after the elimination (scaling, then an inverse by recursive doubling) this made a factorisation
+    // of n = 1024 take 550 us instead of 519; warp 0's chain hides most but not all of it.
     if (warp == 0) {
         if (bs >= kMp) d32_micro_panel<true>(lane, k, 0, kMp, -1, S, g, thr, ids, D);
         else d32_micro_panel<false>(lane, k, 0, bs, -1, S, g, thr, ids, D);
@@ -390,68 +394,47 @@ __device__ __forceinline__ void d32_diag_block(const DiagSmem &m, int ld, int k,
                     if (lb < bs) g[lb] -= gb;
                 }
             }
+            if (warp == kTT / 32 - 1) {
+                // L = S D^-1 (grounded columns are zero) of this micro-panel, back to A
+#pragma unroll
+                for (int q = 0; q < kMp; ++q) {
+                    const int j = c0 + q;
+                    const float id = ids[j];
+#pragma unroll
+                    for (int i = lane; i < kP; i += 32)
+                        if (i > j && i < bs) A[(size_t)(k + j) * ld + (k + i)] = S[i][j] * id;
+                }
+            } else {
+                const int c = (int)(threadIdx.x - 32) % kP, part = (int)(threadIdx.x - 32) / kP;   // 3 threads per column
+                float x[kMp], xd[kMp];   // X_I, D^-1 X_I
+#pragma unroll
+                for (int q = 0; q < kMp; ++q) x[q] = Xs[c0 + q][c];
+#pragma unroll
+                for (int q = 0; q < kMp; ++q) {
+#pragma unroll
+                    for (int e = 0; e < q; ++e) x[q] -= S[c0 + q][c0 + e] * xd[e];
+                    xd[q] = x[q] * ids[c0 + q];
+                }
+                if (part == 0 && c < bs) {
+#pragma unroll
+                    for (int q = 0; q < kMp; ++q)
+                        if (c0 + q < bs) Linv[(size_t)c * ld + (k + c0 + q)] = x[q];
+                }
+                if (c < c1) {
+#pragma unroll 4
+                    for (int r = c1 + part; r < bs; r += 3) {
+                        float v = S[r][c0] * xd[0], w = S[r][c0 + 1] * xd[1];
+#pragma unroll
+                        for (int q = 2; q < kMp; q += 2) {
+                            v += S[r][c0 + q] * xd[q];
+                            w += S[r][c0 + q + 1] * xd[q + 1];
+                        }
+                        Xs[r][c] -= v + w;
+                    }
+                }
+            }
         }
         __syncthreads();
-    }
-    // scale the columns: L = S D^-1 (grounded columns are zero); back to A
-    for (int t = threadIdx.x; t < kP * kP; t += blockDim.x) {
-        const int i = t % kP, j = t / kP;
-        const float l = (i > j && i < bs) ? S[i][j] * ids[j] : 0.f;
-        S[i][j] = l;
-        Xs[i][j] = 0.f;
-        if (i > j && i < bs) A[(size_t)(k + j) * ld + (k + i)] = l;
-    }
-    __syncthreads();
-    // X = L^-1 by recursive doubling.  Level 0: warp w inverts the diagonal 8x8 block w (lane c:
-    // column c by forward substitution).  Level b = 8, 16, 32: for each pair of b-blocks on the
-    // diagonal, X21 = -X22 (L21 X11), the product staged through Ts.  L <= 0 below the diagonal
-    // and X >= 0, so every sum has terms of one sign.  Rows and columns >= bs hold the identity.
-    if (lane < kMp) {
-        const int o = warp * kMp;
-        float x[kMp];
-#pragma unroll
-        for (int r = 0; r < kMp; ++r) {
-            float v = (r == lane) ? 1.f : 0.f;
-#pragma unroll
-            for (int q = 0; q < r; ++q) v -= S[o + r][o + q] * x[q];
-            x[r] = r < lane ? 0.f : v;
-        }
-#pragma unroll
-        for (int r = 0; r < kMp; ++r) Xs[o + r][o + lane] = x[r];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int b = kMp; b < kP; b *= 2) {
-        // 8b threads per pair: column c, rows rg * (b / 8) .. + b / 8 of the pair's b x b product
-        const int pair = threadIdx.x / (8 * b), loc = threadIdx.x % (8 * b);
-        const int c = loc % b, q0 = (loc / b) * (b / 8);
-        const int o = 2 * b * pair;
-        float acc[kP / 16];
-#pragma unroll
-        for (int q = 0; q < b / 8; ++q) acc[q] = 0.f;
-        for (int kk = c; kk < b; ++kk) {
-            const float xk = Xs[o + kk][o + c];
-#pragma unroll
-            for (int q = 0; q < b / 8; ++q) acc[q] += S[o + b + q0 + q][o + kk] * xk;
-        }
-#pragma unroll
-        for (int q = 0; q < b / 8; ++q) Ts[b * pair + q0 + q][c] = acc[q];
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < b / 8; ++q) acc[q] = 0.f;
-        for (int r = 0; r < q0 + b / 8; ++r) {
-            const float t = Ts[b * pair + r][c];
-#pragma unroll
-            for (int q = 0; q < b / 8; ++q)
-                if (r <= q0 + q) acc[q] += Xs[o + b + q0 + q][o + b + r] * t;
-        }
-#pragma unroll
-        for (int q = 0; q < b / 8; ++q) Xs[o + b + q0 + q][o + c] = -acc[q];
-        __syncthreads();
-    }
-    for (int t = threadIdx.x; t < bs * bs; t += blockDim.x) {
-        const int i = t % bs, j = t / bs;
-        Linv[(size_t)j * ld + (k + i)] = Xs[i][j];
     }
 }
 
@@ -468,53 +451,6 @@ d32_diag_kernel(int ld, int k, int bs, float *__restrict__ A, float *__restrict_
             if (r < bs) A[(size_t)(k - kP + j) * ld + k + r] = L0[j * kP + r];
         }
     d32_diag_block(diag_smem(buf), ld, k, bs, A, D, d0, csum, np, per, eps, Linv);
-}
-
-// rows r in [k+64, n) of the panel (bs = 64 whenever rows remain below the block): 64 rows per
-// CTA, 4 rows x 4 columns per thread, T = A21 L11^-T staged through shared memory
-__global__ void __launch_bounds__(kTT)
-d32_panel_kernel(int n, int ld, int k, float *__restrict__ A, const float *__restrict__ D,
-                 const float *__restrict__ Linv, float *__restrict__ LD) {
-    __shared__ __align__(16) float As[kP][kP];   // As[l][r] = A(r0 + r, k + l)
-    __shared__ __align__(16) float Lt[kP][kP];   // Lt[l][j] = (L11^-1)_jl
-    const int r0 = k + kP + blockIdx.x * kP;
-    for (int t = threadIdx.x; t < kP * kP; t += blockDim.x) {
-        const int j = t % kP, l = t / kP;
-        Lt[l][j] = Linv[(size_t)l * ld + (k + j)];
-        As[l][j] = r0 + j < n ? A[(size_t)(k + l) * ld + r0 + j] : 0.f;
-    }
-    __syncthreads();
-    const int tr = threadIdx.x & 15, tc = threadIdx.x >> 4;  // rows tr*4.., columns tc*4..
-    float acc[4][4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int w = 0; w < 4; ++w) acc[u][w] = 0.f;
-#pragma unroll 16
-    for (int l = 0; l < kP; ++l) {
-        const float4 a = *(const float4 *)&As[l][tr * 4];
-        const float4 b = *(const float4 *)&Lt[l][tc * 4];
-        const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int w = 0; w < 4; ++w) acc[u][w] += av[u] * bv[w];
-    }
-#pragma unroll
-    for (int w = 0; w < 4; ++w) {
-        const int j = tc * 4 + w;
-        const float dj = D[k + j];
-        const bool inf = isinf(dj);
-        const float id = inf ? 0.f : 1.f / dj;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int r = r0 + tr * 4 + u;
-            if (r < n) {
-                LD[(size_t)j * ld + r] = inf ? 0.f : acc[u][w];
-                A[(size_t)(k + j) * ld + r] = acc[u][w] * id;
-            }
-        }
-    }
 }
 
 // block row k of X = L^-1 for the columns [c0, c0+64) of [0, k+bs); 4 rows x 4 columns per thread
@@ -565,9 +501,8 @@ d32_invrow_kernel(int ld, int k, int bs, float *__restrict__ X, const float *__r
 }
 
 // The two rank-64 updates of panel k (trailing triangle A22 -= LD L21^T, rows of L^-1 below the
-// panel B -= L21 X_k) are split in two launches: d32_update1_kernel covers what the next panel
-// needs (its 64 columns of A22 and its 64 rows of B, 64x64 tiles) and d32_update_kernel the rest
-// (rows and columns from base2 = k + 128 on, 128x128 tiles, 8x8 per thread).
+// panel B -= L21 X_k): d32_step_kernel covers the blocks that the chain needs next, d32_update_kernel
+// (128x128 tiles, 8x8 per thread) or, two panels at once, d32_tc_update_kernel the rest.
 __device__ __forceinline__ void tri_decode(int idx, int &ti, int &tj) {
     ti = (int)((sqrt(8.0 * idx + 1.0) - 1.0) * 0.5);
     while ((ti + 1) * (ti + 2) / 2 <= idx) ++ti;
@@ -575,109 +510,14 @@ __device__ __forceinline__ void tri_decode(int idx, int &ti, int &tj) {
     tj = idx - ti * (ti + 1) / 2;
 }
 
-// the next panel's part: blocks [0, ts) are the 64-column strip of A22 in 64-row tiles (with the
-// strip's column sums below the next diagonal block, csum[s * 64 + c], fixed-order partials),
-// blocks [ts, ts + tx) the next panel's 64 rows of B in 64-column tiles; all of K = 64 staged once
-__global__ void __launch_bounds__(kTT)
-d32_update1_kernel(int n, int ld, int k, float *__restrict__ A, float *__restrict__ X,
-                   const float *__restrict__ LD, float *__restrict__ csum) {
-    __shared__ __align__(16) float As[kP][kP];   // As[l][r] = A operand (row r0 + r, depth l)
-    __shared__ __align__(16) float Bs[kP][kP];   // Bs[l][c] = B operand (column c0 + c, depth l)
-    const int base = k + kP;
-    const int ts = (n - base + kP - 1) / kP;
-    const bool strip = (int)blockIdx.x < ts;
-    const int r0 = strip ? base + (int)blockIdx.x * kP : base;
-    const int c0 = strip ? base : ((int)blockIdx.x - ts) * kP;
-    const int climit = strip ? n : base;
-    const float *Pa = strip ? LD : A + (size_t)k * ld;
-    const float *Pb = A + (size_t)k * ld;
-    for (int t = threadIdx.x; t < kP * (kP / 4); t += kTT) {
-        const int l = t / (kP / 4), q = (t % (kP / 4)) * 4;
-        const float *src = Pa + (size_t)l * ld + r0 + q;
-        float4 v;
-        if (r0 + q + 4 <= n) v = *(const float4 *)src;
-        else {
-            v.x = r0 + q < n ? src[0] : 0.f;
-            v.y = r0 + q + 1 < n ? src[1] : 0.f;
-            v.z = r0 + q + 2 < n ? src[2] : 0.f;
-            v.w = r0 + q + 3 < n ? src[3] : 0.f;
-        }
-        *(float4 *)&As[l][q] = v;
-        if (strip) {
-            const float *sb = Pb + (size_t)l * ld + c0 + q;
-            float4 w;
-            if (c0 + q + 4 <= climit) w = *(const float4 *)sb;
-            else {
-                w.x = c0 + q < climit ? sb[0] : 0.f;
-                w.y = c0 + q + 1 < climit ? sb[1] : 0.f;
-                w.z = c0 + q + 2 < climit ? sb[2] : 0.f;
-                w.w = c0 + q + 3 < climit ? sb[3] : 0.f;
-            }
-            *(float4 *)&Bs[l][q] = w;
-        } else {
-            const int c = t % kP, lq = (t / kP) * 4;
-            float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (c0 + c < climit) w = *(const float4 *)(X + (size_t)(c0 + c) * ld + k + lq);
-            Bs[lq][c] = w.x;
-            Bs[lq + 1][c] = w.y;
-            Bs[lq + 2][c] = w.z;
-            Bs[lq + 3][c] = w.w;
-        }
-    }
-    __syncthreads();
-    const int tr = threadIdx.x & 15, tc = threadIdx.x >> 4;   // rows tr*4.., columns tc*4..
-    float acc[4][4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int w = 0; w < 4; ++w) acc[u][w] = 0.f;
-#pragma unroll 16
-    for (int l = 0; l < kP; ++l) {
-        const float4 a = *(const float4 *)&As[l][tr * 4];
-        const float4 b = *(const float4 *)&Bs[l][tc * 4];
-        const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int w = 0; w < 4; ++w) acc[u][w] += av[u] * bv[w];
-    }
-    float *C = strip ? A : X;
-    float cs[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-    for (int w = 0; w < 4; ++w) {
-        const int c = c0 + tc * 4 + w;
-        if (c >= climit) continue;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int r = r0 + tr * 4 + u;
-            if (r < n && (!strip || r > c)) {
-                const float v = C[(size_t)c * ld + r] - acc[u][w];
-                C[(size_t)c * ld + r] = v;
-                if (r >= base + kP) cs[w] += v;
-            }
-        }
-    }
-    if (strip) {
-        // the 16 threads with this tc are one half-warp (lanes tr = 0..15)
-#pragma unroll
-        for (int w = 0; w < 4; ++w) {
-            float v = cs[w];
-#pragma unroll
-            for (int o = 1; o < 16; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (tr == 0) csum[(size_t)blockIdx.x * kP + tc * 4 + w] = v;
-        }
-    }
-}
-
-// the rest of the update from base2 = base + skip * 64 on (skip = 1, or 2 when the block after
-// the next panel went to its own d32_update1_kernel launch)
+// the rest of the update of panel k, from base2 = base + 128 on
 __global__ void __launch_bounds__(kTT, 2)
-d32_update_kernel(int n, int ld, int k, int skip, float *__restrict__ A, float *__restrict__ X,
+d32_update_kernel(int n, int ld, int k, float *__restrict__ A, float *__restrict__ X,
                   const float *__restrict__ LD) {
     // two stages: slice s + 1 is fetched into registers while slice s is multiplied
     __shared__ __align__(16) float As[2][kKc][kTile];
     __shared__ __align__(16) float Bs[2][kKc][kTile];
-    const int base = k + kP, base2 = base + skip * kP;
+    const int base = k + kP, base2 = base + 2 * kP;
     const int t = (n - base2 + kTile - 1) / kTile;   // row / column tiles from base2 on
     const int tcn = (base + kTile - 1) / kTile;      // column tiles of the rows of L^-1
     const int idx = blockIdx.x;
@@ -794,7 +634,7 @@ d32_update_kernel(int n, int ld, int k, int skip, float *__restrict__ A, float *
     }
 }
 
-// ------------------------------------------------------------------ fused panel step (SIMT path)
+// ------------------------------------------------------------------ fused panel step
 // One launch per panel k (bs = 64, base = k + 64 < n) does what the next diagonal block waits for,
 // so the panel-to-panel chain is two kernels (this one and the next diagonal block).  Its units are
 // 64-row strips and 64-column blocks, each split over two CTAs (CTA 2 s + h takes half h of unit s),
@@ -803,16 +643,18 @@ d32_update_kernel(int n, int ld, int k, int skip, float *__restrict__ A, float *
 //   strip s (rows R = base + 64 s ..), half rows R_h = R[32 h, 32 h + 32): LD[R_h] = A21[R_h] L11^-T
 //     and L21[R_h] = LD[R_h] D1^-1 (the panel), then the next panel's 64 columns A22[R_h, R0] -=
 //     LD[R_h] L21[R0]^T (R0 = the next panel's rows; L21[R0] recomputed in every CTA from the
-//     unscaled A21[R0]) together with the previous panel's update of the same columns, -= LD'[R_h]
-//     L21'[R0]^T, and the fixed-order partial column sums below the next diagonal block (one row of
+//     unscaled A21[R0]) together with the update of the same columns by the npv previous panels that
+//     the rest-updates have left to it, -= LD'[R_h] L21'[R0]^T, and the fixed-order partial column sums below the next diagonal block (one row of
 //     csum per half: row 2 s + h);
 //   X block s - ts (columns C = 64 (s - ts) .. of block row k of L^-1), half columns C_h:
 //     X[k, C_h] = L11^-1 B[k, C_h] (the block row), then X[R0, C_h] -= L21[R0] X[k, C_h] +
-//     L21'[R0] X[k - 64, C_h] (the previous panel's part);
+//     L21'[R0] X[k - 64, C_h] (+ the one before, likewise);
 // L21[R0] goes to A with the next diagonal block's kernel (the other CTAs read A21[R0] unscaled).
-// What remains of both updates (rows and columns from base + 128) is d32_update_kernel's (skip 2).
-constexpr int kStepSmem = (5 * kP * kP + kP) * 4;
+// What remains of both updates is the rest-update's: d32_update_kernel takes one panel's from base +
+// 128 on (npv = 1), d32_tc_update_kernel that of panels p and p + 1 (p even) from block p + 4 on, so
+// that block p + 3 gets its part of panel p with step p + 2: npv = 2 for even panels, 1 for odd ones.
 constexpr int kHalf = kP / 2;
+constexpr int step_smem(int npv) { return ((5 + 3 * npv) * kP * kP / 2 + kP) * 4; }
 
 // acc[u][w] += sum_l a[l][tr * 4 + u] b[l][tc * 4 + w] (64 x 64 operands, [depth][index])
 __device__ __forceinline__ void mm64(const float *__restrict__ a, const float *__restrict__ b, float (&acc)[4][4],
@@ -829,12 +671,13 @@ __device__ __forceinline__ void mm64(const float *__restrict__ a, const float *_
     }
 }
 
-// 32 x 64 outputs: acc[u][w] += sum_l a[l][tr * 2 + u] b[l][tc * 4 + w] (a's first 32 indices)
+// 32 x 64 outputs: acc[u][w] += sum_l a[l][tr * 2 + u] b[l][tc * 4 + w] (a's rows SA apart)
+template <int SA>
 __device__ __forceinline__ void mm_r32(const float *__restrict__ a, const float *__restrict__ b, float (&acc)[2][4],
                                        int tr, int tc) {
 #pragma unroll 16
     for (int l = 0; l < kP; ++l) {
-        const float2 x = *(const float2 *)(a + l * kP + tr * 2);
+        const float2 x = *(const float2 *)(a + l * SA + tr * 2);
         const float4 y = *(const float4 *)(b + l * kP + tc * 4);
         const float av[2] = {x.x, x.y}, bv[4] = {y.x, y.y, y.z, y.w};
 #pragma unroll
@@ -844,13 +687,13 @@ __device__ __forceinline__ void mm_r32(const float *__restrict__ a, const float 
     }
 }
 
-// 64 x 32 outputs: acc[u][w] += sum_l a[l][tr * 4 + u] b[l][tc * 2 + w] (b's first 32 indices)
+// 64 x 32 outputs: acc[u][w] += sum_l a[l][tr * 4 + u] b[l][tc * 2 + w] (b: 64 x 32)
 __device__ __forceinline__ void mm_c32(const float *__restrict__ a, const float *__restrict__ b, float (&acc)[4][2],
                                        int tr, int tc) {
 #pragma unroll 16
     for (int l = 0; l < kP; ++l) {
         const float4 x = *(const float4 *)(a + l * kP + tr * 4);
-        const float2 y = *(const float2 *)(b + l * kP + tc * 2);
+        const float2 y = *(const float2 *)(b + l * kHalf + tc * 2);
         const float av[4] = {x.x, x.y, x.z, x.w}, bv[2] = {y.x, y.y};
 #pragma unroll
         for (int u = 0; u < 4; ++u)
@@ -860,7 +703,7 @@ __device__ __forceinline__ void mm_c32(const float *__restrict__ a, const float 
 }
 
 // tile[l][r] = G[(col0 + l) ld + row0 + r] for r < R and row0 + r < rlim, else 0 (row0 a multiple
-// of 4; depth 64, tile stride 64)
+// of 4; depth 64, tile stride R)
 template <int R>
 __device__ __forceinline__ void load_cm(float *__restrict__ tile, const float *__restrict__ G, int ld, int col0,
                                         int row0, int rlim) {
@@ -875,12 +718,12 @@ __device__ __forceinline__ void load_cm(float *__restrict__ tile, const float *_
             v.z = row0 + q + 2 < rlim ? src[2] : 0.f;
             v.w = row0 + q + 3 < rlim ? src[3] : 0.f;
         }
-        *(float4 *)(tile + l * kP + q) = v;
+        *(float4 *)(tile + l * R + q) = v;
     }
 }
 
 // tile[l][c] = X(row0 + l, c0 + c) = X[(c0 + c) ld + row0 + l] for c < C and c0 + c < climit, else
-// 0 (depth 64, tile stride 64)
+// 0 (depth 64, tile stride C)
 template <int C>
 __device__ __forceinline__ void load_rows_of_x(float *__restrict__ tile, const float *__restrict__ X, int ld,
                                                int row0, int c0, int climit) {
@@ -888,25 +731,27 @@ __device__ __forceinline__ void load_rows_of_x(float *__restrict__ tile, const f
         const int c = t % C, lq = (t / C) * 4;
         float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
         if (c0 + c < climit) w = *(const float4 *)(X + (size_t)(c0 + c) * ld + row0 + lq);
-        tile[(lq + 0) * kP + c] = w.x;
-        tile[(lq + 1) * kP + c] = w.y;
-        tile[(lq + 2) * kP + c] = w.z;
-        tile[(lq + 3) * kP + c] = w.w;
+        tile[(lq + 0) * C + c] = w.x;
+        tile[(lq + 1) * C + c] = w.y;
+        tile[(lq + 2) * C + c] = w.z;
+        tile[(lq + 3) * C + c] = w.w;
     }
 }
 
 __global__ void __launch_bounds__(kTT)
-d32_step_kernel(int n, int ld, int k, float *__restrict__ A, float *__restrict__ X,
+d32_step_kernel(int n, int ld, int k, int npv, float *__restrict__ A, float *__restrict__ X,
                 const float *__restrict__ D, const float *__restrict__ Linv, float *__restrict__ LDc,
-                const float *__restrict__ LDprev, float *__restrict__ L0buf, float *__restrict__ csum) {
+                const float *__restrict__ LDprev, const float *__restrict__ LDprev2, float *__restrict__ L0buf,
+                float *__restrict__ csum) {
     extern __shared__ __align__(16) float sm[];
-    float *Lt = sm, *T1 = sm + kP * kP, *T2 = sm + 2 * kP * kP, *T3 = sm + 3 * kP * kP, *T4 = sm + 4 * kP * kP;
-    float *idv = sm + 5 * kP * kP;
+    float *idv = sm, *Lt = sm + kP, *T1 = Lt + kP * kP, *T2 = T1 + kP * kHalf;   // T1: 64 x 32
+    // per previous panel a 64 x 64 tile and a 64 x 32 one
+    float *T4 = T2 + kP * kP, *T3 = T4 + kP * kP, *T6 = T3 + kP * kHalf, *T5 = T6 + kP * kP;
     const int base = k + kP;
     const int ts = (n - base + kP - 1) / kP;
     const int unit = (int)blockIdx.x >> 1, h = (int)blockIdx.x & 1;
     const bool strip = unit < ts;
-    const bool prev = k > 0;
+    const bool prev = npv > 0, prev2 = npv > 1;
     const int tr = threadIdx.x & 15, tc = threadIdx.x >> 4;
     // Lt[l][j] = (L11^-1)_jl; idv = D1^+ (0 for grounded pivots)
     for (int t = threadIdx.x; t < kP * kP; t += blockDim.x) {
@@ -945,9 +790,14 @@ d32_step_kernel(int n, int ld, int k, float *__restrict__ A, float *__restrict__
             load_cm<kHalf>(T3, LDprev, ld, 0, rh, n);           // LD'[R_h]     [j][r]
             load_cm<kP>(T4, A, ld, k - kP, base, n);            // L21'[R0]     [j][c]
         }
+        if (prev2) {
+            load_cm<kHalf>(T5, LDprev2, ld, 0, rh, n);
+            load_cm<kP>(T6, A, ld, k - 2 * kP, base, n);
+        }
         __syncthreads();
         // LD(R_h row tr*2+u, j = tc*4+w) (the first strip's rows are R0's: read from T2)
-        mm_r32(rb > 0 ? T1 : T2 + h * kHalf, Lt, acc, tr, tc);
+        if (rb > 0) mm_r32<kHalf>(T1, Lt, acc, tr, tc);
+        else mm_r32<kP>(T2 + h * kHalf, Lt, acc, tr, tc);
         mm64(T2, Lt, acc2, tr, tc);                             // LD(R0 row tr*4+u, j = tc*4+w)
         __syncthreads();
 #pragma unroll
@@ -964,14 +814,15 @@ d32_step_kernel(int n, int ld, int k, float *__restrict__ A, float *__restrict__
                     if (rb == 0) L0buf[j * kP + h * kHalf + rr] = acc[u][w] * id;
                     else A[(size_t)(k + j) * ld + r] = acc[u][w] * id;
                 }
-                T1[j * kP + rr] = ldv;                                      // A operand [j][r]
+                T1[j * kHalf + rr] = ldv;                                   // A operand [j][r]
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) T2[j * kP + tr * 4 + u] = acc2[u][w] * id;   // B operand [j][c]
         }
         __syncthreads();
-        mm_r32(T1, T2, acc3, tr, tc);
-        if (prev) mm_r32(T3, T4, acc3, tr, tc);
+        mm_r32<kHalf>(T1, T2, acc3, tr, tc);
+        if (prev) mm_r32<kHalf>(T3, T4, acc3, tr, tc);
+        if (prev2) mm_r32<kHalf>(T5, T6, acc3, tr, tc);
         // A22[R_h, R0] -= acc3 below the diagonal; column sums of the rows below the next block
         float cs[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -1019,8 +870,12 @@ d32_step_kernel(int n, int ld, int k, float *__restrict__ A, float *__restrict__
         if (before) load_rows_of_x<kHalf>(T1, X, ld, k, ch, k);     // B[k, C_h]      [l][c], c < 32
         load_cm<kP>(T2, A, ld, k, base, n);                          // A21[R0]        [l][r]
         if (prev && before) {
-            load_cm<kP>(T3, A, ld, k - kP, base, n);                 // L21'[R0]       [j][r]
-            load_rows_of_x<kHalf>(T4, X, ld, k - kP, ch, k);         // X[k - 64, C_h] [j][c]
+            load_cm<kP>(T4, A, ld, k - kP, base, n);                 // L21'[R0]       [j][r]
+            load_rows_of_x<kHalf>(T3, X, ld, k - kP, ch, k);         // X[k - 64, C_h] [j][c]
+        }
+        if (prev2 && before) {
+            load_cm<kP>(T6, A, ld, k - 2 * kP, base, n);
+            load_rows_of_x<kHalf>(T5, X, ld, k - 2 * kP, ch, k - kP);
         }
         __syncthreads();
         if (before) mm_c32(Lt, T1, acc, tr, tc);              // X(k + i, c), i = tr*4+u, c = tc*2+w
@@ -1033,7 +888,7 @@ d32_step_kernel(int n, int ld, int k, float *__restrict__ A, float *__restrict__
                 const int i = tr * 4 + u, c = tc * 2 + w;
                 const float x = before ? acc[u][w] : Lt[(h * kHalf + c) * kP + i];
                 X[(size_t)(ch + c) * ld + (k + i)] = x;
-                T1[i * kP + c] = x;                                          // B operand [i][c]
+                T1[i * kHalf + c] = x;                                       // B operand [i][c]
             }
 #pragma unroll
             for (int w = 0; w < 4; ++w)
@@ -1041,7 +896,8 @@ d32_step_kernel(int n, int ld, int k, float *__restrict__ A, float *__restrict__
         }
         __syncthreads();
         mm_c32(T2, T1, acc3, tr, tc);
-        if (prev && before) mm_c32(T3, T4, acc3, tr, tc);
+        if (prev && before) mm_c32(T4, T3, acc3, tr, tc);
+        if (prev2 && before) mm_c32(T6, T5, acc3, tr, tc);
 #pragma unroll
         for (int w = 0; w < 2; ++w) {
             const int c = ch + tc * 2 + w;
@@ -1055,243 +911,291 @@ d32_step_kernel(int n, int ld, int k, float *__restrict__ A, float *__restrict__
 }
 
 // ------------------------------------------------------------------ tensor-core bulk update
-// The bulk update C -= A_op B_op^T (depth 64, one panel) on the fifth-generation tensor cores in
-// split TF32: a = a_hi + a_lo with a_hi the TF32 rounding of a, and C -= a_hi b_hi + a_hi b_lo +
-// a_lo b_hi (the a_lo b_lo term is below FP32 rounding), accumulated in FP32 in tensor memory.
+// The rest-update C -= A_op B_op^T of two panels (depth 128) on the fifth-generation tensor cores, each
+// FP32 operand as the sum of three BF16 pieces (8 + 8 + 8 bits: exact) a = a1 + a2 + a3 and C -= a1 b1 +
+// (a1 b2 + a2 b1 + a1 b3 + a3 b1 + a2 b2) (what is left out is 2^-24 of a b and below).  The tensor cores
+// truncate a sum that they add to, and here all terms have one sign, so every MMA into an accumulator
+// costs it a part of its last place.  So the five small products of both panels go to one accumulator
+// before anything large does, a1 b1 of the first panel to another and a1 b1 of the second, last, on top of the
+// small ones: four MMAs into a large sum.  Relative
+// error of X = L^-1 against FP64 at n = 8281 (RMS, largest): 6.5e-7, 3.2e-6; 1.2e-6, 4.8e-6 with all of a1 b1
+// in one accumulator; 1.5e-6, 4.4e-6 with two TF32 pieces, one panel, and 24 MMAs into one (2.5e-6, 7.5e-6 for
+// two panels).  The FP32 SIMT update has 2.4e-7, 2.2e-6 and stays below n = 8192, where it was the choice
+// before; from there on it takes 15.6 ms against 7.4.
 // Once per panel the operands are split and written in the MMA's shared-memory layout (K-major,
-// no swizzle: 8-row x 16-byte core matrices; core matrix (row / 8, k / 4) of an R-row block at
-// byte ((k / 4) (R / 8) + row / 8) 128, its row (row % 8) at 16-byte steps), so a tile fetches its
-// operands with four bulk copies completing on one mbarrier, one thread issues 3 x 8 MMAs
-// (M = 128, N = 64, K = 8 each), and all four warps read the accumulator back (each warp its 32
-// lanes) and subtract it from C.  Every wait is bounded: a wait that gives up records the failure
-// in *err, waits once more for its own copies or MMAs, releases the tensor memory and returns.
-constexpr int kTcM = 128, kTcN = 256;                 // tile rows, tile columns
-constexpr int kTcApiece = kTcM * kP * 4;              // one A piece (hi or lo): 32 KB
-constexpr int kTcBpiece = kTcN * kP * 4;              // one B piece: 64 KB
-constexpr int kTcSmem = 2 * kTcApiece + 2 * kTcBpiece + 64;
-constexpr int kTcThreads = 160;   // four epilogue warps and one producer warp
+// no swizzle: core matrices of 8 rows x 8 depths (16 bytes), (row / 8, k / 8) of a 128-row piece of 16
+// depths at byte ((k / 8) 16 + row / 8) 128, row row % 8 at 16-byte steps), the three pieces of 16 depths
+// together, so that a stage is two bulk copies completing on one mbarrier.
+constexpr int kTcM = 128;                             // tile rows and columns
+constexpr int kTcK = 16, kTcStages = 4;               // depth of a stage, stages of the ring
+constexpr int kTcPiece = kTcM * kTcK * 2;             // one BF16 piece of a stage: 4 KB
+constexpr int kTcOperand = 3 * kTcPiece;              // one operand of a stage
+constexpr int kTcStage = 2 * kTcOperand;
+constexpr int kTcBlock = kP / kTcK * kTcOperand;      // 128 rows of one panel's operand: 48 KB
+constexpr int kTcPer = 2 * kP / kTcK;                 // stages of a tile: two panels
+constexpr int kTcSmem = 116 * 1024;   // 96 KB used; more than half an SM's, so that a CTA cannot start beside
+                                      // another one that holds all of the tensor memory
+static_assert(kTcSmem >= kTcStages * kTcStage + 128 && 2 * kTcSmem > 228 * 1024, "stages and barriers");
+static_assert(kTcPer == 2 * kTcStages, "the ring holds a panel");
 constexpr int kTcAutoN = 8192;    // tc_mode 0: the tensor-core update from this n on
-__device__ __forceinline__ float tc_tf32(float x) {
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return __uint_as_float(r);
+constexpr uint32_t kTcIdesc = tc_idesc(1u, kTcM, kTcM);   // BF16, both K-major
+
+// Split operands of one panel in blocks of 128 rows: LD rows (A of the trailing tiles), panel rows (their
+// B, and A of the inverse's tiles), rows of L^-1 by column (B of the inverse's)
+struct TcOps { unsigned char *LDs, *Ps, *Xs; };
+__host__ __device__ __forceinline__ size_t tc_op_bytes(int n) { return (size_t)ceil_div(n, kTcM) * kTcBlock; }
+__host__ __device__ __forceinline__ size_t tc_per_panel(int n) { return 3 * tc_op_bytes(n); }
+__host__ __device__ __forceinline__ TcOps tc_ops(unsigned char *buf, int n) {
+    return {buf, buf + tc_op_bytes(n), buf + 2 * tc_op_bytes(n)};
 }
 
-// kind::tf32 instruction descriptor: D = F32, A = B = TF32, both K-major, M = 128, N = 256
-constexpr uint32_t kTcIdesc = tc_idesc(2u, kTcM, kTcN);
+// depths 8 kg .. 8 kg + 7 of row r, split into its three pieces
+__device__ __forceinline__ void tc_put(unsigned char *op, int r, int kg, const float (&v)[8]) {
+    uint32_t w[3][4];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        float x = v[q];
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+            const __nv_bfloat16 b = __float2bfloat16(x);
+            x -= __bfloat162float(b);
+            const uint32_t u = __bfloat16_as_ushort(b);
+            w[e][q >> 1] = q & 1 ? w[e][q >> 1] | (u << 16) : u;
+        }
+    }
+    unsigned char *at = op + (size_t)(r / kTcM) * kTcBlock + (kg >> 1) * kTcOperand + ((kg & 1) * 16 + (r % kTcM) / 8) * 128 +
+                        (r & 7) * 16;
+#pragma unroll
+    for (int e = 0; e < 3; ++e) *(uint4 *)(at + e * kTcPiece) = make_uint4(w[e][0], w[e][1], w[e][2], w[e][3]);
+}
 
-// Rows [row0 + b RB, +RB) of an operand, depth 64, split into TF32 hi / lo pieces in the layout
-// above: piece (b, hi) at out + 2 b P, (b, lo) at out + (2 b + 1) P (P = RB * 64 floats).  The
-// element (row r, depth l) is src[l * ld + r] (a column-major panel) or, kmaj, src[r * ld + l]
-// (rows of L^-1 held by column); rows at or beyond `rows` are zero.
-template <int RB, bool KMAJ>
+// The split operands of panels k0 and k0 + 64 (blockIdx.y) for the rest-update from base2 on, 128 rows per
+// CTA: first the rows of LD and of the panel (T blocks; rows at or beyond n are zero), then the columns
+// of the panel's block row of L^-1 (zero from the panel's end on).
 __global__ void __launch_bounds__(kTT)
-d32_tc_split_kernel(int rows, int ld, const float *__restrict__ src, int row0, float *__restrict__ out) {
-    const int b = blockIdx.x;
-    float *hi = out + (size_t)(2 * b) * RB * kP, *lo = hi + (size_t)RB * kP;
-    for (int t = threadIdx.x; t < RB * (kP / 4); t += blockDim.x) {
-        const int r = t % RB, kq = t / RB;
-        const int row = row0 + b * RB + r;
-        float v[4];
+d32_tc_split_kernel(int n, int ld, int k0, int base2, int T, const float *__restrict__ A, const float *__restrict__ X,
+                    const float *__restrict__ LD0, const float *__restrict__ LD1, unsigned char *__restrict__ buf) {
+    const int k = k0 + (int)blockIdx.y * kP, base = k + kP;
+    const float *LD = blockIdx.y ? LD1 : LD0, *P = A + (size_t)k * ld;
+    const TcOps o = tc_ops(buf + blockIdx.y * tc_per_panel(n), n);
+    const bool rows = (int)blockIdx.x < T;
+    const int b0 = ((int)blockIdx.x - (rows ? 0 : T)) * kTcM;
+    float v[8];
+    if (rows) {
+        for (int t = threadIdx.x; t < kTcM * (kP / 8); t += kTT) {
+            const int r = b0 + t % kTcM, kg = t / kTcM, row = base2 + r;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int l = kq * 4 + q;
-            v[q] = row < rows ? (KMAJ ? src[(size_t)row * ld + l] : src[(size_t)l * ld + row]) : 0.f;
-        }
-        float h[4], w[4];
+            for (int q = 0; q < 8; ++q) v[q] = row < n ? P[(size_t)(kg * 8 + q) * ld + row] : 0.f;
+            tc_put(o.Ps, r, kg, v);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            h[q] = tc_tf32(v[q]);
-            w[q] = v[q] - h[q];
+            for (int q = 0; q < 8; ++q) v[q] = row < n ? LD[(size_t)(kg * 8 + q) * ld + row] : 0.f;
+            tc_put(o.LDs, r, kg, v);
         }
-        const size_t off = ((size_t)kq * (RB / 8) + (r >> 3)) * 32 + (size_t)(r & 7) * 4;  // in floats
-        *(float4 *)(hi + off) = make_float4(h[0], h[1], h[2], h[3]);
-        *(float4 *)(lo + off) = make_float4(w[0], w[1], w[2], w[3]);
-    }
-}
-
-// Tile t of one panel's bulk update: tiles [0, T TJ) are the trailing triangle from base2 (row
-// tile ti of 128, column tile tj of 256; only those that start left of the row tile's last row),
-// then T x tcx tiles of the rows of L^-1 (C = X, columns below base).  False: nothing to do.
-__device__ __forceinline__ bool tc_tile(int t, int n, int base, int base2, int T, int TJ, int tcx, bool &tri, int &ti,
-                                        int &tj, int &r0, int &c0, int &climit) {
-    const int ntri = T * TJ;
-    tri = t < ntri;
-    if (tri) {
-        ti = t / TJ;
-        tj = t % TJ;
-        if (tj * kTcN >= (ti + 1) * kTcM) return false;
     } else {
-        ti = (t - ntri) / tcx;
-        tj = (t - ntri) % tcx;
-    }
-    r0 = base2 + ti * kTcM;
-    c0 = tri ? base2 + tj * kTcN : tj * kTcN;
-    climit = tri ? n : base;
-    return r0 < n && c0 < climit;
-}
-
-__device__ __forceinline__ int tc_next(int t, int step, int ntiles, int n, int base, int base2, int T, int TJ,
-                                       int tcx) {
-    bool tri;
-    int ti, tj, r0, c0, cl;
-    while (t < ntiles && !tc_tile(t, n, base, base2, T, TJ, tcx, tri, ti, tj, r0, c0, cl)) t += step;
-    return t;
-}
-
-// Persistent CTAs (one per SM), each taking tiles gridDim.x apart, warp-specialised: warp 4 (one
-// lane) brings each tile's four operand pieces with two bulk copies on an mbarrier and issues its
-// 3 x 8 MMAs into one of two tensor-memory accumulators, committing them to that accumulator's
-// "full" mbarrier; warps 0-3 (tensor-memory lanes 0-127) wait for it, subtract the accumulator
-// from C and arrive on its "empty" mbarrier.  So tile i + 1's copies and MMAs run while tile i's
-// epilogue does; the single operand stage is refilled once tile i's MMAs are done.  Every wait
-// is bounded: one that gives up records the failure in *err and the CTA winds down (its own
-// copies and MMAs waited for once more) before it releases the tensor memory.  Operand pieces:
-// trailing A = split L D rows, B = split panel rows (256-row blocks); inverse A = split panel rows
-// (128-row blocks), B = split rows of L^-1.
-constexpr int kTcWarps = 5;
-
-__global__ void __launch_bounds__(kTcWarps * 32, 1)
-d32_tc_update_kernel(int n, int ld, int base, int base2, int T, const float *__restrict__ LDs,
-                     const float *__restrict__ PBs, const float *__restrict__ PAs, const float *__restrict__ XBs,
-                     float *__restrict__ A, float *__restrict__ X, int *__restrict__ err) {
-    extern __shared__ __align__(1024) unsigned char smem[];
-    const int TJ = (int)ceil_div(T * kTcM, kTcN), tcx = (int)ceil_div(base, kTcN);
-    const int ntiles = T * TJ + T * tcx, step = (int)gridDim.x;
-    const int first = tc_next((int)blockIdx.x, step, ntiles, n, base, base2, T, TJ, tcx);
-    if (first >= ntiles) return;   // no tile for this CTA: uniform, nothing started
-    uint64_t *mbs = (uint64_t *)(smem + 2 * kTcApiece + 2 * kTcBpiece);
-    // [0] load, [1..2] full (per accumulator), [3..4] empty (per accumulator)
-    uint32_t *tslot = (uint32_t *)(mbs + 5);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     :: "r"(tc_smem_u32(tslot)), "r"(2 * kTcN) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    const uint32_t mbl = tc_smem_u32(mbs), sbase = tc_smem_u32(smem);
-    const uint32_t mfull[2] = {tc_smem_u32(mbs + 1), tc_smem_u32(mbs + 2)};
-    const uint32_t mempty[2] = {tc_smem_u32(mbs + 3), tc_smem_u32(mbs + 4)};
-    if (threadIdx.x == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(mbl) : "memory");
-        for (int q = 0; q < 2; ++q) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(mfull[q]) : "memory");
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;" :: "r"(mempty[q]) : "memory");
+        // a warp takes 8 columns by 32 rows at a time: 128-byte reads, 128-byte writes
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        for (int t = warp; t < kTcM / 8 * (kP / 32); t += kTT / 32) {
+            const int r = b0 + (t / (kP / 32)) * 8 + (lane & 7), kg = (t % (kP / 32)) * 4 + (lane >> 3);
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
+            if (r < base) {
+                const float4 *src = (const float4 *)(X + (size_t)r * ld + k + kg * 8);
+                x = src[0];
+                y = src[1];
+            }
+            v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+            v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
+            tc_put(o.Xs, r, kg, v);
         }
+    }
+}
+
+// Tile t of a rest-update: T (T + 1) / 2 tiles of the trailing triangle from base2, then T x tcx tiles of the
+// rows of L^-1 (C = X, columns below base)
+struct TcTile { bool tri; int ti, tj, r0, c0, climit; };
+__device__ __forceinline__ TcTile tc_tile(int t, int n, int base, int base2, int T, int tcx) {
+    TcTile q;
+    const int ntri = T * (T + 1) / 2;
+    q.tri = t < ntri;
+    if (q.tri) {
+        int ti = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
+        while ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
+        while (ti * (ti + 1) / 2 > t) --ti;
+        q.ti = ti;
+        q.tj = t - ti * (ti + 1) / 2;
+    } else {
+        q.ti = (t - ntri) / tcx;
+        q.tj = (t - ntri) % tcx;
+    }
+    q.r0 = base2 + q.ti * kTcM;
+    q.c0 = q.tri ? base2 + q.tj * kTcM : q.tj * kTcM;
+    q.climit = q.tri ? n : base;
+    return q;
+}
+
+// Persistent CTAs (one per SM), each taking tiles gridDim.x apart, warp-specialised.  One lane of warp 17
+// brings the operands through a ring of four stages of 16 depths (two bulk copies on the stage's "load"
+// mbarrier); one lane of warp 16 issues the MMAs into one of two pairs of accumulators, committing a
+// stage's last to its "free" mbarrier and a tile's last to the pair's "full"; warps 0-15 wait for that,
+// subtract the pair's sum from C and arrive on its "empty".  So the next tile's copies and MMAs run while a
+// tile's epilogue does, and each epilogue warp requests its 32 columns of the next tile's C as soon as it has
+// written this one's.
+// Every wait is bounded: one that gives up records the failure in *err and the CTA winds down (its own
+// copies and MMAs waited for once more) before it releases the tensor memory.
+// What bounds it is C, 64 KB read and 64 KB written per tile, in bursts.  n = 16,384, whole factorisation: 74 ms
+// with four epilogue warps (16 KB of C in flight per SM), one panel per pass and TF32 (66 of them in this
+// kernel, 2.7 TB/s of C); 47 with sixteen warps; 34.8 with two panels per pass; 34.0 so.  n = 8281: 14.1 ->
+// 7.4 ms; with a third of the panels done, 50 us per two panels, DRAM at 44 %, the tensor pipe at 41 %.
+// Bringing and storing C by bulk copies instead was slower (49 and 60 ms: 512-byte copies take about 60
+// clocks each), and so was keeping A in shared memory along a tile row (47 ms: no room for the accumulators'
+// second pair).
+constexpr int kTcEpi = 16, kTcThreads = (kTcEpi + 2) * 32;
+constexpr int kTcCols = kTcM / (kTcEpi / 4);   // columns of one epilogue warp
+
+__global__ void __launch_bounds__(kTcThreads, 1)
+d32_tc_update_kernel(int n, int ld, int base, int base2, int T, unsigned char *__restrict__ ops, float *__restrict__ A,
+                     float *__restrict__ X, int *__restrict__ err) {
+    extern __shared__ __align__(1024) unsigned char smem[];
+    const int tcx = (int)ceil_div(base, kTcM), ntiles = T * (T + 1) / 2 + T * tcx, step = (int)gridDim.x;
+    // load, free (kTcStages each), full, empty (one per pair of accumulators each)
+    uint64_t *mbs = (uint64_t *)(smem + kTcStages * kTcStage);
+    uint32_t *tslot = (uint32_t *)(mbs + 2 * kTcStages + 4);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp == 0) tc_alloc(tslot, 4 * kTcM);
+    const uint32_t sbase = tc_smem_u32(smem), mload = tc_smem_u32(mbs), mfree = mload + 8 * kTcStages;
+    const uint32_t mfull = mfree + 8 * kTcStages, mempty = mfull + 16;
+    if (threadIdx.x == 0) {
+        for (int q = 0; q < 2 * kTcStages + 2; ++q) tc_mbar_init(mload + 8 * q, 1);
+        for (int q = 0; q < 2; ++q) tc_mbar_init(mempty + 8 * q, kTcEpi);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    tc_fence_before();
     __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    tc_fence_after();
     const uint32_t tmem = *tslot;
-    if (warp == 4) {
+    auto copy = [](uint32_t dst, const void *src, uint32_t bytes, uint32_t mb) {
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                     :: "r"(dst), "l"(src), "r"(bytes), "r"(mb) : "memory");
+    };
+    auto expect = [](uint32_t mb, uint32_t bytes) {
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(mb), "r"(bytes) : "memory");
+    };
+    if (warp == kTcEpi) {
         if (lane == 0) {
-            int i = 0, failed = 0;
-            for (int t = first; t < ntiles && !failed; t = tc_next(t + step, step, ntiles, n, base, base2, T, TJ, tcx), ++i) {
+            const uint64_t d0 = tc_desc(sbase, (kTcM / 8) * 128);
+            constexpr uint32_t kPieceD = kTcPiece >> 4, kStageD = kTcStage >> 4;   // in the descriptor's address units
+            bool ok = true;
+            int g = 0, i = 0;   // stages whose last MMA is committed, tiles
+            for (int t = (int)blockIdx.x; t < ntiles && ok; t += step, ++i) {
                 const int bsel = i & 1;
-                // the stage is free once the previous tile's MMAs are done
-                if (i >= 1 && !tc_wait(mfull[(i - 1) & 1], (uint32_t)(((i - 1) >> 1) & 1))) { failed = 1; break; }
-                bool tri;
-                int ti, tj, r0, c0, cl;
-                tc_tile(t, n, base, base2, T, TJ, tcx, tri, ti, tj, r0, c0, cl);
-                const float *pa = (tri ? LDs : PAs) + (size_t)(2 * ti) * kTcM * kP;
-                const float *pb = (tri ? PBs : XBs) + (size_t)(2 * tj) * kTcN * kP;
-                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
-                             :: "r"(mbl), "r"((uint32_t)(2 * kTcApiece + 2 * kTcBpiece)) : "memory");
-                asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                             :: "r"(sbase), "l"(pa), "r"((uint32_t)(2 * kTcApiece)), "r"(mbl) : "memory");
-                asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                             :: "r"(sbase + 2 * kTcApiece), "l"(pb), "r"((uint32_t)(2 * kTcBpiece)), "r"(mbl) : "memory");
-                if (!tc_wait(mbl, (uint32_t)(i & 1))) {
-                    failed = 1;
-                    tc_wait(mbl, (uint32_t)(i & 1));   // the copies target this CTA's shared memory
-                    break;
-                }
-                // the accumulator is free once the epilogue of tile i - 2 is done
-                if (i >= 2 && !tc_wait(mempty[bsel], (uint32_t)(((i - 2) >> 1) & 1))) { failed = 1; break; }
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t acc = tmem + (uint32_t)(bsel * kTcN);
-                const uint32_t ah = sbase, al = sbase + kTcApiece;
-                const uint32_t bh = sbase + 2 * kTcApiece, bl = bh + kTcBpiece;
-                const uint32_t lboA = (kTcM / 8) * 128, lboB = (kTcN / 8) * 128;
+                const uint32_t first = tmem + (uint32_t)(bsel * 2 * kTcM), second = first + kTcM;
+                // the accumulators are free once the epilogue of tile i - 2 is done
+                if (i >= 2 && !tc_wait(mempty + 8 * bsel, (uint32_t)(((i - 2) >> 1) & 1))) { ok = false; break; }
 #pragma unroll
-                for (int ks = 0; ks < kP / 8; ++ks) {
-                    const uint32_t ka = (uint32_t)ks * 2 * lboA, kb = (uint32_t)ks * 2 * lboB;
-                    const uint64_t dah = tc_desc(ah + ka, lboA), dal = tc_desc(al + ka, lboA);
-                    const uint64_t dbh = tc_desc(bh + kb, lboB), dbl = tc_desc(bl + kb, lboB);
-                    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                                 " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n"
-                                 :: "r"(acc), "l"(dah), "l"(dbh), "r"(kTcIdesc), "r"(ks > 0 ? 1u : 0u) : "memory");
-                    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                                 " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n"
-                                 :: "r"(acc), "l"(dah), "l"(dbl), "r"(kTcIdesc), "r"(1u) : "memory");
-                    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                                 " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n"
-                                 :: "r"(acc), "l"(dal), "l"(dbh), "r"(kTcIdesc), "r"(1u) : "memory");
+                for (int q = 0; q < kTcPer + kTcStages; ++q) {
+                    // stages of panel 0, of panel 1 without a1 b1, then a1 b1 of panel 1
+                    const int slot = q % kTcStages;
+                    const uint64_t a0 = d0 + slot * kStageD, a1 = a0 + kPieceD, a2 = a1 + kPieceD;
+                    const uint64_t b0 = a2 + kPieceD, b1 = b0 + kPieceD, b2 = b1 + kPieceD;
+                    if (q < kTcPer) {
+                        if (!tc_wait(mload + 8 * slot, (uint32_t)((2 * i + q / kTcStages) & 1))) { ok = false; break; }
+                        tc_fence_after();
+                        tc_mma<true>(second, a0, b2, kTcIdesc, q > 0);
+                        tc_mma<true>(second, a2, b0, kTcIdesc, true);
+                        tc_mma<true>(second, a1, b1, kTcIdesc, true);
+                        tc_mma<true>(second, a0, b1, kTcIdesc, true);
+                        tc_mma<true>(second, a1, b0, kTcIdesc, true);
+                    }
+                    if (q < kTcStages) tc_mma<true>(first, a0, b0, kTcIdesc, q > 0);
+                    if (q >= kTcPer) tc_mma<true>(second, a0, b0, kTcIdesc, true);
+                    if (q < kTcStages || q >= kTcPer) {
+                        tc_commit(mfree + 8 * slot);
+                        ++g;
+                    }
                 }
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                             :: "r"(mfull[bsel]) : "memory");
+                if (ok) tc_commit(mfull + 8 * bsel);
             }
-            if (failed) atomicExch(err, 1);
-            // before the CTA ends: the last MMAs issued must be complete (bounded)
-            if (i >= 1) tc_wait(mfull[(i - 1) & 1], (uint32_t)(((i - 1) >> 1) & 1));
+            if (!ok) {
+                atomicExch(err, 1);
+                tc_commit(mfree + 8 * (g % kTcStages));   // the MMAs issued since the last commit
+                ++g;
+            }
+            // before the CTA ends: the last MMAs (bounded)
+            if (g > 0) tc_wait(mfree + 8 * ((g - 1) % kTcStages), (uint32_t)(((g - 1) / kTcStages) & 1));
         }
-    } else {
-        // epilogue warps: warp w owns tensor-memory lanes (tile rows) 32 w .. 32 w + 31
-        int i = 0;
-        for (int t = first; t < ntiles; t = tc_next(t + step, step, ntiles, n, base, base2, T, TJ, tcx), ++i) {
-            const int bsel = i & 1;
-            bool tri;
-            int ti, tj, r0, c0, climit;
-            tc_tile(t, n, base, base2, T, TJ, tcx, tri, ti, tj, r0, c0, climit);
-            float *C = tri ? A : X;
-            const int r = r0 + warp * 32 + lane;
-            float cv[2][32];
-            auto load_part = [&](float (&dst)[32], int part) {
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const int c = c0 + part * 32 + j;
-                    dst[j] = (r < n && c < climit && (!tri || r > c)) ? C[(size_t)c * ld + r] : 0.f;
-                }
-            };
-            load_part(cv[0], 0);   // while the MMAs run
-            if (!tc_wait(mfull[bsel], (uint32_t)((i >> 1) & 1))) {
-                if (lane == 0) atomicExch(err, 1);
-                break;
-            }
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t accrow = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(bsel * kTcN);
-#pragma unroll 2
-            for (int part = 0; part < kTcN / 32; ++part) {
-                if (part + 1 < kTcN / 32) load_part(cv[(part + 1) & 1], part + 1);
-                uint32_t v[32];
-                asm volatile(
-                    "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-                    "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-                    "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n"
-                    : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                      "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
-                      "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]),
-                      "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]),
-                      "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-                    : "r"(accrow + (uint32_t)(part * 32)));
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                if (r < n) {
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        const int c = c0 + part * 32 + j;
-                        if (c < climit && (!tri || r > c)) C[(size_t)c * ld + r] = cv[part & 1][j] - __uint_as_float(v[j]);
+    } else if (warp == kTcEpi + 1) {
+        if (lane == 0) {
+            bool ok = true;
+            int g = 0;   // stages requested
+            for (int t = (int)blockIdx.x; t < ntiles && ok; t += step) {
+                const TcTile q = tc_tile(t, n, base, base2, T, tcx);
+                for (int p = 0; p < 2 && ok; ++p) {
+                    const TcOps o = tc_ops(ops + p * tc_per_panel(n), n);
+                    const unsigned char *pa = (q.tri ? o.LDs : o.Ps) + (size_t)q.ti * kTcBlock;
+                    const unsigned char *pb = (q.tri ? o.Ps : o.Xs) + (size_t)q.tj * kTcBlock;
+                    for (int e = 0; e < kP / kTcK; ++e, ++g) {
+                        const uint32_t slot = (uint32_t)(g % kTcStages), mb = mload + 8 * slot;
+                        if (g >= kTcStages && !tc_wait(mfree + 8 * slot, (uint32_t)((g / kTcStages - 1) & 1))) { ok = false; break; }
+                        expect(mb, (uint32_t)kTcStage);
+                        copy(sbase + slot * kTcStage, pa + e * kTcOperand, (uint32_t)kTcOperand, mb);
+                        copy(sbase + slot * kTcStage + kTcOperand, pb + e * kTcOperand, (uint32_t)kTcOperand, mb);
                     }
                 }
             }
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            if (!ok) atomicExch(err, 1);
+            // before the CTA ends: its copies in flight (bounded)
+            for (int q = max(0, g - kTcStages); q < g; ++q) tc_wait(mload + 8 * (q % kTcStages), (uint32_t)((q / kTcStages) & 1));
+        }
+    } else {
+        // epilogue warps: warp w owns tensor-memory lanes (tile rows) 32 (w % 4) .. + 31 and columns
+        // kTcCols (w / 4) .. + kTcCols - 1
+        const int wrow = (warp & 3) * 32, wcol = (warp >> 2) * kTcCols;
+        float cv[kTcCols];
+        // this warp's part of a tile: first entry of row r and the columns it has an entry in
+        auto place = [&](int t, float *&C, int &live) {
+            const TcTile q = tc_tile(t, n, base, base2, T, tcx);
+            const int r = q.r0 + wrow + lane, c0 = q.c0 + wcol;
+            C = (q.tri ? A : X) + (size_t)c0 * ld + r;
+            live = r < n ? (q.tri ? min(q.climit, r) : q.climit) - c0 : 0;
+        };
+        auto fetch = [&](const float *C, int live, int j0) {
+#pragma unroll
+            for (int j = j0; j < j0 + 16; ++j) cv[j] = j < live ? C[(size_t)j * ld] : 0.f;
+        };
+        float *C = nullptr, *Cn = nullptr;
+        int live = 0, liven = 0, i = 0;
+        if ((int)blockIdx.x < ntiles) place((int)blockIdx.x, C, live);
+        fetch(C, live, 0);
+        fetch(C, live, 16);
+        for (int t = (int)blockIdx.x; t < ntiles; t += step, ++i) {
+            const int bsel = i & 1;
+            liven = 0;
+            if (t + step < ntiles) place(t + step, Cn, liven);
+            if (!__all_sync(0xffffffffu, tc_wait(mfull + 8 * bsel, (uint32_t)((i >> 1) & 1)))) {
+                if (lane == 0) atomicExch(err, 1);
+                break;
+            }
+            tc_fence_after();
+            const uint32_t acc = tmem + ((uint32_t)wrow << 16) + (uint32_t)(bsel * 2 * kTcM + wcol);
+#pragma unroll
+            for (int j0 = 0; j0 < kTcCols; j0 += 16) {
+                float u[16];
+                tc_ld16x2(acc + (uint32_t)j0, kTcM, u);   // first + second
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                    if (j0 + j < live) C[(size_t)(j0 + j) * ld] = cv[j0 + j] - u[j];
+                fetch(Cn, liven, j0);
+            }
+            tc_fence_before();
             __syncwarp();
-            if (lane == 0) tc_arrive(mempty[bsel]);
+            if (lane == 0) tc_arrive(mempty + 8 * bsel);
+            C = Cn;
+            live = liven;
         }
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    tc_fence_before();
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(2 * kTcN) : "memory");
+    tc_fence_after();
+    if (warp == 0) tc_dealloc(tmem, 4 * kTcM);
 }
 
 // partial sums of y = X r: CTA (rb, cb) covers rows [rb*256, +256) (four per thread, float4 loads)
@@ -1415,7 +1319,7 @@ Error d32_alloc(Dense32 &F, int32_t n) {
         attr_err = cudaFuncSetAttribute(d32_assemble_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)(sizeof(unsigned long long) * kSlice));
         if (attr_err == cudaSuccess)
-            attr_err = cudaFuncSetAttribute(d32_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStepSmem);
+            attr_err = cudaFuncSetAttribute(d32_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, step_smem(2));
     });
     if (attr_err != cudaSuccess) return fail(OT_ERR_CUDA, cudaGetErrorString(attr_err));
     if (n > kMaxN) return fail(OT_ERR_ARG, "dense32: n above the supported size");
@@ -1461,39 +1365,14 @@ struct Dag {
     int64_t nodes = 0;
     cudaError_t err = cudaSuccess;
     template <typename... Args>
-    cudaGraphNode_t kernel(std::vector<cudaGraphNode_t> deps, void (*fn)(Args...), unsigned grid, unsigned block,
-                           Args... args) {
+    cudaGraphNode_t kernel_grid(std::vector<cudaGraphNode_t> deps, void (*fn)(Args...), dim3 grid, unsigned block,
+                                unsigned smem, Args... args) {
         cudaGraphNode_t node = nullptr;
         if (err != cudaSuccess) return node;
         void *ptrs[] = {(void *)&args...};
         cudaKernelNodeParams kp = {};
         kp.func = (void *)fn;
-        kp.gridDim = dim3(grid);
-        kp.blockDim = dim3(block);
-        kp.sharedMemBytes = 0;
-        kp.kernelParams = ptrs;
-        kp.extra = nullptr;
-        deps.erase(std::remove(deps.begin(), deps.end(), nullptr), deps.end());
-        err = cudaGraphAddKernelNode(&node, g, deps.data(), deps.size(), &kp);
-        if (err == cudaSuccess) ++nodes;
-        return node;
-    }
-    // launch priority of a kernel node (stream-priority scale: lower values run first)
-    void priority(cudaGraphNode_t node, int value) {
-        if (err != cudaSuccess || !node) return;
-        cudaKernelNodeAttrValue v = {};
-        v.priority = value;
-        err = cudaGraphKernelNodeSetAttribute(node, cudaKernelNodeAttributePriority, &v);
-    }
-    template <typename... Args>
-    cudaGraphNode_t kernel_smem(std::vector<cudaGraphNode_t> deps, void (*fn)(Args...), unsigned grid,
-                                unsigned block, unsigned smem, Args... args) {
-        cudaGraphNode_t node = nullptr;
-        if (err != cudaSuccess) return node;
-        void *ptrs[] = {(void *)&args...};
-        cudaKernelNodeParams kp = {};
-        kp.func = (void *)fn;
-        kp.gridDim = dim3(grid);
+        kp.gridDim = grid;
         kp.blockDim = dim3(block);
         kp.sharedMemBytes = smem;
         kp.kernelParams = ptrs;
@@ -1502,6 +1381,18 @@ struct Dag {
         err = cudaGraphAddKernelNode(&node, g, deps.data(), deps.size(), &kp);
         if (err == cudaSuccess) ++nodes;
         return node;
+    }
+    template <typename... Args>
+    cudaGraphNode_t kernel(std::vector<cudaGraphNode_t> deps, void (*fn)(Args...), unsigned grid, unsigned block,
+                           Args... args) {
+        return kernel_grid(deps, fn, dim3(grid), block, 0u, args...);
+    }
+    // launch priority of a kernel node (stream-priority scale: lower values run first)
+    void priority(cudaGraphNode_t node, int value) {
+        if (err != cudaSuccess || !node) return;
+        cudaKernelNodeAttrValue v = {};
+        v.priority = value;
+        err = cudaGraphKernelNodeSetAttribute(node, cudaKernelNodeAttributePriority, &v);
     }
     cudaGraphNode_t memset0(float *dst, size_t count, std::vector<cudaGraphNode_t> deps) {
         cudaGraphNode_t node = nullptr;
@@ -1527,10 +1418,6 @@ struct Dag {
 };
 }  // namespace
 
-// split operand storage for one panel parity: two 128-row-block operands and two 64-row-block ones
-static size_t tc_a_floats(int n) { return (size_t)ceil_div(n, kTcM) * 2 * kTcM * kP; }
-static size_t tc_b_floats(int n) { return (size_t)ceil_div(n, kTcN) * 2 * kTcN * kP; }
-static size_t tc_per_parity(int n) { return 2 * tc_a_floats(n) + 2 * tc_b_floats(n); }
 static Error d32_build(Dense32 &F, float eps, cudaGraph_t g, int64_t *nodes) {
     const int n = F.n, ld = F.ld;
     Dag c;
@@ -1541,38 +1428,57 @@ static Error d32_build(Dense32 &F, float eps, cudaGraph_t g, int64_t *nodes) {
     int sms = 0, dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         sms = 1;
-    if (!F.use_tc) {
-        // SIMT: the first diagonal block, then one fused step per panel (which also factors the next
-        // diagonal block) on the chain, the rest of each panel's update (from base + 128) beside
-        // it.  The step of panel p waits for the rest-update of panel p - 2 (which covered its
-        // columns); the rest-updates run in order.  Three LD buffers: the rest-update of panel p
-        // still reads its own while the steps of p + 1 and p + 2 write theirs.
-        const int bs0 = std::min(kP, n);
-        prev = c.kernel({prev}, d32_colsum_kernel, (unsigned)bs0, kTT, n, ld, bs0, (const float *)F.A, F.csum);
-        cudaGraphNode_t chain = c.kernel({prev}, d32_diag_kernel, 1u, kTT, ld, 0, bs0, F.A, F.D, (const float *)F.d0,
-                                         (const float *)F.csum, 1, 1, eps, F.Linv, (const float *)nullptr);
-        c.priority(chain, hi_prio);
-        cudaGraphNode_t rest1 = nullptr, rest2 = nullptr;   // rest-updates of panels p - 1 and p - 2
-        int k = 0, p = 0;
-        for (; k + kP < n; k += kP, ++p) {
-            const int base = k + kP;
-            const int ts = (int)ceil_div(n - base, kP), tx = (int)ceil_div(base, kP);
-            float *LDc = F.LD + (size_t)(p % 3) * ld * kP;
-            const float *LDprev = F.LD + (size_t)((p + 2) % 3) * ld * kP;
-            const cudaGraphNode_t sn =
-                c.kernel_smem({chain, rest2}, d32_step_kernel, (unsigned)(2 * (ts + tx)), kTT, (unsigned)kStepSmem, n, ld,
-                              k, F.A, F.X, (const float *)F.D, (const float *)F.Linv, LDc, LDprev, F.L0, F.csum);
-            c.priority(sn, hi_prio);
-            const cudaGraphNode_t dn =
-                c.kernel({sn}, d32_diag_kernel, 1u, kTT, ld, base, std::min(kP, n - base), F.A, F.D,
-                         (const float *)F.d0, (const float *)F.csum, ts, 2, eps, F.Linv, (const float *)F.L0);
-            c.priority(dn, hi_prio);
-            const int b2 = base + 2 * kP;
+    // The first diagonal block, then one fused step and the next diagonal block per panel on the chain,
+    // the rest of the updates beside it and in order.  SIMT: one rest-update per panel, which the
+    // step two panels on waits for (it covered its columns).  Tensor cores: one per two panels p, p + 1
+    // (p even), from block p + 4 on, which step p + 3 waits for; their operands are split behind step
+    // p + 1 into buffers that alternate (the rest-update before may still read the other).  Three LD
+    // buffers: a rest-update (or split) still reads its panels' while the next steps write theirs.
+    const int bs0 = std::min(kP, n);
+    prev = c.kernel({prev}, d32_colsum_kernel, (unsigned)bs0, kTT, n, ld, bs0, (const float *)F.A, F.csum);
+    cudaGraphNode_t chain = c.kernel({prev}, d32_diag_kernel, 1u, kTT, ld, 0, bs0, F.A, F.D, (const float *)F.d0,
+                                     (const float *)F.csum, 1, 1, eps, F.Linv, (const float *)nullptr);
+    c.priority(chain, hi_prio);
+    cudaGraphNode_t rest1 = nullptr, rest2 = nullptr;   // the newest rest-update and the one before
+    int k = 0, p = 0;
+    for (; k + kP < n; k += kP, ++p) {
+        const int base = k + kP;
+        const int ts = (int)ceil_div(n - base, kP), tx = (int)ceil_div(base, kP);
+        float *LDc = F.LD + (size_t)(p % 3) * ld * kP;
+        float *LDprev = F.LD + (size_t)((p + 2) % 3) * ld * kP, *LDprev2 = F.LD + (size_t)((p + 1) % 3) * ld * kP;
+        const int npv = std::min(p, F.use_tc && p % 2 == 0 ? 2 : 1);
+        // the rest-update that covered this step's columns last
+        const cudaGraphNode_t wait = !F.use_tc ? rest2 : p % 2 == 1 ? rest1 : nullptr;
+        const cudaGraphNode_t sn =
+            c.kernel_grid({chain, wait}, d32_step_kernel, dim3(2 * (ts + tx)), kTT, (unsigned)step_smem(npv), n, ld,
+                          k, npv, F.A, F.X, (const float *)F.D, (const float *)F.Linv, LDc, (const float *)LDprev,
+                          (const float *)LDprev2, F.L0, F.csum);
+        c.priority(sn, hi_prio);
+        const cudaGraphNode_t dn =
+            c.kernel({sn}, d32_diag_kernel, 1u, kTT, ld, base, std::min(kP, n - base), F.A, F.D,
+                     (const float *)F.d0, (const float *)F.csum, ts, 2, eps, F.Linv, (const float *)F.L0);
+        c.priority(dn, hi_prio);
+        const int b2 = base + 2 * kP;
+        cudaGraphNode_t rest = nullptr;
+        if (F.use_tc) {
+            if (p % 2 == 1 && b2 < n) {
+                const int T = (int)ceil_div(n - b2, kTcM), nx = (int)ceil_div(base, kTcM);
+                unsigned char *buf = F.tc + (size_t)((p / 2) & 1) * 2 * tc_per_panel(n);
+                const cudaGraphNode_t sp =
+                    c.kernel_grid({sn}, d32_tc_split_kernel, dim3(T + nx, 2), kTT, 0u, n, ld, k - kP, b2, T,
+                                  (const float *)F.A, (const float *)F.X, (const float *)LDprev, (const float *)LDc, buf);
+                c.priority(sp, lo_prio);
+                const int tiles = T * (T + 1) / 2 + T * nx;   // persistent CTAs: one per SM at most
+                rest = c.kernel_grid({sp, rest1}, d32_tc_update_kernel, dim3(std::min(tiles, sms)), kTcThreads,
+                                     (unsigned)kTcSmem, n, ld, base, b2, T, buf, F.A, F.X, F.tc_err);
+                c.priority(rest, lo_prio);
+                rest1 = rest;
+            }
+        } else {
             const int t2 = b2 < n ? (int)ceil_div(n - b2, kTile) : 0, tcn = (int)ceil_div(base, kTile);
             const int n2 = t2 * (t2 + 1) / 2 + t2 * tcn;
-            cudaGraphNode_t rest = nullptr;
             if (n2 > 0) {
-                rest = c.kernel({sn, rest1}, d32_update_kernel, (unsigned)n2, kTT, n, ld, k, 2, F.A, F.X,
+                rest = c.kernel({sn, rest1}, d32_update_kernel, (unsigned)n2, kTT, n, ld, k, F.A, F.X,
                                 (const float *)LDc);
                 c.priority(rest, lo_prio);
             } else {
@@ -1580,73 +1486,16 @@ static Error d32_build(Dense32 &F, float eps, cudaGraph_t g, int64_t *nodes) {
             }
             rest2 = rest1;
             rest1 = rest;
-            chain = dn;
         }
-        // the last panel: its diagonal block came with the last step (or is the first block); its
-        // block row of L^-1, then the end of the graph after all writes
-        const int bs = n - k;
-        const cudaGraphNode_t ir = c.kernel({chain}, d32_invrow_kernel, (unsigned)ceil_div(n, kP), kTT, ld, k, bs,
-                                            F.X, (const float *)F.Linv);
-        c.priority(ir, hi_prio);
-        prev = c.join({ir, rest1, rest2});
-    } else {
-    // tensor cores: per panel diag -> panel / invrow -> first update part (the next panel's block) on
-    // the chain, the bulk update of the rest beside it (the next panel's first part waits for it)
-    cudaGraphNode_t u1 = nullptr, u2 = nullptr;
-    int np = 1;  // partial column sums feeding the next diagonal block
-    for (int k = 0, p = 0; k < n; k += kP, ++p) {
-        const int bs = std::min(kP, n - k), base = k + bs;
-        float *LDp = F.LD + (size_t)(p % 3) * ld * kP;
-        if (k == 0) prev = c.kernel({prev}, d32_colsum_kernel, (unsigned)bs, kTT, n, ld, bs, (const float *)F.A, F.csum);
-        const cudaGraphNode_t dg = c.kernel({k == 0 ? prev : u1}, d32_diag_kernel, 1u, kTT, ld, k, bs, F.A, F.D,
-                                            (const float *)F.d0, (const float *)F.csum, np, 1, eps, F.Linv,
-                                            (const float *)nullptr);
-        c.priority(dg, hi_prio);
-        std::vector<cudaGraphNode_t> ready;
-        if (base < n)
-            ready.push_back(c.kernel({dg}, d32_panel_kernel, (unsigned)ceil_div(n - base, kP), kTT, n, ld, k, F.A,
-                                     (const float *)F.D, (const float *)F.Linv, LDp));
-        ready.push_back(c.kernel({dg}, d32_invrow_kernel, (unsigned)ceil_div(base, kP), kTT, ld, k, bs, F.X,
-                                 (const float *)F.Linv));
-        for (cudaGraphNode_t r : ready) c.priority(r, hi_prio);
-        if (u2) ready.push_back(u2);
-        if (base >= n) {
-            // the last panel: join everything so the graph ends after all writes
-            prev = c.join(ready);
-            break;
-        }
-        const int ts = (int)ceil_div(n - base, kP), tx = (int)ceil_div(base, kP);
-        np = ts;
-        u1 = c.kernel(ready, d32_update1_kernel, (unsigned)(ts + tx), kTT, n, ld, k, F.A, F.X, (const float *)LDp,
-                      F.csum);
-        c.priority(u1, hi_prio);
-        const int base2 = base + kP;
-        u2 = nullptr;
-        if (base2 < n) {
-            // the operands of this panel's bulk update split for the tensor cores (buffers by panel
-            // parity: the previous panel's update may still read the other half)
-            const int T = (int)ceil_div(n - base2, kTcM), nb = (int)ceil_div(n - base2, kTcN);
-            const int nx = (int)ceil_div(base, kTcN);
-            float *LDs = F.tc + (size_t)(p & 1) * tc_per_parity(n);
-            float *PAs = LDs + tc_a_floats(n), *PBs = PAs + tc_a_floats(n), *XBs = PBs + tc_b_floats(n);
-            const float *panel = F.A + (size_t)k * ld;
-            std::vector<cudaGraphNode_t> sp;
-            sp.push_back(c.kernel(ready, d32_tc_split_kernel<kTcM, false>, (unsigned)T, kTT, n, ld, (const float *)LDp,
-                                  base2, LDs));
-            sp.push_back(c.kernel(ready, d32_tc_split_kernel<kTcN, false>, (unsigned)nb, kTT, n, ld, panel, base2, PBs));
-            sp.push_back(c.kernel(ready, d32_tc_split_kernel<kTcM, false>, (unsigned)T, kTT, n, ld, panel, base2, PAs));
-            sp.push_back(c.kernel(ready, d32_tc_split_kernel<kTcN, true>, (unsigned)nx, kTT, base, ld,
-                                  (const float *)(F.X + k), 0, XBs));
-            for (cudaGraphNode_t q : sp) c.priority(q, lo_prio);
-            const int TJ = (int)ceil_div(T * kTcM, kTcN);
-            const int tiles = T * TJ + T * nx;   // persistent CTAs: one per SM at most
-            u2 = c.kernel_smem(sp, d32_tc_update_kernel, (unsigned)std::max(1, std::min(tiles, sms)), kTcThreads,
-                               (unsigned)kTcSmem, n, ld, base, base2, T, (const float *)LDs, (const float *)PBs,
-                               (const float *)PAs, (const float *)XBs, F.A, F.X, F.tc_err);
-            c.priority(u2, lo_prio);
-        }
+        chain = dn;
     }
-    }
+    // the last panel: its diagonal block came with the last step (or is the first block); its
+    // block row of L^-1, then the end of the graph after all writes
+    const int bs = n - k;
+    const cudaGraphNode_t ir = c.kernel({chain}, d32_invrow_kernel, (unsigned)ceil_div(n, kP), kTT, ld, k, bs,
+                                        F.X, (const float *)F.Linv);
+    c.priority(ir, hi_prio);
+    c.join({ir, rest1, rest2});
     if (c.err != cudaSuccess) return fail(OT_ERR_CUDA, cudaGetErrorString(c.err));
     *nodes = c.nodes;
     return ok();
@@ -1658,7 +1507,7 @@ Error d32_factor(Dense32 &F, float eps, cudaStream_t st) {
     if (!F.graph || F.eps != eps) {
         const bool want_tc = F.tc_mode > 0 || (F.tc_mode == 0 && F.n >= kTcAutoN);
         if (want_tc && !F.tc) {
-            OT_CUDA(cudaMalloc((void **)&F.tc, sizeof(float) * 2 * tc_per_parity(F.n)));
+            OT_CUDA(cudaMalloc((void **)&F.tc, 4 * tc_per_panel(F.n)));
             OT_CUDA(cudaMalloc((void **)&F.tc_err, sizeof(int)));
             OT_CUDA(cudaMemset(F.tc_err, 0, sizeof(int)));
             OT_CUDA(cudaMallocHost((void **)&F.tc_err_host, sizeof(int)));

@@ -32,12 +32,12 @@ struct Dense32 {
     float eps = 0.f;
     cudaGraphExec_t graph = nullptr;  // the factorisation's launch sequence for this n
     int64_t graph_nodes = 0;
-    // bulk update on the tensor cores (split TF32, tcgen05): tc_mode 1 = on, -1 = the FP32 SIMT
-    // update, 0 = on from n = 8192 (read when the launch sequence is built); split operands,
-    // double-buffered by panel
+    // rest-update on the tensor cores (three BF16 pieces per operand, tcgen05): tc_mode 1 = on, -1 = the
+    // FP32 SIMT update, 0 = on from n = 8192 (read when the launch sequence is built); split operands
+    // of two panels, double-buffered
     int tc_mode = 0;
     bool use_tc = false;
-    float *tc = nullptr;
+    unsigned char *tc = nullptr;
     int *tc_err = nullptr;      // a bounded wait of the tensor-core update gave up (device)
     int *tc_err_host = nullptr; // pinned copy, read at the next factorisation
 };

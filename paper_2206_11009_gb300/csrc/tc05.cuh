@@ -125,4 +125,22 @@ __device__ __forceinline__ void tc_ld8(uint32_t taddr, float (&out)[8]) {
     for (int j = 0; j < 8; ++j) out[j] = __uint_as_float(v[j]);
 }
 
+// the sums of 16 columns of two accumulators `apart` columns from one another: two reads, one wait
+__device__ __forceinline__ void tc_ld16x2(uint32_t t, uint32_t apart, float (&out)[16]) {
+    uint32_t v[2][16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, "
+        "%8, %9, %10, %11, %12, %13, %14, %15}, [%32];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16, %17, %18, %19, %20, %21, %22, %23, "
+        "%24, %25, %26, %27, %28, %29, %30, %31}, [%33];\n"
+        "tcgen05.wait::ld.sync.aligned;"
+                 : "=&r"(v[0][0]), "=&r"(v[0][1]), "=&r"(v[0][2]), "=&r"(v[0][3]), "=&r"(v[0][4]), "=&r"(v[0][5]), "=&r"(v[0][6]), "=&r"(v[0][7]),
+                   "=&r"(v[0][8]), "=&r"(v[0][9]), "=&r"(v[0][10]), "=&r"(v[0][11]), "=&r"(v[0][12]), "=&r"(v[0][13]), "=&r"(v[0][14]), "=&r"(v[0][15]),
+                   "=&r"(v[1][0]), "=&r"(v[1][1]), "=&r"(v[1][2]), "=&r"(v[1][3]), "=&r"(v[1][4]), "=&r"(v[1][5]), "=&r"(v[1][6]), "=&r"(v[1][7]),
+                   "=&r"(v[1][8]), "=&r"(v[1][9]), "=&r"(v[1][10]), "=&r"(v[1][11]), "=&r"(v[1][12]), "=&r"(v[1][13]), "=&r"(v[1][14]), "=&r"(v[1][15])
+                 : "r"(t), "r"(t + apart) : "memory");
+#pragma unroll
+    for (int j = 0; j < 16; ++j) out[j] = __uint_as_float(v[0][j]) + __uint_as_float(v[1][j]);
+}
+
 }  // namespace ot
