@@ -510,7 +510,13 @@ __device__ __forceinline__ void tri_decode(int idx, int &ti, int &tj) {
     tj = idx - ti * (ti + 1) / 2;
 }
 
-// the rest of the update of panel k, from base2 = base + 128 on
+// the rest of the update of panel k, from base2 = base + 128 on.  Launched with kRestPad bytes of shared
+// memory that it does not use, which halves an SM's room beside its CTAs: factorisations of n = 4096 take
+// 2737 us instead of 2935 and of n = 6400 7.61 ms instead of 7.81 (50 to 60 KB alike, 84 KB leaves one CTA per
+// SM: 3228; n = 2025 takes 1063 us either way).  Registers already keep a third CTA off the SM, and
+// asking for the same carve-out without the bytes does not do it (2936), so how it favours the chain is not
+// explained.
+constexpr int kRestPad = 52 * 1024;
 __global__ void __launch_bounds__(kTT, 2)
 d32_update_kernel(int n, int ld, int k, float *__restrict__ A, float *__restrict__ X,
                   const float *__restrict__ LD) {
@@ -1319,6 +1325,8 @@ Error d32_alloc(Dense32 &F, int32_t n) {
         attr_err = cudaFuncSetAttribute(d32_assemble_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)(sizeof(unsigned long long) * kSlice));
         if (attr_err == cudaSuccess)
+            attr_err = cudaFuncSetAttribute(d32_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRestPad);
+        if (attr_err == cudaSuccess)
             attr_err = cudaFuncSetAttribute(d32_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, step_smem(2));
     });
     if (attr_err != cudaSuccess) return fail(OT_ERR_CUDA, cudaGetErrorString(attr_err));
@@ -1478,8 +1486,8 @@ static Error d32_build(Dense32 &F, float eps, cudaGraph_t g, int64_t *nodes) {
             const int t2 = b2 < n ? (int)ceil_div(n - b2, kTile) : 0, tcn = (int)ceil_div(base, kTile);
             const int n2 = t2 * (t2 + 1) / 2 + t2 * tcn;
             if (n2 > 0) {
-                rest = c.kernel({sn, rest1}, d32_update_kernel, (unsigned)n2, kTT, n, ld, k, F.A, F.X,
-                                (const float *)LDc);
+                rest = c.kernel_grid({sn, rest1}, d32_update_kernel, dim3(n2), kTT, (unsigned)kRestPad, n, ld, k, F.A, F.X,
+                                     (const float *)LDc);
                 c.priority(rest, lo_prio);
             } else {
                 rest = c.join({sn, rest1});
