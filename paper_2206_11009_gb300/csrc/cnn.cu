@@ -8,10 +8,11 @@
 // that a tile's im2col operand is 16-byte copies; pre-normalisation outputs z in FP32, four channels of
 // a pixel together in blocks of 128 pixels (zoff), so that a thread per pixel reads and writes whole
 // lines.  Weights are kept in FP32 (Adam's master copy) with BF16 copies for the convolutions.
-// The convolutions from 32 channels (forward, data and weight gradients) are implicit GEMMs on the
+// The convolutions from 32 channels (forward, data and weight gradients; of the head the
+// weight gradient) are implicit GEMMs on the
 // tensor cores, with the bias, the normalisation, its backward and the sums of the bias and gain
-// gradients in their epilogues; the 2 -> 32 convolution and the gradients around the two 2-channel
-// ends run on the FP32 pipes.  Every reduction runs in a fixed order (per-CTA partials, one pass).
+// gradients in their epilogues; the 2 -> 32 convolution, the head and the data gradients around the two
+// 2-channel ends run on the FP32 pipes.  Every reduction runs in a fixed order (per-CTA partials, one pass).
 #include <cuda_bf16.h>
 
 #include <cmath>
@@ -81,13 +82,15 @@ __device__ __forceinline__ void norm_fwd8(int64_t p, int q, float ss, const floa
     st_bf16x8(h + p * 32 + 8 * q, o);
 }
 
-// dh -> dz of eight of a pixel's channels through silu and the RMS normalisation, the pixel's dot product
-// over its four threads through sdot[4][128] (called by all threads of the CTA; others' pixels with
-// valid = false); dgl: the part of the gain's gradient.
+// dh -> dz of eight of a pixel's channels through silu and the RMS normalisation (called by all threads
+// of the CTA; others' pixels with valid = false); dgl: the part of the gain's gradient.  The pixel's dot
+// product runs through its four threads in the order of the channels (sdot[4][128]): dz is rounded to BF16,
+// and other orders turn roundings over that three layers' gradients then carry (four partial sums added:
+// 1e-5 of the gradient at 21x21 x 5).
 __device__ __forceinline__ void norm_bwd8(bool valid, int64_t p, int row, int q, float (&dh)[8],
                                           const float *__restrict__ zb, const float *__restrict__ r, const float *g,
                                           float (&dgl)[8], float (*sdot)[kPix]) {
-    float dot = 0.f, rr = 1.f;
+    float rr = 1.f;
     float xh[8] = {};
     if (valid) {
         rr = r[p];
@@ -103,11 +106,17 @@ __device__ __forceinline__ void norm_bwd8(bool valid, int64_t p, int row, int q,
         const float dyn = dh[c] * (s + yn * s * (1.f - s));
         dgl[c] = dyn * xh[c];
         dh[c] = dyn * g[8 * q + c];
-        dot += dh[c] * xh[c];
     }
-    sdot[q][row] = dot;
-    __syncthreads();
-    dot = ((sdot[0][row] + sdot[1][row]) + (sdot[2][row] + sdot[3][row])) / 32;
+    for (int k = 0; k < 4; ++k) {
+        if (q == k) {
+            float d = k ? sdot[k - 1][row] : 0.f;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) d += dh[c] * xh[c];
+            sdot[k][row] = d;
+        }
+        __syncthreads();
+    }
+    const float dot = sdot[3][row] / 32;
 #pragma unroll
     for (int c = 0; c < 8; ++c) dh[c] = (dh[c] - xh[c] * dot) / rr;
 }
@@ -193,6 +202,67 @@ block0_kernel(int B, int H, int Wd, int dil, const float *__restrict__ x, const 
 #pragma unroll
     for (int c = 0; c < 32; ++c) ss += sz[row][c] * sz[row][c];
     norm_fwd8(p, q, ss, acc, sg, zb, r, h);
+}
+
+// Head: y[o] = bias[o] + sum_{c, t} W[o, c, t] h[pixel + offset_t, c], a thread per pixel, channels outermost.
+// Its last bits decide BF16 roundings throughout the backward pass, so the sum keeps one FP32 chain in
+// this order (as MMAs with eight partial sums it gave gradients up to 5e-5 apart).  A
+// pixel's channels lie together: nine 16-byte loads for eight channels, the next nine already in flight.
+// Latency-bound, a chain of 288 multiply-adds per output; 64x64 x 16: 35 -> 11.6 us (as MMAs 12).
+constexpr int kHdThr = 64;
+__global__ void __launch_bounds__(kHdThr)
+head_kernel(int B, int H, int Wd, int dil, const __nv_bfloat16 *__restrict__ h, const __nv_bfloat16 *__restrict__ w,
+            const float *__restrict__ bias, float *__restrict__ out, float *__restrict__ out2) {
+    __shared__ __align__(16) float2 ws[32 * 9];   // [c][t] of both outputs
+    pdl_start();
+    for (int q = threadIdx.x; q < 32 * 9; q += kHdThr)
+        ws[q] = make_float2(__bfloat162float(w[q]), __bfloat162float(w[32 * 9 + q]));
+    __syncthreads();
+    pdl_wait();
+    const int HW = H * Wd;
+    const int64_t p = (int64_t)blockIdx.x * kHdThr + threadIdx.x;
+    if (p >= (int64_t)B * HW) return;
+    const int yx = (int)(p % HW), y = yx / Wd, x = yx % Wd;
+    const __nv_bfloat16 *src = h + p * 32;
+    int off[9];
+    unsigned in = 0;
+#pragma unroll
+    for (int t = 0; t < 9; ++t) {
+        const int dy = (t / 3 - 1) * dil, dx = (t % 3 - 1) * dil;
+        off[t] = (dy * Wd + dx) * 32;
+        if (y + dy >= 0 && y + dy < H && x + dx >= 0 && x + dx < Wd) in |= 1u << t;
+    }
+    uint4 nxt[9], cur[9];
+    auto load = [&](int c0) {
+#pragma unroll
+        for (int t = 0; t < 9; ++t)
+            nxt[t] = in >> t & 1 ? *(const uint4 *)(src + off[t] + c0) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    float a0 = bias[0], a1 = bias[1];
+    load(0);
+#pragma unroll 1
+    for (int c0 = 0; c0 < 32; c0 += 8) {
+#pragma unroll
+        for (int t = 0; t < 9; ++t) cur[t] = nxt[t];
+        if (c0 < 24) load(c0 + 8);
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+#pragma unroll
+            for (int t = 0; t < 9; ++t) {
+                const uint32_t u = e < 2 ? cur[t].x : e < 4 ? cur[t].y : e < 6 ? cur[t].z : cur[t].w;
+                const float v = __uint_as_float(e & 1 ? u & 0xffff0000u : u << 16);
+                const float2 wv = ws[(c0 + e) * 9 + t];
+                a0 += v * wv.x;
+                a1 += v * wv.y;
+            }
+    }
+    const int64_t at = (p / HW) * 2 * HW + yx;
+    out[at] = a0;
+    out[at + HW] = a1;
+    if (out2) {
+        out2[at] = a0;
+        out2[at + HW] = a1;
+    }
 }
 
 // Head's data gradient dh[c] = sum_{o, t} W[o, c, t] dy[o, y - oy_t, x - ox_t], then the last block's
@@ -345,8 +415,8 @@ block0_wgrad_kernel(int B, int H, int Wd, int dil, const __nv_bfloat16 *__restri
 // the MMAs.  No swizzle: core matrices of 8 rows x 8 BF16 (16 bytes), element (row, k) of an R-row
 // operand in core matrix (row / 8, k / 8) at byte ((k / 8)(R / 8) + row / 8) 128, its row row % 8 at
 // 16-byte steps.  A tile's im2col operand has 128 pixels as rows and k = 32 tap + channel (288):
-//   conv:   D[pixel, o] = sum_k A[pixel, k] Wop[o, k], both K-major: M = 128, N = 32 (the head:
-//           N = 16), K = 288 (18 MMAs).  The data gradient is the same product over the output gradient with
+//   conv:   D[pixel, o] = sum_k A[pixel, k] Wop[o, k], both K-major: M = 128, N = 32, K = 288
+//           (18 MMAs).  The data gradient is the same product over the output gradient with
 //           the taps mirrored.
 //   wgrad:  D[k, o] = sum_pixel A[pixel, k] dz[pixel, o]: the same A read MN-major (channels contiguous,
 //           pixels as depth), dz likewise: M = 128 at rows 0, 128 and 160 of the 288, K = 128 pixels
@@ -354,17 +424,16 @@ block0_wgrad_kernel(int B, int H, int Wd, int dil, const __nv_bfloat16 *__restri
 // The operand is copied by the CTA's threads, 16 bytes of a neighbour pixel at a time (36 copies per
 // pixel, zero-filled outside the image): with one channel plane after another it took 288 two-byte
 // loads per pixel and bound both kernels.  Device times at 64x64 x 16 (65,536 pixels), before -> now: convolution
-// and normalisation 26.5 + 8 -> 15.0 us, data gradient and normalisation backward 26.5 + 25 -> 18.5, weight
-// gradient 95 -> 13.6 (head: 49 -> 11.9), the head forward 35 -> 12, sums of the partials 381 -> 12.  At these
+// and normalisation 26.5 + 8 -> 15.0 us, data gradient and normalisation backward 26.5 + 25 -> 18.7, weight
+// gradient 95 -> 13.6 (head: 49 -> 11.9), sums of the partials 381 -> 12.  At these
 // sizes neither memory (12 MB per convolution) nor the tensor cores bound them but one tile's chain of copies,
 // MMAs, read-back and epilogue, twice (512 tiles on 304 resident CTAs).
 constexpr int kCvM = 128, kCvK = 9 * 32;
 constexpr int kCvAbytes = kCvM * kCvK * 2;     // 73,728
-constexpr int kCvSlot = 32 * kCvK;             // elements of one layer's weight operand (the head's: 16 rows)
+constexpr int kCvSlot = 32 * kCvK;             // elements of one layer's weight operand
 constexpr int kWgStride = kCvK * 32;           // one CTA's partial of a weight gradient
 
-template <int N>
-constexpr int cv_smem() { return kCvAbytes + N * kCvK * 2 + 32; }
+constexpr int kCvSmem = kCvAbytes + 32 * kCvK * 2 + 32;
 template <int N>
 constexpr int wg_smem() { return kCvAbytes + kCvM * N * 2 + 32; }
 
@@ -409,27 +478,20 @@ __device__ __forceinline__ void copies_visible() {   // to the MMAs (async proxy
 // Where parameter j of a layer goes among the convolution operands: BF16 copy and, for a layer with 32
 // inputs, its places in the forward operand (Wop[o, 32 t + c] = W[o, c, t]) and the mirrored one of the
 // data gradient (Wop'[c, 32 t + o] = W[o, c, 8 - t]); operand (layer l, mirrored f) at wop + (2 (l - 1) + f)
-// kCvSlot.  The head's at slot 6: output o's weights are spread over rows 8 o .. 8 o + 7 (zeros elsewhere),
-// the 16 depths of MMA ks in row 8 o + ks % 8, so that a column sums two or three MMAs and the eight are added
-// in FP32.  Relative L2 error of the prediction against FP64 from the same inputs, 64x64: 1.2e-7 with FP32
-// FMAs in a thread, 2.7e-7 with all 18 MMAs on one column, 7.3e-8 so.
-struct WopMap { int64_t off[4]; };   // W offsets of layers 1 .. 4
+// kCvSlot.
+struct WopMap { int64_t off[3]; };   // W offsets of layers 1 .. 3
 
 __device__ __forceinline__ void place_param(int64_t j, float v, const WopMap &mp, __nv_bfloat16 *__restrict__ wb,
                                             __nv_bfloat16 *__restrict__ wop) {
     const __nv_bfloat16 b = __float2bfloat16(v);
     wb[j] = b;
 #pragma unroll
-    for (int l = 0; l < 4; ++l) {
+    for (int l = 0; l < 3; ++l) {
         const int64_t e = j - mp.off[l];
-        if (e < 0 || e >= (l < 3 ? 32 * 288 : 2 * 288)) continue;
+        if (e < 0 || e >= 32 * 288) continue;
         const int o = (int)(e / 288), c = (int)(e % 288) / 9, t = (int)(e % 9);
-        if (l < 3) {
-            wop[(int64_t)(2 * l) * kCvSlot + cv_off(o, t * 32 + c, 32) / 2] = b;
-            wop[(int64_t)(2 * l + 1) * kCvSlot + cv_off(c, (8 - t) * 32 + o, 32) / 2] = b;
-        } else {
-            wop[(int64_t)6 * kCvSlot + cv_off(8 * o + (2 * t + c / 16) % 8, t * 32 + c, 16) / 2] = b;
-        }
+        wop[(int64_t)(2 * l) * kCvSlot + cv_off(o, t * 32 + c, 32) / 2] = b;
+        wop[(int64_t)(2 * l + 1) * kCvSlot + cv_off(c, (8 - t) * 32 + o, 32) / 2] = b;
     }
 }
 
@@ -444,10 +506,9 @@ struct ConvIo {
     float *z, *r;                 // forward: written; data gradient: the block before's, read
     __nv_bfloat16 *h;             // forward: the next layer's input; data gradient: dz in BF16 (or NULL)
     float *dz32;                  // data gradient: dz in FP32, z layout (or NULL)
-    float *y, *y2;                // head: prediction NCHW (y2 may be NULL)
     float *part;                  // data gradient: rows of kSumRow
 };
-enum { CV_BLOCK, CV_HEAD, CV_GRAD };
+enum { CV_BLOCK, CV_GRAD };
 
 // A 3x3 convolution from 32 channels over `in` and what follows it on the same pixel.  Persistent CTAs
 // of 512 threads take 128-pixel tiles gridDim.x apart; all copy the operand, thread 0 issues the 18 MMAs
@@ -458,7 +519,7 @@ template <int MODE>
 __global__ void __launch_bounds__(kThr, 2)
 conv_tc_kernel(int B, int H, int Wd, int dil, const __nv_bfloat16 *__restrict__ in,
                const __nv_bfloat16 *__restrict__ wop, ConvIo io, int *__restrict__ err) {
-    constexpr int N = MODE == CV_HEAD ? 16 : 32, Bbytes = N * kCvK * 2;
+    constexpr int N = 32, Bbytes = N * kCvK * 2;
     constexpr uint32_t idesc = tc_idesc(1u, kCvM, N);
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ float sh[16][16], sdot[4][kPix], sg[32], sbias[32];
@@ -478,9 +539,9 @@ conv_tc_kernel(int B, int H, int Wd, int dil, const __nv_bfloat16 *__restrict__ 
     pdl_wait();
     gather_tile(a0, (int64_t)blockIdx.x * kCvM, P, H, Wd, dil, in, 0, nullptr);
     for (int e = threadIdx.x; e < Bbytes / 16; e += kThr) copy16(b0 + 16 * e, (const uint4 *)wop + e, true);
-    if (threadIdx.x < (MODE == CV_HEAD ? 2 : 32)) {
+    if (threadIdx.x < 32) {
         if (MODE != CV_GRAD) sbias[threadIdx.x] = io.bias[threadIdx.x];
-        if (MODE != CV_HEAD) sg[threadIdx.x] = io.gain[threadIdx.x];
+        sg[threadIdx.x] = io.gain[threadIdx.x];
     }
     tc_fence_before();
     __syncthreads();
@@ -527,17 +588,6 @@ conv_tc_kernel(int B, int H, int Wd, int dil, const __nv_bfloat16 *__restrict__ 
 #pragma unroll
             for (int c = 0; c < 8; ++c) z[c] = sbias[8 * q + c] + z[c];
             if (valid) norm_fwd8(pix, q, ss, z, sg, io.z, io.r, io.h);
-        } else if constexpr (MODE == CV_HEAD) {
-            if (q < 2) {   // output q
-                float v[8];
-                tc_ld8(trow + 8 * q, v);
-                if (valid) {
-                    const float yo = sbias[q] + (((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7])));
-                    const int64_t at = ((pix / HW) * 2 + q) * HW + pix % HW;
-                    io.y[at] = yo;
-                    if (io.y2) io.y2[at] = yo;
-                }
-            }
         } else {
             float v[8], dgl[8];
             tc_ld8(trow + 8 * q, v);
@@ -812,7 +862,7 @@ struct ot_cnn {
     cudaStream_t st = nullptr;
     float *w = nullptr, *m = nullptr, *v = nullptr;   // FP32 master weights and Adam moments
     __nv_bfloat16 *wb = nullptr;                      // BF16 copy
-    __nv_bfloat16 *wop = nullptr;   // tensor-core weight operands of layers 1-3 (forward, mirrored) and 4
+    __nv_bfloat16 *wop = nullptr;   // tensor-core weight operands of layers 1-3 (forward, mirrored)
     // pinned host memory that the kernels write, read after a synchronisation (a copy into pageable memory
     // took longer than a small image's kernels): flag of a tensor-core wait that gave up, loss per image
     int *derr = nullptr;
@@ -922,7 +972,7 @@ int ensure_grads(ot_cnn *c) {
 
 WopMap wop_map(const ot_cnn *c) {
     WopMap m;
-    for (int l = 0; l < 4; ++l) m.off[l] = c->L[l + 1].W;
+    for (int l = 0; l < 3; ++l) m.off[l] = c->L[l + 1].W;
     return m;
 }
 
@@ -934,7 +984,7 @@ int place_params(ot_cnn *c) {
     return OT_OK;
 }
 
-// weight operand of layer l: forward (1 .. 4) or mirrored (1 .. 3)
+// weight operand of layer l = 1 .. 3, forward or mirrored
 const __nv_bfloat16 *wop_of(const ot_cnn *c, int l, int mirrored) {
     return c->wop + (int64_t)(2 * (l - 1) + mirrored) * kCvSlot;
 }
@@ -996,7 +1046,7 @@ int ot_cnn_create(int32_t channels, const float *params, void *stream, ot_cnn_t 
     if (cudaMalloc((void **)&c->w, nb) != cudaSuccess || cudaMalloc((void **)&c->m, nb) != cudaSuccess ||
         cudaMalloc((void **)&c->v, nb) != cudaSuccess ||
         cudaMalloc((void **)&c->wb, sizeof(__nv_bfloat16) * c->nparam) != cudaSuccess ||
-        cudaMalloc((void **)&c->wop, sizeof(__nv_bfloat16) * 7 * kCvSlot) != cudaSuccess ||
+        cudaMalloc((void **)&c->wop, sizeof(__nv_bfloat16) * 6 * kCvSlot) != cudaSuccess ||
         cudaHostAlloc((void **)&c->derr, 64 + sizeof(float) * kMaxBatch, cudaHostAllocDefault) != cudaSuccess) {
         ot_cnn_destroy(c);
         return cnn_fail(nullptr, OT_ERR_OOM, "ot_cnn_create: weight allocation failed");
@@ -1006,14 +1056,11 @@ int ot_cnn_create(int32_t channels, const float *params, void *stream, ot_cnn_t 
     cudaMemsetAsync(c->v, 0, nb, c->st);
     *c->derr = 0;
     c->lpart = (float *)((unsigned char *)c->derr + 64);
-    // (the head's operand has rows without weights)
-    cudaMemsetAsync(c->wop, 0, sizeof(__nv_bfloat16) * 7 * kCvSlot, c->st);
     {
         int dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaFuncSetAttribute(conv_tc_kernel<CV_BLOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize, cv_smem<32>()) != cudaSuccess ||
-            cudaFuncSetAttribute(conv_tc_kernel<CV_GRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, cv_smem<32>()) != cudaSuccess ||
-            cudaFuncSetAttribute(conv_tc_kernel<CV_HEAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, cv_smem<16>()) != cudaSuccess ||
+            cudaFuncSetAttribute(conv_tc_kernel<CV_BLOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCvSmem) != cudaSuccess ||
+            cudaFuncSetAttribute(conv_tc_kernel<CV_GRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCvSmem) != cudaSuccess ||
             cudaFuncSetAttribute(conv_wgrad_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, wg_smem<32>()) != cudaSuccess ||
             cudaFuncSetAttribute(conv_wgrad_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, wg_smem<16>()) != cudaSuccess) {
             ot_cnn_destroy(c);
@@ -1051,20 +1098,18 @@ int ot_cnn_forward(ot_cnn_t *c, int32_t batch, int32_t k, const float *x, float 
     CNN_LAUNCHED(c);
     for (int l = 1; l < kLayers; ++l) {
         const Layer &Ly = c->L[l];
-        ConvIo io{};
-        io.bias = c->w + Ly.b;
         if (Ly.norm) {
+            ConvIo io{};
+            io.bias = c->w + Ly.b;
             io.gain = c->w + Ly.g;
             io.z = c->z[l];
             io.r = c->r[l];
             io.h = c->h[l + 1];
-            launch_pdl(conv_tc_kernel<CV_BLOCK>, grid, kThr, cv_smem<32>(), st, batch, k, k, Ly.dil, c->h[l], wop_of(c, l, 0),
-                       io, c->derr);
+            launch_pdl(conv_tc_kernel<CV_BLOCK>, grid, kThr, kCvSmem, st, batch, k, k, Ly.dil, c->h[l], wop_of(c, l, 0), io,
+                       c->derr);
         } else {
-            io.y = c->z[l];
-            io.y2 = y;
-            launch_pdl(conv_tc_kernel<CV_HEAD>, grid, kThr, cv_smem<16>(), st, batch, k, k, Ly.dil, c->h[l], wop_of(c, l, 0),
-                       io, c->derr);
+            launch_pdl(head_kernel, blocks_for(pix, kHdThr), kHdThr, 0, st, batch, k, k, Ly.dil, c->h[l], c->wb + Ly.W,
+                       c->w + Ly.b, c->z[l], y);
         }
         CNN_LAUNCHED(c);
     }
@@ -1128,7 +1173,7 @@ int ot_cnn_backward(ot_cnn_t *c, const float *dy, float *grad, float *dx) {
         io.h = l > 1 ? c->gb[(l - 1) & 1] : nullptr;
         io.dz32 = l > 1 ? nullptr : c->g0;
         io.part = sums + (l - 1) * ctas * kSumRow;
-        launch_pdl(conv_tc_kernel<CV_GRAD>, grid, kThr, cv_smem<32>(), st, B, k, k, Ly.dil, dz, wop_of(c, l, 1), io, c->derr);
+        launch_pdl(conv_tc_kernel<CV_GRAD>, grid, kThr, kCvSmem, st, B, k, k, Ly.dil, dz, wop_of(c, l, 1), io, c->derr);
         CNN_LAUNCHED(c);
     }
     launch_pdl(block0_wgrad_kernel, (unsigned)n0, 256, 0, st, B, k, k, c->L[0].dil, c->h[0], c->g0, w0part);
