@@ -5,11 +5,13 @@
 //   diag    one CTA factors the 64x64 diagonal block in shared memory, each pivot being minus the
 //           sum of its column's remaining off-diagonal entries (in the block, plus the below-block
 //           sum updated as columns are eliminated), and writes the inverse of the unit block;
-//   panel   L21 = A21 L11^-T D1^-1 through the inverse block (a product of non-positive entries
-//           with non-negative ones: no cancellation), LD = L21 D1;
-//   invrow  block row k of X = L^-1: X_kj = L11^-1 B_kj (B: the updates accumulated in X);
-//   update  one launch over 128x128 tiles of both rank-64 updates: the trailing lower triangle
-//           A22 -= LD L21^T and the rows of X below the panel, B -= L21 X_k.
+//   step    L21 = A21 L11^-T D1^-1 through the inverse block (a product of non-positive entries
+//           with non-negative ones: no cancellation), LD = L21 D1; block row k of X = L^-1: X_kj =
+//           L11^-1 B_kj (B: the updates accumulated in X); the part of both updates that the next
+//           panel needs;
+//   update  the rest of both rank-64 updates beside the chain, the trailing lower triangle
+//           A22 -= LD L21^T and the rows of X below the panel, B -= L21 X_k: FP32 128x128 tiles, or two
+//           panels at once on the tensor cores.
 // The sequence depends on n only, so it is captured once into a CUDA graph.
 #include "dense32.cuh"
 #include "primitives.cuh"
@@ -19,7 +21,6 @@
 
 #include <algorithm>
 #include <cmath>
-#include <mutex>
 #include <vector>
 
 namespace ot {
@@ -1328,19 +1329,12 @@ Error d32_alloc(Dense32 &F, int32_t n) {
     OT_CUDA(cudaMemset(F.A, 0, big));
     OT_CUDA(cudaMemset(F.LD, 0, 3 * sizeof(float) * (size_t)F.ld * kP));
     OT_CUDA(cudaMemset(F.Linv, 0, sizeof(float) * (size_t)F.ld * kP));
-    // one process-wide limit, the largest any n of this path needs (a per-n value set by one
-    // handle could undercut another handle's launch on another thread)
-    static std::once_flag once;
-    static cudaError_t attr_err = cudaSuccess;
-    std::call_once(once, [] {
-        attr_err = cudaFuncSetAttribute(d32_assemble_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)(sizeof(unsigned long long) * kSlice));
-        if (attr_err == cudaSuccess)
-            attr_err = cudaFuncSetAttribute(d32_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRestPad);
-        if (attr_err == cudaSuccess)
-            attr_err = cudaFuncSetAttribute(d32_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, step_smem(2));
-    });
-    if (attr_err != cudaSuccess) return fail(OT_ERR_CUDA, cudaGetErrorString(attr_err));
+    // the largest limits any n of this path needs (a per-n value set by one handle could undercut
+    // another handle's launch on another thread), for the current device
+    OT_CUDA(cudaFuncSetAttribute(d32_assemble_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(sizeof(unsigned long long) * kSlice)));
+    OT_CUDA(cudaFuncSetAttribute(d32_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRestPad));
+    OT_CUDA(cudaFuncSetAttribute(d32_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, step_smem(2)));
     if (n > kMaxN) return fail(OT_ERR_ARG, "dense32: n above the supported size");
     return ok();
 }
@@ -1531,12 +1525,7 @@ Error d32_factor(Dense32 &F, float eps, cudaStream_t st) {
             OT_CUDA(cudaMemset(F.tc_err, 0, sizeof(int)));
             OT_CUDA(cudaMallocHost((void **)&F.tc_err_host, sizeof(int)));
             *F.tc_err_host = 0;
-            static std::once_flag once;
-            static cudaError_t attr = cudaSuccess;
-            std::call_once(once, [] {
-                attr = cudaFuncSetAttribute(d32_tc_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
-            });
-            if (attr != cudaSuccess) return fail(OT_ERR_CUDA, cudaGetErrorString(attr));
+            OT_CUDA(cudaFuncSetAttribute(d32_tc_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem));
         }
         F.use_tc = want_tc;
         if (F.graph) {

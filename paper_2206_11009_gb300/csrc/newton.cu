@@ -10,7 +10,6 @@
 
 #include <cmath>
 #include <cstring>
-#include <mutex>
 #include <type_traits>
 #include <vector>
 
@@ -1047,12 +1046,6 @@ Error launch_pcg(Newton &W, const Support &S, const T *th, const T *thc, const T
       }
     }
     if (!clustered) {
-        static std::once_flag once;
-        static cudaError_t attr = cudaSuccess;
-        std::call_once(once, [] {
-            attr = cudaFuncSetAttribute(pcg_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPcgSmem);
-        });
-        if (attr != cudaSuccess) return fail(OT_ERR_CUDA, cudaGetErrorString(attr));
         int sb = kPcgSmem;
         void *args[] = {&A, &g, &sb};
         ktimer_begin(kid, st);
@@ -1924,6 +1917,9 @@ Error newton_alloc(Newton &W, int32_t m, int32_t n, int64_t cap, int num_sms) {
         OT_TRY(dev_alloc(p, n));
     for (float **p : {&W.Dinv32, &W.b32, &W.x32, &W.r32, &W.q32}) OT_TRY(dev_alloc(p, n));
     OT_TRY(dev_alloc(&W.pcg_node, 5 * (int64_t)n));
+    // (per handle: the attribute belongs to the current device)
+    OT_CUDA(cudaFuncSetAttribute(pcg_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPcgSmem));
+    OT_CUDA(cudaFuncSetAttribute(pcg_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPcgSmem));
     // grid PCG lane groups: one block of at most 1024 threads per SM
     W.pcg_bnd_cap = 1024LL * std::max(num_sms, 1) + 1;
     OT_TRY(dev_alloc(&W.pcg_bnd, 2 * W.pcg_bnd_cap));
