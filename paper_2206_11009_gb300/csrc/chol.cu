@@ -378,6 +378,9 @@ Error chol_assemble(Chol &C, Newton &W, const Support &S, double drop, bool *pat
         OT_CUDA(cudaStreamSynchronize(st));
     }
     if ((int64_t)nu > C.capA) {
+        // a2l goes with the arrays: the next sparse factorisation runs chol_symbolic, which fills it, even where
+        // the pattern is the one on the host (a dense call may come between two of the same pattern)
+        C.have_symbolic = false;
         dfree(C.Aj); dfree(C.Ax); dfree(C.a2l);
         C.capA = std::max<int64_t>(nu, (int64_t)(1.5 * C.capA));
         OT_TRY(dalloc(&C.Aj, C.capA));
