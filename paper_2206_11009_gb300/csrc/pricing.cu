@@ -132,15 +132,19 @@ __device__ __forceinline__ float key32(const float4 &R, float cB, float cx, floa
     return __fsub_rn(__fsub_rn(c, R.x), cB);
 }
 
-// Order-preserving signed key of a double's high word (the low word only refines it).
+// Order-preserving signed key of a double's high word (the low word only refines it), shifted so that
+// -infinity is the least: the quiet NaNs with the sign bit set, below it before, wrap to the top, next to
+// the others (as the least key of a thread's part of a tile, one of them hid the pairs there from pass 2).
+constexpr int kKeyShift = 0xfffff;
 __device__ __forceinline__ int hi_key(double d) {
     const int h = __double2hiint(d);
-    return h ^ ((h >> 31) & 0x7fffffff);
+    return (int)((unsigned)(h ^ ((h >> 31) & 0x7fffffff)) - kKeyShift);
 }
 // A float at or below every double whose hi_key is k.
 __device__ __forceinline__ float hi_key_floor(int k) {
+    k = (int)((unsigned)k + kKeyShift);
     const int h = k ^ ((k >> 31) & 0x7fffffff);
-    return __double2float_rd(__hiloint2double(h, h < 0 ? -1 : 0));
+    return __double2float_rd(__hiloint2double(h, h < 0 && h != (int)0xfff00000 ? -1 : 0));   // (-infinity has no low bits)
 }
 
 // --------------------------------------------------------------------------------- prep
@@ -640,7 +644,7 @@ scan64_kernel(int m, int n, int TI, int ncb, int64_t ntiles, SupArgs S,
         __syncthreads();
         // Tg <= 0 here.  A pair is taken when float(d) <= Tg (d < 0 in the histogram pass): its high
         // word's key is then at most one above Tg's (the rounding to float)
-        const int kthr = GATHER ? hi_key((double)Tg) + 1 : -1;
+        const int kthr = GATHER ? hi_key((double)Tg) + 1 : hi_key(-0.0);
         int kmin = INT_MAX;
         for (int r = 0; r < nrows; ++r) {
             double dd[RJ];
