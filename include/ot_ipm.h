@@ -163,7 +163,9 @@ typedef struct {
     int32_t tc_update;
     /* Relative residual at which the CG preconditioned by a factorisation (the FP32 dense factor,
      * the direct branch) stops: 0 = min(CG tolerance, 1e-10) (near-exact Newton directions);
-     * > 0: max(direct_cg_tol, min(CG tolerance, 1e-10)). */
+     * > 0: max(direct_cg_tol, min(CG tolerance, 1e-10)).  With the FP32 factor and a connected support
+     * the residual of the last column's equation counts as minus the sum of the others (which it is
+     * but for rounding that no iteration reduces). */
     double direct_cg_tol;
 } ot_options;
 

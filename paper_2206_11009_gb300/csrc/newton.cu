@@ -448,15 +448,14 @@ __global__ void beta1_group_kernel(int m, const int32_t *__restrict__ rp, const 
 }
 
 // every block sums the gridDim partials of `slots` (fixed order: deterministic, identical in
-// all blocks); warp 0 does it, lanes taking strided partials
+// all blocks); warp s does slot s, lanes taking strided partials
 __device__ __forceinline__ void sum_partials(const double *part, unsigned G, int nslots, double *out_sh) {
-    if (threadIdx.x < 32) {
-        for (int s = 0; s < nslots; ++s) {
-            double a = 0;
-            for (unsigned k = threadIdx.x; k < G; k += 32) a += part[(int64_t)s * G + k];
-            a = warp_sum(a);
-            if (threadIdx.x == 0) out_sh[s] = a;
-        }
+    const int s = (int)threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (s < nslots) {
+        double a = 0;
+        for (unsigned k = lane; k < G; k += 32) a += part[(int64_t)s * G + k];
+        a = warp_sum(a);
+        if (lane == 0) out_sh[s] = a;
     }
     __syncthreads();
 }
@@ -1264,28 +1263,35 @@ __global__ void mvg_cols_kernel(int n, const int32_t *__restrict__ cp, const int
 }
 
 // x += a p, r -= a q with a = r.z / p.q: p.q reduced here from its partials (nbq of them), r.z
-// read from its scalar slot; block 0 records p.q; partial r.r
+// read from its scalar slot; block 0 records p.q; partial r.r and, with `implied` >= 0, the sum of the
+// entries other than that one, which goes to its own slot squared
 __global__ void dcg_step2_kernel(int n, int nbq, double *__restrict__ scal, int rz_slot, const double *__restrict__ p,
                                  const double *__restrict__ q, double *__restrict__ x, double *__restrict__ r,
-                                 double *part) {
+                                 int implied, double *part) {
     __shared__ double sh[kT / 32];
     __shared__ double bc;
     const double pq = sum_slot(part, SC_SUM_A, nbq, sh, &bc);
     const double rz = scal[rz_slot];
     if (blockIdx.x == 0 && threadIdx.x == 0) scal[SC_SUM_A] = pq;
     const double a = (pq > 0 && rz > 0) ? rz / pq : 0.0;
-    double rr = 0;
+    double rr = 0, rs = 0;
     GRID_STRIDE(j, n) {
         x[j] += a * p[j];
         const double rj = r[j] - a * q[j];
         r[j] = rj;
-        rr += rj * rj;
+        if (j == implied) {
+            scal[SC_RIMPL] = rj * rj;
+        } else {
+            rr += rj * rj;
+            rs += rj;
+        }
     }
     put_sum(rr, part, SC_NORM_A, sh);
+    put_sum(rs, part, SC_SUM_B, sh);
 }
 
 // p = z + b p with b = r.z(new) / r.z(old): r.z(new) reduced here (nbz partials of new_slot) and
-// recorded by block 0, which also records r.r (nbr partials)
+// recorded by block 0, which also records the step's two sums over r (nbr partials)
 __global__ void dcg_dir2_kernel(int n, int nbz, int nbr, double *__restrict__ scal, int old_slot, int new_slot,
                                 const double *__restrict__ z, double *__restrict__ p, const double *__restrict__ part) {
     __shared__ double sh[kT / 32];
@@ -1296,9 +1302,11 @@ __global__ void dcg_dir2_kernel(int n, int nbz, int nbr, double *__restrict__ sc
     GRID_STRIDE(j, n) p[j] = z[j] + b * p[j];
     if (blockIdx.x == 0) {
         const double rr = sum_slot(part, SC_NORM_A, nbr, sh, &bc);
+        const double rs = sum_slot(part, SC_SUM_B, nbr, sh, &bc);
         if (threadIdx.x == 0) {
             scal[new_slot] = rzn;
             scal[SC_NORM_A] = rr;
+            scal[SC_SUM_B] = rs;
         }
     }
 }
@@ -1413,7 +1421,15 @@ constexpr int kD32MaxCg = 60;
 // step with r.r, the convergence test, the three stages of the preconditioner (partial products of
 // X r by 512 x 64 tiles, their row sums scaled by D^+, the column products of X^T), r.z and the new
 // direction, seven grid barriers.  Every block sums the partials of a dot product in the same fixed
-// order, so all take the same decisions.  Same arithmetic as the launch-per-stage loop.
+// order, so all take the same decisions.  Same arithmetic and stopping rule as the launch-per-stage loop.
+//
+// Stopping rule.  The equations of a connected component add up to zero, and the factor grounds its last
+// column (nothing is left of that column's pivot), so M^-1 neither reads nor moves the residual there: in
+// exact arithmetic it is minus the sum of the others, in FP64 the rounding of every q adds up in it and no
+// iteration reduces that (1e-12 .. 5e-7 of b; 60 iterations then pass in vain).  With one component the test
+// therefore takes minus that sum for the last entry; the residual reported keeps the entry as it stands.
+// (A test of r.z in place of it lets go of residuals along large eigenvalues: 8e-3 of b at 1e-6.)
+// With several components every entry counts as it stands.
 constexpr int kCgT = 512;
 constexpr int kCgRows = 512, kCgCols = 64;   // preconditioner tile: 128 row quads x 4 column groups
 
@@ -1424,10 +1440,11 @@ struct D32CgArgs {
     const float *X, *D;
     float *part, *w32;
     double *x, *r, *z, *p, *q, *w64;
-    double *red;          // 3 slots x gridDim partial sums
+    double *red;          // 4 slots x gridDim partial sums
     unsigned *bar;
     int *err;
     double target2;       // stop when r.r <= target2 * b.b
+    int implied;          // entry given by the others' sum (n - 1: one component), or -1
     int maxit;
     double *scal;         // SC_PCG_ITERS, SC_PCG_RELRES
 };
@@ -1552,9 +1569,9 @@ __device__ __forceinline__ double cg_bwd(const D32CgArgs &A, const double *__res
 }
 
 template <int LG>
-__global__ void __launch_bounds__(kCgT) d32_cg_kernel(D32CgArgs A) {
-    __shared__ double sh[kCgT / 32];
-    __shared__ double s_val[3];
+__global__ void __launch_bounds__(kCgT, 1) d32_cg_kernel(D32CgArgs A) {
+    __shared__ double sh[kCgT / 32], sh2[kCgT / 32];
+    __shared__ double s_val[4];
     __shared__ float rs[kCgCols];
     __shared__ float4 red4[3 * (kCgRows / 4)];
     const unsigned G = gridDim.x;
@@ -1563,7 +1580,7 @@ __global__ void __launch_bounds__(kCgT) d32_cg_kernel(D32CgArgs A) {
     const int64_t stride = (int64_t)G * blockDim.x;
     const int lg = threadIdx.x & (LG - 1);
     const int64_t grp = tid / LG, ngrp = stride / LG, wgrp0 = (tid & ~(int64_t)31) / LG;
-    double *P0 = A.red, *P1 = A.red + G, *P2 = A.red + 2 * G;
+    double *P0 = A.red, *P1 = A.red + G, *P2 = A.red + 2 * G, *P3 = A.red + 3 * G;
     // x = 0, r = rhs, z = M^-1 r, p = z
     double rr = 0.0;
     for (int64_t j = tid; j < n; j += stride) {
@@ -1593,7 +1610,6 @@ __global__ void __launch_bounds__(kCgT) d32_cg_kernel(D32CgArgs A) {
     int it = 0;
     bool extra = false;
     double rr_test = rr;
-    const double rz0 = rz;
     if (bb > 0.0 && rz > 0.0 && A.maxit > 0) {
         for (;;) {
             // the new direction p must be complete before the row pass gathers it
@@ -1630,25 +1646,40 @@ __global__ void __launch_bounds__(kCgT) d32_cg_kernel(D32CgArgs A) {
             pq = s_val[0];
             if (!(pq > 0.0)) break;   // breakdown: the step would be a no-op
             const double alpha = rz > 0.0 ? rz / pq : 0.0;
-            double rrn = 0.0;
+            double rrn = 0.0, rsum = 0.0;   // of the entries but the implied one
             for (int64_t j = tid; j < n; j += stride) {
                 A.x[j] += alpha * A.p[j];
                 const double rj = A.r[j] - alpha * A.q[j];
                 A.r[j] = rj;
-                rrn += rj * rj;
+                if (j != A.implied) {
+                    rrn += rj * rj;
+                    rsum += rj;
+                }
             }
             {
-                const double s2 = block_sum(rrn, sh);
-                if (threadIdx.x == 0) P2[blockIdx.x] = s2;
+                // both sums at once: warp sums, then a thread for each (in the order of block_sum)
+                rrn = warp_sum(rrn);
+                rsum = warp_sum(rsum);
+                if ((threadIdx.x & 31) == 0) { sh[threadIdx.x >> 5] = rrn; sh2[threadIdx.x >> 5] = rsum; }
+                __syncthreads();
+                if ((threadIdx.x & ~32) == 0) {
+                    const double *v = threadIdx.x ? sh2 : sh;
+                    double t = 0.0;
+                    for (int w = 0; w < kCgT / 32; ++w) t += v[w];
+                    (threadIdx.x ? P3 : P2)[blockIdx.x] = t;
+                }
             }
             if (!grid_barrier(A.bar, G, A.err)) return;
-            sum_partials(A.red + 2 * G, G, 1, s_val + 2);
-            rr = s_val[2];
+            sum_partials(A.red + 2 * G, G, 2, s_val + 2);
+            if (blockIdx.x == 0 && threadIdx.x == 0) {   // (reported only)
+                const double ri = A.implied >= 0 ? A.r[A.implied] : 0.0;
+                rr = s_val[2] + ri * ri;
+            }
             if (extra) break;
             ++it;
             rr_test = rr;
             if (it >= A.maxit) break;
-            if (rr <= A.target2 * bb) extra = true;
+            if (s_val[2] + (A.implied >= 0 ? s_val[3] * s_val[3] : 0.0) <= A.target2 * bb) extra = true;
             cg_fwd(A, A.r, rs, red4);
             if (!grid_barrier(A.bar, G, A.err)) return;
             cg_mid(A);
@@ -1661,9 +1692,6 @@ __global__ void __launch_bounds__(kCgT) d32_cg_kernel(D32CgArgs A) {
             if (!grid_barrier(A.bar, G, A.err)) return;
             sum_partials(A.red + G, G, 1, s_val + 1);
             rzn = s_val[1];
-            // what is left of r when its preconditioned norm has fallen that far lies in the null space
-            // of S_M (rounding of the mean, about 1e-12 of b from n = 9216 on): no iteration reduces it
-            if (rzn <= A.target2 * rz0) extra = true;
             const double beta = (rz > 0.0 && rzn > 0.0) ? rzn / rz : 0.0;
             for (int64_t j = tid; j < n; j += stride) A.p[j] = A.z[j] + beta * A.p[j];
             rz = rzn;
@@ -1694,7 +1722,7 @@ static Error solve_d32_persistent(Newton &W, const Support &S, double target, in
     OT_CUDA(cudaMemsetAsync(W.err, 0, sizeof(int), st));
     D32CgArgs A{W.m, W.n, F.ld, (int)ceil_div(W.n, kCgCols), S.row_ptr, S.j, S.col_ptr, S.col_row, W.theta,
                 W.theta_col, W.Minv, W.rhs, F.X, F.D, F.part, F.w, dv, W.r64, W.z64, W.p64, W.q64, W.w64, W.part,
-                W.bar, W.err, target * target, cap, W.scal};
+                W.bar, W.err, target * target, W.onecomp ? W.n - 1 : -1, cap, W.scal};
     void *args[] = {&A};
     ktimer_begin(KT_DCG, st);
     const cudaError_t le = cudaLaunchCooperativeKernel(fn, dim3(G), dim3(kCgT), args, 0, st);
@@ -1777,6 +1805,8 @@ static Error solve_direct(Newton &W, const Support &S, double tol, int max_cg, d
         // per column the offset, q, p twice and the step's reads of x, r and writes of x, r
         const double dcg_bytes = 40.0 * (double)S.psi + 20.0 * (double)W.m + 68.0 * (double)W.n;
         const bool ahead = C == nullptr;  // iterations queued ahead only where the preconditioner is cheap
+        // the entry implied by the others (the stopping rule above d32_cg_kernel)
+        const int implied = W.d32 && !C && !W.tree && W.onecomp ? W.n - 1 : -1;
         auto direction = [&](int k) -> Error {   // z = M^-1 r and the direction after iteration k
             const int cur = (k & 1) ? SC_RZ1 : SC_RZ0, nxt = (k & 1) ? SC_RZ0 : SC_RZ1;
             OT_TRY(precond(r, z));
@@ -1803,12 +1833,12 @@ static Error solve_direct(Newton &W, const Support &S, double tol, int max_cg, d
                 mvg_cols_kernel<4><<<gnc, kT, 0, st>>>(W.n, S.col_ptr, S.col_row, W.theta_col, W.w64, p, q, W.part);
             }
             OT_LAUNCHED();
-            dcg_step2_kernel<<<gn, kT, 0, st>>>(W.n, (int)gnc, W.scal, cur, p, q, x, r, W.part);
+            dcg_step2_kernel<<<gn, kT, 0, st>>>(W.n, (int)gnc, W.scal, cur, p, q, x, r, implied, W.part);
             OT_LAUNCHED();
             ktimer_end(KT_DCG, st);
             ktimer_add_work(KT_DCG, dcg_bytes);
             if (!ahead) {   // r.r for the test, before the next preconditioner is paid for
-                Finish f{1, {SC_NORM_A}, {(int)gn}, {0}};
+                Finish f{2, {SC_NORM_A, SC_SUM_B}, {(int)gn, (int)gn}, {0, 0}};
                 OT_TRY(finish(f, W, st));
             } else {
                 OT_TRY(direction(k));
@@ -1839,9 +1869,9 @@ static Error solve_direct(Newton &W, const Support &S, double tol, int max_cg, d
             }
             const double pq = h[SC_SUM_A];
             if (!(pq > 0)) break;  // breakdown: this step was a no-op
-            rr = h[SC_NORM_A];
+            rr = h[SC_NORM_A] + (implied >= 0 ? h[SC_RIMPL] : 0.0);
             ++it;
-            if (rr <= target * target * bb) break;
+            if (h[SC_NORM_A] + (implied >= 0 ? h[SC_SUM_B] * h[SC_SUM_B] : 0.0) <= target * target * bb) break;
             if (!ahead && it < cap) {
                 OT_TRY(direction(it - 1));
                 OT_TRY(issue(issued));

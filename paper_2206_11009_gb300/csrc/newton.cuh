@@ -13,6 +13,7 @@ enum Scalar : int {
     SC_MUAFF, SC_PSNEW, SC_SUM_A, SC_SUM_B, SC_NORM_A, SC_NORM_B, SC_ONECOMP,
     SC_PCG_ITERS, SC_PCG_RELRES,
     SC_RZ0, SC_RZ1,          // ping-pong r.z of the refinement CG (alpha, beta formed on the device)
+    SC_RIMPL,                // square of the residual entry that the others imply
     SC_COUNT
 };
 
