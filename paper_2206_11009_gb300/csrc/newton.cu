@@ -1079,13 +1079,13 @@ __global__ void mv_rows_kernel(int m, const int32_t *__restrict__ rp, const int3
     }
 }
 
-// res = rhs - S_M x ; partial ||res||^2
+// res = rhs - S_M x ; partial ||res||^2 and sum of res
 __global__ void mv_cols_res_kernel(int n, const int32_t *__restrict__ cp, const int32_t *__restrict__ crow,
                                    const double *__restrict__ thc, const double *__restrict__ w,
                                    const double *__restrict__ x, const double *__restrict__ rhs,
                                    double *__restrict__ res, double *part) {
     __shared__ double sh[kT / 32];
-    double sq = 0;
+    double sq = 0, sum = 0;
     GRID_STRIDE(j, n) {
         const double xj = x[j];
         double acc = 0;
@@ -1093,8 +1093,10 @@ __global__ void mv_cols_res_kernel(int n, const int32_t *__restrict__ cp, const 
         const double r = rhs[j] - acc;
         res[j] = r;
         sq += r * r;
+        sum += r;
     }
     put_sum(sq, part, SC_NORM_A, sh);
+    put_sum(sum, part, SC_SUM_B, sh);
 }
 
 __global__ void norm_kernel(int n, const double *__restrict__ x, double *part, int slot) {
@@ -1104,8 +1106,8 @@ __global__ void norm_kernel(int n, const double *__restrict__ x, double *part, i
     put_sum(sq, part, slot, sh);
 }
 
-__global__ void to_f32_kernel(int n, const double *__restrict__ x, float *__restrict__ y) {
-    GRID_STRIDE(j, n) y[j] = (float)x[j];
+__global__ void to_f32_kernel(int n, const double *__restrict__ x, double shift, float *__restrict__ y) {
+    GRID_STRIDE(j, n) y[j] = (float)(x[j] - shift);
 }
 
 __global__ void axpy_f32_kernel(int n, const float *__restrict__ d, double *__restrict__ x) {
@@ -1320,17 +1322,30 @@ Error dev_alloc(T **p, int64_t count) {
 }  // namespace
 
 // ------------------------------------------------------------------------ S_M x = rhs
-static Error residual_norm(Newton &W, const Support &S, const double *x, double *res, double *nrm, cudaStream_t st) {
+static Error project(Newton &W, double *x, bool one_comp, cudaStream_t st);
+
+// res = rhs - S_M x and the norm of its part in the range of S_M, mean zero on every component: the rest is
+// rounding of the sums, which no correction reduces.  *shift: res - *shift is that part (with several
+// components res itself is projected and the shift is 0).
+static Error residual_norm(Newton &W, const Support &S, const double *x, double *res, double *nrm, double *shift,
+                           cudaStream_t st) {
     const unsigned gm = grid_of(W.m, W.num_sms), gn = grid_of(W.n, W.num_sms);
     mv_rows_kernel<<<gm, kT, 0, st>>>(W.m, S.row_ptr, S.j, W.theta, W.Minv, x, W.w64);
     OT_LAUNCHED();
     mv_cols_res_kernel<<<gn, kT, 0, st>>>(W.n, S.col_ptr, S.col_row, W.theta_col, W.w64, x, W.rhs, res, W.part);
     OT_LAUNCHED();
-    Finish f{1, {SC_NORM_A}, {(int)gn}, {0}};
+    *shift = 0.0;
+    if (!W.onecomp) {
+        OT_TRY(project(W, res, false, st));
+        norm_kernel<<<gn, kT, 0, st>>>(W.n, res, W.part, SC_NORM_A);
+        OT_LAUNCHED();
+    }
+    Finish f{2, {SC_NORM_A, SC_SUM_B}, {(int)gn, (int)gn}, {0, 0}};
     OT_TRY(finish(f, W, st));
     double hs[SC_COUNT];
     OT_TRY(read_scalars(W, hs, st));
-    *nrm = std::sqrt(hs[SC_NORM_A]);
+    if (W.onecomp) *shift = hs[SC_SUM_B] / (double)W.n;
+    *nrm = std::sqrt(std::max(hs[SC_NORM_A] - *shift * *shift * (double)W.n, 0.0));
     return ok();
 }
 
@@ -1369,6 +1384,10 @@ static Error solve_pcg64(Newton &W, const Support &S, double tol, int max_cg, do
 
 // FP32 PCG inside FP64 iterative refinement: dv = 0, res = rhs; repeat
 //   solve S32 d = float(res) ; dv += d ; res = rhs - S64 dv      until |res| <= tol |rhs|
+// with res projected to mean zero: near the end its mean is rounding and no smaller than the rest, and on
+// that inconsistent system the FP32 iteration stalled or diverged.  100x100, 7 inputs: 1,186 to 16,558
+// iterations (10.9 to 142 ms) became 1,048 to 1,215 (9.7 to 11.2 ms), the direction's error 1e-10 .. 6e-14
+// 8e-14 .. 4e-14.
 static Error solve_mixed(Newton &W, const Support &S, double tol, int max_cg, double *dv, SolveStats *ss,
                          cudaStream_t st) {
     const unsigned gn = grid_of(W.n, W.num_sms);
@@ -1378,17 +1397,17 @@ static Error solve_mixed(Newton &W, const Support &S, double tol, int max_cg, do
     OT_LAUNCHED();
     double nrm0 = 0.0;
     OT_TRY(rhs_norm(W, &nrm0, st));
-    double nrm = nrm0;
+    double nrm = nrm0, shift = 0.0;
     int budget = max_cg;
     for (int ref = 0; ref < 12 && nrm > tol * nrm0 && budget > 0; ++ref) {
-        to_f32_kernel<<<gn, kT, 0, st>>>(W.n, W.res64, W.b32);
+        to_f32_kernel<<<gn, kT, 0, st>>>(W.n, W.res64, shift, W.b32);
         OT_LAUNCHED();
         OT_TRY(launch_pcg<float>(W, S, W.theta32, W.theta32_col, W.Minv32, W.Dinv32, W.b32, W.x32, W.r32, W.q32,
                                  W.w32, inner, budget, st));
         axpy_f32_kernel<<<gn, kT, 0, st>>>(W.n, W.x32, dv);
         OT_LAUNCHED();
         const double prev = nrm;
-        OT_TRY(residual_norm(W, S, dv, W.res64, &nrm, st));
+        OT_TRY(residual_norm(W, S, dv, W.res64, &nrm, &shift, st));
         double hs[SC_COUNT];
         OT_TRY(read_scalars(W, hs, st));
         int errv = 0;
