@@ -459,6 +459,12 @@ __device__ __forceinline__ void take_key(float d, bool neg64, float E, float Tg,
     }
 }
 
+// Pass 2 has nothing to do when its bound exceeds the buffer: the host redoes it with a larger one, or in
+// FP64 (evaluating and counting the 151M pairs of a flooded FP32 window took 3.0 ms; 0.01 so).
+__device__ __forceinline__ bool gather_in_vain(const Geo *geo, unsigned long long cap) {
+    return geo->gather_bound > cap;
+}
+
 // The support pairs entered the histogram too (the scan does not test membership): their own
 // histogram, with the same arithmetic as the scan so that every key lands in the same bin, by the
 // blocks `part` of `parts` of the histogram launch (shared-memory counts first: global atomics on
@@ -521,6 +527,7 @@ tile_scan_kernel(int m, int n, int G, int nrg, SupArgs S, const float4 *__restri
                  unsigned long long cap, unsigned int *__restrict__ ncand) {
     __shared__ float4 srow[kPT / 32][kStage];
     __shared__ unsigned sh_hist[GATHER ? 1 : kBins];
+    if (GATHER && gather_in_vain(geo, cap)) return;
     if (!GATHER) {
         for (int b = threadIdx.x; b < kBins; b += kPT) sh_hist[b] = 0;
         __syncthreads();
@@ -612,6 +619,7 @@ scan64_kernel(int m, int n, int TI, int ncb, int64_t ntiles, SupArgs S,
     __shared__ double srowu[256];
     __shared__ unsigned sh_hist[GATHER ? 1 : kBins];
     __shared__ float sred[kPT / 32];
+    if (GATHER && gather_in_vain(geo, cap)) return;
     if (!GATHER) {
         for (int b = threadIdx.x; b < kBins; b += kPT) sh_hist[b] = 0;
         __syncthreads();
@@ -713,6 +721,7 @@ jscan_kernel(int n, int64_t jn, int64_t ntiles, SupArgs S, const int32_t *__rest
              int32_t *__restrict__ cj, unsigned long long cap, unsigned int *__restrict__ ncand) {
     __shared__ unsigned sh_hist[GATHER ? 1 : kBins];
     __shared__ float sred[kPT / 32];
+    if (GATHER && gather_in_vain(geo, cap)) return;
     if (!GATHER) {
         for (int b = threadIdx.x; b < kBins; b += kPT) sh_hist[b] = 0;
         __syncthreads();
@@ -1390,7 +1399,7 @@ Error price_topk(const PriceInput &in, int32_t *out_i, int32_t *out_j, double *o
     OT_LAUNCHED();
     Geo hg;
     {
-        // the gathered set rarely passes a few times kmax (its last bin is a sixteenth of an octave of
+        // the gathered set rarely passes a few times kmax (its last bin is a sixty-fourth of an octave of
         // |d|, plus the support's pairs and the FP32 window)
         const unsigned cap = spec_capacity(in.kmax);
         DevTemp<char> cand;

@@ -57,10 +57,10 @@ def test_selection_at_the_capacity(kmax, over, precision):
 
 
 def test_flooded_window_is_not_gathered():
-    """151M pairs inside the FP32 window, three columns of negative ones: the FP32 pass 2 of this call has
-    nothing to do and the FP64 one skips all but three columns' tiles, so that together they take less than
-    the two histogram passes, which evaluate every pair (pass 2 evaluates and counts every pair of the window
-    when it does not look at the bound: 151M atomics on one word)."""
+    """151M pairs inside the FP32 window, three columns of negative ones: the FP32 pass 2 has nothing to do
+    and the call is redone in FP64, so pass 2 takes what it takes in a call in FP64 from the start (less than
+    half of that more; when the FP32 pass does not look at its bound it evaluates every pair and counts those
+    of the window one by one, more than the FP64 pass 2 over half of the columns)."""
     import torch
     from paper_2206_11009_gb300 import kernel_timing, price_topk
     m = n = 12288
@@ -68,12 +68,14 @@ def test_flooded_window_is_not_gathered():
     u, v = np.full(m, 1e5), np.full(n, -1e5)
     v[[17, 4000, 9001]] += np.array([1.0, 3.0, 2.0])
     T = U.cuda_tensors(z, z, z, z, u, v, NONE, NONE)
-    price_topk(*T, kmax=50000, precision=1)
-    torch.cuda.synchronize()
-    kernel_timing(True)
-    out = price_topk(*T, kmax=50000, precision=1)
-    t = kernel_timing()
-    kernel_timing(False)
-    print({k: x for k, x in t.items() if k.startswith("scan")})
-    assert len(out[0]) == 3 * m
-    assert t["scan_gather"][0] < t["scan_hist"][0]
+    ms = {}
+    for precision in (0, 1):
+        price_topk(*T, kmax=50000, precision=precision)
+        torch.cuda.synchronize()
+        kernel_timing(True)
+        out = price_topk(*T, kmax=50000, precision=precision)
+        ms[precision] = kernel_timing()["scan_gather"][0]
+        kernel_timing(False)
+        assert len(out[0]) == 3 * m
+    print(ms)
+    assert ms[1] <= 1.5 * ms[0]
