@@ -914,10 +914,25 @@ void layout(ot_cnn *c) {
     c->nparam = off;
 }
 
+// the activations and everything that says there are some: no forward to take a loss or a gradient of
 void free_acts(ot_cnn *c) {
     if (c->acts) cudaFree(c->acts);
     c->acts = nullptr;
     c->cap_pix = 0;
+    c->B = c->k = 0;
+    for (int l = 0; l < kLayers; ++l) {
+        c->h[l] = nullptr;
+        c->z[l] = nullptr;
+        c->r[l] = nullptr;
+    }
+}
+
+// cudaMalloc whose failure is reported here and not by the next launch's check too
+bool dev_malloc(void **p, int64_t bytes) {
+    if (cudaMalloc(p, (size_t)bytes) == cudaSuccess) return true;
+    *p = nullptr;
+    cudaGetLastError();
+    return false;
 }
 
 // CTAs of the tensor-core kernels and of the head's backward: two per SM at most
@@ -931,7 +946,7 @@ int ensure_acts(ot_cnn *c, int B, int k) {
         const int64_t tp = (pix + kCvM - 1) / kCvM * kCvM;
         int64_t per = 0;   // bytes per pixel
         for (int l = 0; l < kLayers; ++l) per += 2 * c->L[l].cin + 4 * c->L[l].cout + 4;
-        if (cudaMalloc((void **)&c->acts, per * tp) != cudaSuccess)
+        if (!dev_malloc((void **)&c->acts, per * tp))
             return cnn_fail(c, OT_ERR_OOM, "ot_cnn: activation allocation failed");
         unsigned char *p = c->acts;
         for (int l = 0; l < kLayers; ++l) {
@@ -959,7 +974,7 @@ int ensure_grads(ot_cnn *c) {
         c->cap_grad = 0;
         const int64_t tp = (pix + kCvM - 1) / kCvM * kCvM, ctas = tc_ctas(c, pix);
         const int64_t parts = 4 * ctas * (kSumRow + kWgStride) + (pix + kW0 - 1) / kW0 * 576;
-        if (cudaMalloc((void **)&c->grads, 4 * parts + tp * c->ch * (4 + 2 + 2)) != cudaSuccess)
+        if (!dev_malloc((void **)&c->grads, 4 * parts + tp * c->ch * (4 + 2 + 2)))
             return cnn_fail(c, OT_ERR_OOM, "ot_cnn: gradient allocation failed");
         c->g0 = (float *)c->grads;
         c->gb[0] = (__nv_bfloat16 *)(c->g0 + tp * c->ch);
