@@ -51,9 +51,7 @@ __global__ void dense_scatter_kernel(int n, const int32_t *__restrict__ Ap, cons
 
 // (1) Panel [k, k + bs): warps 0-3 hold the diagonal block's rows, warps 4-7 the CTA's 32 rows below
 // (one row per lane, columns w, w + 4, ... of warp w in registers).  Step j: the owners of column j
-// publish it, then every row takes l = a_rj / d_j and a_rc -= l a_cj for its later columns.  1 / d
-// from the hardware's approximation by one step of Halley's iteration (cubic: the relative error e
-// becomes e^3), applied to the quotient: three dependent multiply-adds instead of a division.
+// publish it, then every row takes l = a_rj / d_j (quotient) and a_rc -= l a_cj for its later columns.
 // CTA 0 writes D and the block's L.  32 steps of about 500 cycles; the substitution with one thread
 // per row that it replaced took 350 us per 64 columns at n = 961 (and the diagonal block 210 us).
 __global__ void __launch_bounds__(kT)
@@ -79,11 +77,7 @@ dense_panel_kernel(int n, int k, int bs, double *__restrict__ A, double *__restr
         __syncthreads();
         const double d = cj[0][j], v = cj[half][lane];
         const bool inf = !(d > thr[j]);
-        double r0;
-        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(d));
-        const double e = fma(-d, r0, 1.0), v0 = v * r0;
-        const double t = fma(e, e, e);
-        const double l = inf ? 0.0 : fma(v0, t, v0);
+        const double l = inf ? 0.0 : quotient(v, d);
 #pragma unroll
         for (int q = 0; q < kB / 4; ++q)
             if (w + 4 * q > j) a[q] = fma(-l, cj[0][w + 4 * q], a[q]);

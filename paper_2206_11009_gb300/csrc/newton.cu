@@ -460,14 +460,6 @@ __device__ __forceinline__ void sum_partials(const double *part, unsigned G, int
     __syncthreads();
 }
 
-// 1 / d for normal d by the hardware's approximation and one step of Halley's iteration
-__device__ __forceinline__ double halley_rcp(double d) {
-    double r0;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(d));
-    const double e = fma(-d, r0, 1.0);
-    return fma(r0, fma(e, e, e), r0);
-}
-
 // Hand-over between all blocks: one released increment of a counter per block, polled by one thread
 // of each (1.5 us whatever the number of blocks; with a flag per block and every block polling all
 // of them it took 5 us at 152 blocks).  `target`: arrivals after which it opens.  Bounded; false when it
@@ -706,9 +698,9 @@ __global__ void __launch_bounds__(kPcgT<T>, 1) pcg_kernel(PcgArgs<T> A, int g, i
         __syncthreads();
         if (threadIdx.x == 0) {
             const double pq = s_val[0], qs = s_val[1], rz = s_val[2], zq = s_val[4];
-            const double al = rz * halley_rcp(pq), next = fma(al, fma(al, qs, -2.0 * zq), rz);
+            const double al = quotient(rz, pq), next = fma(al, fma(al, qs, -2.0 * zq), rz);
             s_ab[0] = (T)al;
-            s_ab[1] = (T)fmax(next * halley_rcp(rz), 0.0);
+            s_ab[1] = (T)fmax(quotient(next, rz), 0.0);
             const double rrv = s_val[3], lim = it == 0 ? rrv : bb;
             // stop: converged, out of iterations, or breakdown (exact zero direction or residual, loss
             // of definiteness)
