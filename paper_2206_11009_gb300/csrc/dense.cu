@@ -211,7 +211,8 @@ __device__ __forceinline__ bool await8(const double *p, int valid, double &v, in
     for (unsigned spin = 0;; ++spin) {
         if (b == kUnset) asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(b) : "l"(p + q) : "memory");
         if (__all_sync(0xffffffffu, b != kUnset)) break;
-        if (spin > kSpinLimit || ((spin & 63u) == 63u && *(volatile int *)err)) {
+        // (one decision for the warp: a lane that left alone would leave the others in the votes)
+        if ((spin & 63u) == 63u && __any_sync(0xffffffffu, spin > kSpinLimit || *(volatile int *)err != 0)) {
             atomicCAS(err, 0, (int)OT_ERR_TIMEOUT);
             return false;
         }
