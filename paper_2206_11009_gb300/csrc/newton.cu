@@ -500,7 +500,7 @@ __device__ __forceinline__ bool count_reach(unsigned *cnt, unsigned target, int 
 template <typename T>
 __global__ void __launch_bounds__(kPcgT<T>, 1) pcg_kernel(PcgArgs<T> A, int g, int smem_bytes) {
     constexpr int NT = kPcgT<T>;
-    extern __shared__ __align__(16) unsigned char dsm[];
+    extern __shared__ __align__(32) unsigned char dsm[];   // (of a PcgNode<double>)
     __shared__ double dots[kPcgDots][NT];
     __shared__ double s_val[kPcgDots];
     __shared__ T s_ab[2];   // (one conversion: a warp's takes the FP64 pipe 64 cycles)
@@ -814,7 +814,7 @@ __host__ __device__ inline ClLayout cl_layout(int m, int n, int R) {
 }
 
 __global__ void __launch_bounds__(kClT, 1) pcg_cluster_kernel(PcgArgs<float> A, int g, int smem_bytes) {
-    extern __shared__ __align__(16) unsigned char dsm[];
+    extern __shared__ __align__(32) unsigned char dsm[];
     __shared__ float sh[kClT / 32];
     __shared__ int shi[kClT / 32];
     __shared__ float s_part[6];  // 0: p.q  1: r.z  2: r.r  3, 4: b.b, b.z at the start
