@@ -359,7 +359,7 @@ int ot_price_topk_ex(int32_t m, int32_t n, const int32_t *sx, const int32_t *sy,
  * on the device holds those 24 MiB until the process exits.  Every call looks up the array's
  * device address (with the calling thread's current device); make the first call on a device
  * before any stream capture.  Limits: m, n <= 16384, and the candidate set the selection has to
- * recheck must fit the array (about 400k pairs); beyond either limit the call returns OT_ERR_ARG
+ * recheck must fit the array (about 570k pairs); beyond either limit the call returns OT_ERR_ARG
  * or OT_ERR_BUF_TOO_SMALL with a message (ot_last_error) and changes no output.  Every call on a
  * device uses the same array and leaves its contents behind (each call clears what it needs), so
  * calls that overlap on the GPU -- on two streams, or from two threads -- race and must be

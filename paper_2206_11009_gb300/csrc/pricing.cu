@@ -996,14 +996,14 @@ __global__ void recheck_kernel(int m, int n, int kind, unsigned long long count,
                                const int32_t *__restrict__ row_ptr,
                                const int32_t *__restrict__ sup_j, Geo *geo,
                                uint64_t *__restrict__ key, uint32_t *__restrict__ val,
-                               uint64_t *__restrict__ dkey, double *__restrict__ dval) {
+                               uint64_t *__restrict__ dkey) {
     const unsigned ncand = geo->ncand;
     for (unsigned long long g = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; g < count;
          g += (unsigned long long)gridDim.x * blockDim.x) {
         uint64_t kj = ~0ull, kd = ~0ull;
-        double d = 0.0;
         if (g < ncand) {
             const int i = ci[g], j = cj[g];
+            double d;
             kj = (uint64_t)i + (uint64_t)j * (uint64_t)m;
             if (recheck_pair(i, j, n, kind, sx, sy, tx, ty, u, v, C, row_ptr, sup_j, d)) {
                 kd = f64_key(d);
@@ -1013,7 +1013,6 @@ __global__ void recheck_kernel(int m, int n, int kind, unsigned long long count,
         key[g] = kj;
         val[g] = (uint32_t)g;
         dkey[g] = kd;
-        dval[g] = d;
     }
 }
 
@@ -1024,8 +1023,9 @@ __global__ void rekey_kernel(unsigned long long count, const uint32_t *__restric
         key[g] = dkey[val[g]];
 }
 
+// (key: the reduced costs' keys, sorted)
 __global__ void finalize_kernel(int kmax, const uint32_t *__restrict__ val, const int32_t *__restrict__ ci,
-                                const int32_t *__restrict__ cj, const double *__restrict__ dval,
+                                const int32_t *__restrict__ cj, const uint64_t *__restrict__ key,
                                 const Geo *__restrict__ geo, int32_t *__restrict__ out_i,
                                 int32_t *__restrict__ out_j, double *__restrict__ out_d,
                                 int32_t *__restrict__ out_count) {
@@ -1034,7 +1034,7 @@ __global__ void finalize_kernel(int kmax, const uint32_t *__restrict__ val, cons
         const uint32_t g = val[k];
         out_i[k] = ci[g];
         out_j[k] = cj[g];
-        if (out_d) out_d[k] = dval[g];
+        if (out_d) out_d[k] = f64_from_key(key[k]);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) *out_count = cnt;
 }
@@ -1446,15 +1446,13 @@ Error price_topk(const PriceInput &in, int32_t *out_i, int32_t *out_j, double *o
     OT_TRY(pass(true, ci.p, cj.p, cap));
     DevTemp<uint64_t> key, dkey;
     DevTemp<uint32_t> val;
-    DevTemp<double> dval;
     OT_TRY(key.alloc(cnt, st));
     OT_TRY(dkey.alloc(cnt, st));
     OT_TRY(val.alloc(cnt, st));
-    OT_TRY(dval.alloc(cnt, st));
     const int rb = (int)std::min<int64_t>(8 * sms, ceil_div(cnt, 256));
     ktimer_begin(KT_RECHECK, st);
     recheck_kernel<<<rb, 256, 0, st>>>(m, n, kind, cap, ci.p, cj.p, in.sx, in.sy, in.tx, in.ty, in.u, in.v, in.C, rp,
-                                       in.sup_j, geo, key.p, val.p, dkey.p, dval.p);
+                                       in.sup_j, geo, key.p, val.p, dkey.p);
     OT_LAUNCHED();
     ktimer_end(KT_RECHECK, st);
     int jbits = 1;
@@ -1464,7 +1462,7 @@ Error price_topk(const PriceInput &in, int32_t *out_i, int32_t *out_j, double *o
     OT_LAUNCHED();
     OT_TRY(radix_sort_pairs(key.p, val.p, cnt, 64, st));
     finalize_kernel<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(in.kmax, 256), 4 * sms)), 256, 0, st>>>(
-        in.kmax, val.p, ci.p, cj.p, dval.p, geo, out_i, out_j, out_d, out_count);
+        in.kmax, val.p, ci.p, cj.p, key.p, geo, out_i, out_j, out_d, out_count);
     OT_LAUNCHED();
     OT_CUDA(cudaMemcpyAsync(&hg, geo, sizeof(Geo), cudaMemcpyDeviceToHost, st));
     OT_CUDA(cudaStreamSynchronize(st));

@@ -13,7 +13,7 @@ namespace {
 
 // 24 MiB of scratch on every device where the library's module is loaded (held until the process
 // exits).  With lazy module loading that happens at the first call on the device.  Enough for
-// m, n <= 16384 and a pricing candidate set of about 400k pairs.
+// m, n <= 16384 and a pricing candidate set of about 570k pairs (40 bytes each, beside the points and tiles).
 constexpr size_t kScratchBytes = (size_t)24 << 20;
 constexpr int32_t kMaxSide = 16384;
 
