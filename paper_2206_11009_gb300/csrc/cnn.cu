@@ -520,7 +520,7 @@ __global__ void __launch_bounds__(kThr, 2)
 conv_tc_kernel(int B, int H, int Wd, int dil, const __nv_bfloat16 *__restrict__ in,
                const __nv_bfloat16 *__restrict__ wop, ConvIo io, int *__restrict__ err) {
     constexpr int N = 32, Bbytes = N * kCvK * 2;
-    constexpr uint32_t idesc = tc_idesc(1u, kCvM, N);
+    constexpr uint32_t idesc = tc_idesc(kCvM, N);
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ float sh[16][16], sdot[4][kPix], sg[32], sbias[32];
     unsigned char *sB = smem + kCvAbytes;
@@ -561,7 +561,7 @@ conv_tc_kernel(int B, int H, int Wd, int dil, const __nv_bfloat16 *__restrict__ 
             const uint32_t lboA = (kCvM / 8) * 128, lboB = (N / 8) * 128;
 #pragma unroll
             for (int ks = 0; ks < kCvK / 16; ++ks)
-                tc_mma<true>(tmem, tc_desc(a0 + ks * 2 * lboA, lboA), tc_desc(b0 + ks * 2 * lboB, lboB), idesc, ks > 0);
+                tc_mma(tmem, tc_desc(a0 + ks * 2 * lboA, lboA), tc_desc(b0 + ks * 2 * lboB, lboB), idesc, ks > 0);
             tc_commit(mbar);
         }
         const bool done = tc_wait(mbar, (uint32_t)(it & 1));
@@ -625,7 +625,7 @@ conv_wgrad_tc_kernel(int B, int H, int Wd, int dil, const __nv_bfloat16 *__restr
                      int *__restrict__ err) {
     constexpr int N = HEAD ? 16 : 32, Bbytes = kCvM * N * 2;
     // both operands MN-major (bits 15 and 16)
-    constexpr uint32_t idesc = tc_idesc(1u, kCvM, N) | (1u << 15) | (1u << 16);
+    constexpr uint32_t idesc = tc_idesc(kCvM, N) | (1u << 15) | (1u << 16);
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char *sB = smem + kCvAbytes;
     uint64_t *mb = (uint64_t *)(sB + Bbytes);
@@ -683,7 +683,7 @@ conv_wgrad_tc_kernel(int B, int H, int Wd, int dil, const __nv_bfloat16 *__restr
                 const uint32_t am = a0 + (mt == 0 ? 0 : mt == 1 ? 16 : 20) * sbo;
 #pragma unroll
                 for (int ks = 0; ks < kCvM / 16; ++ks)
-                    tc_mma<true>(tmem + (uint32_t)(mt * 32), tc_desc2(am + ks * 256, 128, sbo),
+                    tc_mma(tmem + (uint32_t)(mt * 32), tc_desc2(am + ks * 256, 128, sbo),
                                  tc_desc2(b0 + ks * 256, 128, sbo), idesc, ks > 0);
             }
             tc_commit(mbar);

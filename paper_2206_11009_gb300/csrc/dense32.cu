@@ -956,7 +956,7 @@ constexpr int kTcSmem = 116 * 1024;   // 96 KB used; more than half an SM's, so 
 static_assert(kTcSmem >= kTcStages * kTcStage + 128 && 2 * kTcSmem > 228 * 1024, "stages and barriers");
 static_assert(kTcPer == 2 * kTcStages, "the ring holds a panel");
 constexpr int kTcAutoN = 8192;    // tc_mode 0: the tensor-core update from this n on
-constexpr uint32_t kTcIdesc = tc_idesc(1u, kTcM, kTcM);   // BF16, both K-major
+constexpr uint32_t kTcIdesc = tc_idesc(kTcM, kTcM);   // BF16, both K-major
 
 // Split operands of one panel in blocks of 128 rows: LD rows (A of the trailing tiles), panel rows (their
 // B, and A of the inverse's tiles), rows of L^-1 by column (B of the inverse's)
@@ -1117,14 +1117,14 @@ d32_tc_update_kernel(int n, int ld, int base, int base2, int T, unsigned char *_
                     if (q < kTcPer) {
                         if (!tc_wait(mload + 8 * slot, (uint32_t)((2 * i + q / kTcStages) & 1))) { ok = false; break; }
                         tc_fence_after();
-                        tc_mma<true>(second, a0, b2, kTcIdesc, q > 0);
-                        tc_mma<true>(second, a2, b0, kTcIdesc, true);
-                        tc_mma<true>(second, a1, b1, kTcIdesc, true);
-                        tc_mma<true>(second, a0, b1, kTcIdesc, true);
-                        tc_mma<true>(second, a1, b0, kTcIdesc, true);
+                        tc_mma(second, a0, b2, kTcIdesc, q > 0);
+                        tc_mma(second, a2, b0, kTcIdesc, true);
+                        tc_mma(second, a1, b1, kTcIdesc, true);
+                        tc_mma(second, a0, b1, kTcIdesc, true);
+                        tc_mma(second, a1, b0, kTcIdesc, true);
                     }
-                    if (q < kTcStages) tc_mma<true>(first, a0, b0, kTcIdesc, q > 0);
-                    if (q >= kTcPer) tc_mma<true>(second, a0, b0, kTcIdesc, true);
+                    if (q < kTcStages) tc_mma(first, a0, b0, kTcIdesc, q > 0);
+                    if (q >= kTcPer) tc_mma(second, a0, b0, kTcIdesc, true);
                     if (q < kTcStages || q >= kTcPer) {
                         tc_commit(mfree + 8 * slot);
                         ++g;

@@ -54,8 +54,8 @@ struct PriceStats {
     float err_bound = 0.f;   // proven |d_fp32 - d_fp64| bound used for the window
 };
 
-// Selection written to out_i/out_j/out_d (capacity kmax, device) and *out_count (device).
-// Synchronises the stream once, at the end.  Stats filled when non-null.
+// Selection written to out_i/out_j/out_d (capacity kmax, device) and *out_count (device or pinned host
+// memory).  Synchronises the stream once, at the end.  Stats filled when non-null.
 Error price_topk(const PriceInput &in, int32_t *out_i, int32_t *out_j, double *out_d,
                  int32_t *out_count, PriceStats *stats, cudaStream_t st);
 

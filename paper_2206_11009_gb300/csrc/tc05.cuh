@@ -2,7 +2,7 @@
 // memory, accumulators in tensor memory, completion on mbarriers).
 //
 // Operand layout used by every caller: no swizzle, K-major unless said, core matrices of 8 rows x
-// 16 bytes (4 TF32 or 8 BF16 values along K).  The shared-memory matrix descriptor carries the
+// 16 bytes (8 BF16 values along K).  The shared-memory matrix descriptor carries the
 // start address, the leading byte offset (between core matrices adjacent along K) and the stride
 // byte offset (between core matrices adjacent along M or N, here always 128: the 8-row groups are
 // packed), each shifted right by 4, and the descriptor version 1 at bit 46.
@@ -36,11 +36,10 @@ __device__ __forceinline__ uint64_t tc_desc2(uint32_t addr, uint32_t lbo, uint32
     return d;
 }
 
-// Instruction descriptor of kind::f16 / kind::tf32 MMAs with an FP32 accumulator and K-major A and
-// B: ab = 1 for BF16 operands (kind::f16), 2 for TF32 (kind::tf32); N at bits 17-22 (N / 8), M at
-// bits 24-28 (M / 16).
-__host__ __device__ constexpr uint32_t tc_idesc(uint32_t ab, int M, int N) {
-    return (1u << 4) | (ab << 7) | (ab << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+// Instruction descriptor of kind::f16 MMAs with an FP32 accumulator and K-major BF16 A and B: N at bits
+// 17-22 (N / 8), M at bits 24-28 (M / 16).
+__host__ __device__ constexpr uint32_t tc_idesc(int M, int N) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 // bounded wait for phase `parity` of an mbarrier; false when it gave up
@@ -78,17 +77,11 @@ __device__ __forceinline__ void tc_mbar_init(uint32_t mbar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(mbar), "r"(count) : "memory");
 }
 
-// D (tensor memory) = A B^T (+ D when accumulate), one MMA of the kind named by the template
-template <bool BF16>
+// D (tensor memory) = A B^T (+ D when accumulate), one BF16 MMA
 __device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, bool accumulate) {
-    if constexpr (BF16)
-        asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                     " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-                     :: "r"(d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate ? 1u : 0u) : "memory");
-    else
-        asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                     " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n"
-                     :: "r"(d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate ? 1u : 0u) : "memory");
+    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                 " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
+                 :: "r"(d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate ? 1u : 0u) : "memory");
 }
 
 // the MMAs issued so far by this thread arrive on `mbar` when complete
